@@ -88,6 +88,7 @@ struct EsLayout {
         fix_count, sk, total;
     int n_tiles;
     int64_t Tc;
+    int64_t ldv;  // row stride of E and z: V, for fp32 rounded up to 8 (16-byte rows)
     int algo;  // the algorithm that runs: FPO_ES_RECOMPUTE, _STORED_LOGITS or _DIRECT
 };
 
@@ -126,6 +127,8 @@ EsLayout es_layout(const fpo_error_signal_desc* d) {
     // power-capped clock settles higher), and the chunk buffers shrink accordingly.
     const int64_t chunk = d->t_chunk > 0 ? d->t_chunk : FPO_AUTO_T_CHUNK;
     L.Tc = d->T == 0 ? 0 : (chunk < d->T ? chunk : d->T);
+    L.ldv = d->dtype == FPO_BF16 ? d->V : (d->V + 7) / 8 * 8;
+    const size_t ldv = static_cast<size_t>(L.ldv);
     size_t off = kStatusBytes;
     L.yhat = off; off = align_up(off + T * D * esz);
     L.rho = off;  off = align_up(off + T * 4);
@@ -137,8 +140,8 @@ EsLayout es_layout(const fpo_error_signal_desc* d) {
     const bool stored = L.algo == FPO_ES_STORED_LOGITS, direct = L.algo == FPO_ES_DIRECT;
     // g in fp32 for the separate VJP (the direct algorithm writes g~ from the projection)
     L.g = off;    off = align_up(off + (direct ? 0 : T * D * 4));
-    L.E = off;    off = align_up(off + static_cast<size_t>(L.Tc) * V * esz);
-    L.z = off;    off = align_up(off + (stored ? static_cast<size_t>(L.Tc) * V * 4 : 0));
+    L.E = off;    off = align_up(off + static_cast<size_t>(L.Tc) * ldv * esz);
+    L.z = off;    off = align_up(off + (stored ? static_cast<size_t>(L.Tc) * ldv * 4 : 0));
     const size_t Tdir = direct ? T : 0, Tcdir = direct ? static_cast<size_t>(L.Tc) : 0;
     L.anchor = off;    off = align_up(off + Tdir * 4);
     L.su = off;        off = align_up(off + Tdir * static_cast<size_t>(L.n_tiles) * 4);
@@ -314,8 +317,8 @@ int32_t fpo_error_signal(const fpo_error_signal_desc* desc, const void* h, const
                                             nullptr, status, st));
         else
             FPO_TRY(launch_lse_partial_f32(static_cast<const float*>(yhat),
-                                           static_cast<const float*>(W_U), targets, T, d, V, part,
-                                           L.n_tiles, zy, nullptr, st));
+                                           static_cast<const float*>(W_U), targets, T, T, d, V,
+                                           part, L.n_tiles, zy, nullptr, L.ldv, st));
         FPO_TRY(per_chunk ? ev(2) : mark(2));
         FPO_TRY(launch_lse_combine(part, L.n_tiles, T, zy, lse, ce, st));
         if (loss_out) FPO_TRY(launch_mean(ce, T, loss_out, st));
@@ -336,10 +339,12 @@ int32_t fpo_error_signal(const fpo_error_signal_desc* desc, const void* h, const
             } else {
                 FPO_TRY(launch_error_f32(static_cast<const float*>(yh),
                                          static_cast<const float*>(W_U), targets + c0, lse + c0,
-                                         tc, d, V, desc->loss_scale, static_cast<float*>(E), st));
+                                         tc, T, d, V, desc->loss_scale, static_cast<float*>(E),
+                                         L.ldv, st));
                 FPO_TRY(cmark(ci, 4));
-                FPO_TRY(launch_proj_f32(static_cast<const float*>(E), static_cast<const float*>(W_U),
-                                        tc, d, V, g + c0 * d, st));
+                FPO_TRY(launch_proj_f32(static_cast<const float*>(E), L.ldv,
+                                        static_cast<const float*>(W_U), tc, T, d, V, g + c0 * d,
+                                        st));
             }
             FPO_TRY(cmark(ci, 5));
         }
@@ -358,20 +363,21 @@ int32_t fpo_error_signal(const fpo_error_signal_desc* desc, const void* h, const
                                                 z, status, st));
             else
                 FPO_TRY(launch_lse_partial_f32(static_cast<const float*>(yh),
-                                               static_cast<const float*>(W_U), targets + c0, tc, d,
-                                               V, pc, L.n_tiles, zyc, z, st));
+                                               static_cast<const float*>(W_U), targets + c0, tc, T,
+                                               d, V, pc, L.n_tiles, zyc, z, L.ldv, st));
             FPO_TRY(cmark(ci, 2));
             FPO_TRY(launch_lse_combine(pc, L.n_tiles, tc, zyc, lse + c0, cec, st));
             if (last && loss_out) FPO_TRY(launch_mean(ce, T, loss_out, st));
             FPO_TRY(cmark(ci, 3));
             FPO_TRY(launch_error_from_logits(desc->dtype, z, lse + c0, targets + c0, tc, V,
-                                             desc->loss_scale, E, st));
+                                             L.ldv, desc->loss_scale, E, st));
             FPO_TRY(cmark(ci, 4));
             if (bf16)
                 FPO_TRY(launch_proj_bf16(E, W_U, tc, d, V, g + c0 * d, sk, status, st));
             else
-                FPO_TRY(launch_proj_f32(static_cast<const float*>(E), static_cast<const float*>(W_U),
-                                        tc, d, V, g + c0 * d, st));
+                FPO_TRY(launch_proj_f32(static_cast<const float*>(E), L.ldv,
+                                        static_cast<const float*>(W_U), tc, T, d, V, g + c0 * d,
+                                        st));
             FPO_TRY(cmark(ci, 5));
         }
     }

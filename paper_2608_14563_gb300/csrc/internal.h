@@ -194,10 +194,12 @@ cudaError_t launch_direct_fixup_factors(const float* sx, const float* qz, const 
 cudaError_t launch_lse_combine(const float2* part, int n_tiles, int T, const float* zy,
                                float* lse, float* ce, cudaStream_t st);
 cudaError_t launch_mean(const float* x, int n, float* out, cudaStream_t st);
-// Stored-logits algorithm: E[M, V] = s (exp(z - lse) - onehot(y)) from z[M, V] fp32, in
-// dtype (bf16 through the same formula as the recompute epilogue, or fp32).
+// Stored-logits algorithm: E[M, ld] = s (exp(z - lse) - onehot(y)) from z[M, ld] fp32, in
+// dtype (bf16 through the same formula as the recompute epilogue, or fp32); ld, a multiple
+// of 8, is the row stride of both, and columns V and above are left unspecified.
 cudaError_t launch_error_from_logits(int dtype, const float* z, const float* lse, const int32_t* y,
-                                     int M, int V, float s, void* E, cudaStream_t st);
+                                     int M, int V, long long ld, float s, void* E,
+                                     cudaStream_t st);
 // dst[n] = src[n] rounded to dtype (a plain copy for fp32).
 cudaError_t launch_cast_f32(int dtype, const float* src, size_t n, void* dst, cudaStream_t st);
 cudaError_t launch_rmsnorm_vjp(int dtype, const float* g, const void* h, const void* w,
@@ -233,15 +235,18 @@ cudaError_t launch_cosine(int dtype, int64_t n, const void* X, const void* Y, do
                           int blocks, double* out, cudaStream_t st);
 
 // ------------------------------------------------------------ fp32 SIMT path
-constexpr int kSimtTile = 64;
+constexpr int kSimtTile = 64;  // columns of one (max, sum exp) partial
+// T: the rows of this call (a token chunk), T_all: the rows of the whole batch, from which
+// the split of the k range is chosen (so that it does not depend on the chunking).
+// ldz, ldE: row strides of the logits and the error matrix, multiples of 4.
 cudaError_t launch_lse_partial_f32(const float* yhat, const float* W_U, const int32_t* y, int T,
-                                   int d, int V, float2* part, int part_ld, float* zy, float* z,
-                                   cudaStream_t st);
+                                   int T_all, int d, int V, float2* part, int part_ld, float* zy,
+                                   float* z, long long ldz, cudaStream_t st);
 cudaError_t launch_error_f32(const float* yhat, const float* W_U, const int32_t* y,
-                             const float* lse, int Tc, int d, int V, float s, float* E,
-                             cudaStream_t st);
-cudaError_t launch_proj_f32(const float* E, const float* W_U, int Tc, int d, int V, float* g,
-                            cudaStream_t st);
+                             const float* lse, int Tc, int T_all, int d, int V, float s, float* E,
+                             long long ldE, cudaStream_t st);
+cudaError_t launch_proj_f32(const float* E, long long ldE, const float* W_U, int Tc, int T_all,
+                            int d, int V, float* g, cudaStream_t st);
 cudaError_t launch_update_f32(int n, int T, int d, int d_ff, const float* const* g,
                               const float* const* A, float lr, float* const* W_master,
                               float* const* W_out, float* const* G_out, cudaStream_t st);

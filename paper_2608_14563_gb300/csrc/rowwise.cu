@@ -560,13 +560,13 @@ constexpr int kErrThreads = 256;
 template <bool kBf16>
 __global__ void __launch_bounds__(kErrThreads)
     error_from_logits_kernel(const float* __restrict__ z, const float* __restrict__ lse,
-                             const int32_t* __restrict__ y, int M, int V, float s,
+                             const int32_t* __restrict__ y, int M, int V, long long ld, float s,
                              void* __restrict__ E) {
     for (int row = blockIdx.x; row < M; row += gridDim.x) {
         const float l = lse[row];
         const float l2 = l * kLog2e;
         const int yt = y[row];
-        const float* zr = z + static_cast<size_t>(row) * V;
+        const float* zr = z + row * ld;  // V <= ld, a multiple of 8
         for (int c = threadIdx.x * 8; c < V; c += kErrThreads * 8) {
             const float4 a = __ldcs(reinterpret_cast<const float4*>(zr + c));
             const float4 b = __ldcs(reinterpret_cast<const float4*>(zr + c + 4));
@@ -577,32 +577,17 @@ __global__ void __launch_bounds__(kErrThreads)
                 for (int k = 0; k < 8; k += 2)
                     w[k / 2] = pack_bf16x2(error_value(v[k], l2, c + k == yt, s),
                                            error_value(v[k + 1], l2, c + k + 1 == yt, s));
-                *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(E) +
-                                          static_cast<size_t>(row) * V + c) =
+                *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(E) + row * ld + c) =
                     make_uint4(w[0], w[1], w[2], w[3]);
             } else {
                 float o[8];
 #pragma unroll
                 for (int k = 0; k < 8; ++k) o[k] = error_value_f32(v[k], l, c + k == yt, s);
-                float* dst = static_cast<float*>(E) + static_cast<size_t>(row) * V + c;
+                float* dst = static_cast<float*>(E) + row * ld + c;
                 *reinterpret_cast<float4*>(dst) = make_float4(o[0], o[1], o[2], o[3]);
                 *reinterpret_cast<float4*>(dst + 4) = make_float4(o[4], o[5], o[6], o[7]);
             }
         }
-    }
-}
-
-// Scalar variant for fp32 rows whose length is not a multiple of 8.
-__global__ void __launch_bounds__(kErrThreads)
-    error_from_logits_scalar_kernel(const float* __restrict__ z, const float* __restrict__ lse,
-                                    const int32_t* __restrict__ y, int M, int V, float s,
-                                    float* __restrict__ E) {
-    for (int row = blockIdx.x; row < M; row += gridDim.x) {
-        const float l = lse[row];
-        const int yt = y[row];
-        for (int c = threadIdx.x; c < V; c += kErrThreads)
-            E[static_cast<size_t>(row) * V + c] =
-                error_value_f32(z[static_cast<size_t>(row) * V + c], l, c == yt, s);
     }
 }
 
@@ -1106,20 +1091,17 @@ cudaError_t launch_cast_f32(int dtype, const float* src, size_t n, void* dst, cu
 }
 
 cudaError_t launch_error_from_logits(int dtype, const float* z, const float* lse, const int32_t* y,
-                                     int M, int V, float s, void* E, cudaStream_t st) {
+                                     int M, int V, long long ld, float s, void* E,
+                                     cudaStream_t st) {
     if (M <= 0) return cudaSuccess;
     DevInfo di;
     const int sms = current_device_info(&di) ? di.sm_count : 148;
     const int grid = M < sms * 8 ? M : sms * 8;
     if (dtype == 1)
-        error_from_logits_kernel<true><<<grid, kErrThreads, 0, st>>>(z, lse, y, M, V, s, E),
-            ::fpo::note_launch();
-    else if (V % 8 == 0)
-        error_from_logits_kernel<false><<<grid, kErrThreads, 0, st>>>(z, lse, y, M, V, s, E),
+        error_from_logits_kernel<true><<<grid, kErrThreads, 0, st>>>(z, lse, y, M, V, ld, s, E),
             ::fpo::note_launch();
     else
-        error_from_logits_scalar_kernel<<<grid, kErrThreads, 0, st>>>(z, lse, y, M, V, s,
-                                                                      static_cast<float*>(E)),
+        error_from_logits_kernel<false><<<grid, kErrThreads, 0, st>>>(z, lse, y, M, V, ld, s, E),
             ::fpo::note_launch();
     return cudaGetLastError();
 }
