@@ -306,7 +306,7 @@ int32_t fpo_error_signal(const fpo_error_signal_desc* desc, const void* h, const
             FPO_TRY(launch_proj_vjp_bf16(
                 E, W_U, targets + c0, alpha + c0, beta + c0, cv + c0, rho + c0,
                 static_cast<const uint8_t*>(h) + static_cast<size_t>(c0) * d * esz, norm_w,
-                desc->min_rms, tc, d, V,
+                desc->min_rms, tc, T, d, V,
                 static_cast<uint8_t*>(g_out) + static_cast<size_t>(c0) * d * esz, sk, status, st));
             FPO_TRY(cmark(ci, 5));
         }
@@ -335,7 +335,7 @@ int32_t fpo_error_signal(const fpo_error_signal_desc* desc, const void* h, const
                 FPO_TRY(launch_error_bf16(yh, W_U, targets + c0, lse + c0, tc, d, V,
                                           desc->loss_scale, E, status, st));
                 FPO_TRY(cmark(ci, 4));
-                FPO_TRY(launch_proj_bf16(E, W_U, tc, d, V, g + c0 * d, sk, status, st));
+                FPO_TRY(launch_proj_bf16(E, W_U, tc, T, d, V, g + c0 * d, sk, status, st));
             } else {
                 FPO_TRY(launch_error_f32(static_cast<const float*>(yh),
                                          static_cast<const float*>(W_U), targets + c0, lse + c0,
@@ -373,7 +373,7 @@ int32_t fpo_error_signal(const fpo_error_signal_desc* desc, const void* h, const
                                              L.ldv, desc->loss_scale, E, st));
             FPO_TRY(cmark(ci, 4));
             if (bf16)
-                FPO_TRY(launch_proj_bf16(E, W_U, tc, d, V, g + c0 * d, sk, status, st));
+                FPO_TRY(launch_proj_bf16(E, W_U, tc, T, d, V, g + c0 * d, sk, status, st));
             else
                 FPO_TRY(launch_proj_f32(static_cast<const float*>(E), L.ldv,
                                         static_cast<const float*>(W_U), tc, T, d, V, g + c0 * d,

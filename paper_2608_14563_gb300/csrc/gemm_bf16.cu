@@ -179,13 +179,13 @@ SkPlan tail_plan(long long tiles, long long clusters, int k_blocks) {
     return p;
 }
 
-// With sk_scratch non-null, the tiles of the last partial wave are split by tail_plan
-// (SegCursor); the caller then runs sk_fixup over them (plan->tail_tiles > 0).
-// sk_scratch holds kTailWaves x clusters x 256 x BN fp32.
+// With sk_scratch non-null, the tiles are split by `split` k ranges each when that is above
+// 1, else those of the last partial wave by tail_plan (SegCursor); the caller then runs
+// sk_fixup over them (plan->tail_tiles > 0).  sk_scratch holds 256 x BN fp32 per unit.
 template <int BN, bool A_MN, bool B_MN, int STAGES, int MAXG, class Epi>
 cudaError_t run_gemm_pair(const GemmMaps<MAXG>& maps, const typename Epi::Params& ep,
                           const GemmShape& sh_in, unsigned* status, cudaStream_t st,
-                          float* sk_scratch = nullptr, SkPlan* plan = nullptr) {
+                          float* sk_scratch = nullptr, SkPlan* plan = nullptr, int split = 0) {
     if (plan) *plan = SkPlan{};
     if (sh_in.tiles <= 0 || sh_in.k_blocks <= 0) return cudaSuccess;
     using L = GemmPairSmem<BN, STAGES, pair_ksub<BN, A_MN, B_MN>()>;
@@ -196,10 +196,17 @@ cudaError_t run_gemm_pair(const GemmMaps<MAXG>& maps, const typename Epi::Params
     DevInfo di;
     if (!current_device_info(&di)) return cudaErrorUnknown;
     const int max_clusters = resident_clusters<kern>(L::kBytes, di.sm_count, 2);
-    const long long clusters = sh_in.tiles < max_clusters ? sh_in.tiles : max_clusters;
+    const long long units = split > 1 ? sh_in.tiles * split : sh_in.tiles;
+    const long long clusters = units < max_clusters ? units : max_clusters;
     GemmShape sh = sh_in;
     if (sk_scratch) {
-        const SkPlan p = tail_plan(sh.tiles, clusters, sh.k_blocks);
+        SkPlan p;
+        if (split > 1) {
+            p.tail_tiles = sh.tiles;
+            p.tail_split = split;
+        } else {
+            p = tail_plan(sh.tiles, clusters, sh.k_blocks);
+        }
         if (p.tail_tiles > 0) {
             sh.tail_tiles = p.tail_tiles;
             sh.tail_split = p.tail_split;
@@ -234,9 +241,11 @@ __device__ __forceinline__ bool sk_tail_sum(const GemmShape& sh, const float* __
     n = nb * BN + col;
     if (row >= sh.M || n >= sh.N) return false;  // N % 8 == 0: whole groups of 4
     s4[0] = s4[1] = s4[2] = s4[3] = 0.f;
+    const float* p = scratch + (static_cast<size_t>(r_tile) * kPairBM + r) * BN + col;
+    const size_t step = static_cast<size_t>(R) * kPairBM * BN;  // one range to the next
+#pragma unroll 4
     for (int q = 0; q < sh.tail_split; ++q) {
-        const float4 u = *reinterpret_cast<const float4*>(
-            scratch + ((static_cast<size_t>(q) * R + r_tile) * kPairBM + r) * BN + col);
+        const float4 u = *reinterpret_cast<const float4*>(p + q * step);
         s4[0] += u.x;
         s4[1] += u.y;
         s4[2] += u.z;
@@ -332,6 +341,8 @@ cudaError_t launch_sk_fixup_vjp(const SkPlan& plan, const GemmShape& sh, const f
     return cudaGetLastError();
 }
 
+constexpr int kProjBN = 256;     // projection tiles where 512 columns are too wide
+constexpr int kProjStages = 4;   // (single-CTA kernel)
 constexpr int kPairStages = 3;   // 256 x 256 pair tiles: 64 KB stages of two k-blocks
 constexpr int kWideBN = 512;     // pair tiles 256 x 512: 48 KB stages
 constexpr int kWideStages = 4;
@@ -365,17 +376,58 @@ void set_gemm_variant(int v) {
 }
 int gemm_variant() { return g_gemm_variant.load(std::memory_order_relaxed); }
 
-size_t proj_sk_scratch_bytes() {
-    // kTailWaves x clusters units of 256 x 512 fp32; clusters of the 256 x 512 pair kernel
-    // on the current device, or an upper bound of 128 without one
+namespace {
+
+// Pair clusters of the 256 x 512 projection kernel resident at once on the current device
+// (an upper bound of 128 without one).
+int proj_clusters() {
     using L = GemmPairSmem<kWideBN, kWideStages, pair_ksub<kWideBN, false, true>()>;
     constexpr auto kern = tc_gemm_pair_kernel<kWideBN, false, true, kWideStages, 1, EpiProjVjp>;
     DevInfo di;
-    long long c = 128;
+    int c = 128;
     if (current_device_info(&di) && set_smem_limit<kern>(L::kBytes) == cudaSuccess)
         c = resident_clusters<kern>(L::kBytes, di.sm_count, 2);
     cudaGetLastError();
-    return static_cast<size_t>(kTailWaves) * c * kPairBM * kWideBN * sizeof(float);
+    return c;
+}
+
+// K ranges per tile of the projection of a batch of T tokens, or 0: batches with at least
+// one 256 x 512 tile per pair cluster take those tiles whole, with the split tail of the
+// last wave.  Below that the clusters without a tile would idle through a K loop over the
+// whole vocabulary, so such a batch runs on 256 x 256 tiles, each in the number of ranges
+// that costs least.  Measured, in ns: a 64-deep k-block 344 (at the clock the tensor cores
+// hold under load), with a split the fixup's launch 4000 and its read of the fp32 parts
+// 4.3 bytes a ns.  Ranges have at least 32 k-blocks, and the units fit the scratch.  T is
+// the whole batch, not a token chunk, so that the sums do not depend on the chunking.
+// Projection with its fixup, T x d x V: 333 x 4096 x 100352 (16 tiles of 512 columns on 76
+// clusters) 887 us whole, 246 us in 7 ranges; 2048 x 2048 x 50304 (32 tiles) 434 and 276.
+int proj_split(int T, int d, int V) {
+    const long long clusters = proj_clusters();
+    const long long m_blocks = (T + kPairBM - 1) / kPairBM;
+    if (m_blocks * ((d + kWideBN - 1) / kWideBN) >= clusters) return 0;
+    const int kb = (V + kBK - 1) / kBK;
+    const long long tiles = m_blocks * ((d + kProjBN - 1) / kProjBN);
+    const long long cap = kTailWaves * clusters * (kWideBN / kProjBN);  // units of scratch
+    double best_cost = 0.0;
+    int best = 1;
+    for (int S = 1; S <= 64; ++S) {
+        if (S > 1 && (kb / S < 32 || tiles * S > cap)) break;
+        double cost = static_cast<double>((tiles * S + clusters - 1) / clusters) *
+                          ((kb + S - 1) / S) * 344.0;
+        if (S > 1) cost += 4000.0 + tiles * S * (kProjBN * 1024.0) / 4300.0;
+        if (S == 1 || cost < best_cost) {
+            best_cost = cost;
+            best = S;
+        }
+    }
+    return best;
+}
+
+}  // namespace
+
+size_t proj_sk_scratch_bytes() {
+    // kTailWaves x clusters units of 256 x 512 fp32 (twice as many of 256 x 256)
+    return static_cast<size_t>(kTailWaves) * proj_clusters() * kPairBM * kWideBN * sizeof(float);
 }
 
 constexpr int kLseBN = 256;
@@ -509,14 +561,11 @@ cudaError_t launch_fixup_logits_bf16(const void* yfix, const void* W_U, const in
     return run_gemm_pair<kLseBN, false, false, kPairStages, 1, EpiFixProb>(maps, ep, sh, status, st);
 }
 
-constexpr int kProjBN = 256;
-constexpr int kProjStages = 4;
-
 cudaError_t launch_proj_vjp_bf16(const void* P, const void* W_U, const int32_t* y,
                                  const float* alpha, const float* beta, const float* cv,
                                  const float* rho, const void* h, const void* w, float min_rms,
-                                 int Tc, int d, int V, void* g_tilde, float* sk_scratch,
-                                 unsigned* status, cudaStream_t st) {
+                                 int Tc, int T_all, int d, int V, void* g_tilde,
+                                 float* sk_scratch, unsigned* status, cudaStream_t st) {
     GemmMaps<1> maps;
     if (!map_kmajor(&maps.a[0], P, Tc, V, kBM) || !map_mnmajor(&maps.b[0], W_U, V, d))
         return cudaErrorInvalidValue;
@@ -536,13 +585,22 @@ cudaError_t launch_proj_vjp_bf16(const void* P, const void* W_U, const int32_t* 
     ep.M = Tc;
     ep.N = d;
     if (wide_proj()) {
-        ep.tile_n = kWideBN;
-        const GemmShape sh = make_shape(Tc, d, V, kWideBN, 1, band_for(true), kPairBM);
         SkPlan plan;
-        cudaError_t e = run_gemm_pair<kWideBN, false, true, kWideStages, 1, EpiProjVjp>(
-            maps, ep, sh, status, st, sk_scratch, &plan);
+        const int split = proj_split(T_all, d, V);
+        if (split == 0) {
+            ep.tile_n = kWideBN;
+            const GemmShape sh = make_shape(Tc, d, V, kWideBN, 1, band_for(true), kPairBM);
+            const cudaError_t e = run_gemm_pair<kWideBN, false, true, kWideStages, 1, EpiProjVjp>(
+                maps, ep, sh, status, st, sk_scratch, &plan);
+            if (e != cudaSuccess) return e;
+            return launch_sk_fixup_vjp<kWideBN>(plan, sh, sk_scratch, g_tilde, va, st);
+        }
+        ep.tile_n = kProjBN;
+        const GemmShape sh = make_shape(Tc, d, V, kProjBN, 1, band_for(true), kPairBM);
+        const cudaError_t e = run_gemm_pair<kProjBN, false, true, kPairStages, 1, EpiProjVjp>(
+            maps, ep, sh, status, st, split > 1 ? sk_scratch : nullptr, &plan, split);
         if (e != cudaSuccess) return e;
-        return launch_sk_fixup_vjp<kWideBN>(plan, sh, sk_scratch, g_tilde, va, st);
+        return launch_sk_fixup_vjp<kProjBN>(plan, sh, sk_scratch, g_tilde, va, st);
     }
     ep.tile_n = kProjBN;
     if (use_pair())
@@ -552,8 +610,8 @@ cudaError_t launch_proj_vjp_bf16(const void* P, const void* W_U, const int32_t* 
         maps, ep, make_shape(Tc, d, V, kProjBN, 1, band_for(false)), status, st);
 }
 
-cudaError_t launch_proj_bf16(const void* E, const void* W_U, int Tc, int d, int V, float* g,
-                             float* sk_scratch, unsigned* status, cudaStream_t st) {
+cudaError_t launch_proj_bf16(const void* E, const void* W_U, int Tc, int T_all, int d, int V,
+                             float* g, float* sk_scratch, unsigned* status, cudaStream_t st) {
     GemmMaps<1> maps;
     if (!map_kmajor(&maps.a[0], E, Tc, V, kBM) || !map_mnmajor(&maps.b[0], W_U, V, d))
         return cudaErrorInvalidValue;
@@ -562,12 +620,20 @@ cudaError_t launch_proj_bf16(const void* E, const void* W_U, int Tc, int d, int 
     ep.M = Tc;
     ep.N = d;
     if (wide_proj()) {
-        const GemmShape sh = make_shape(Tc, d, V, kWideBN, 1, band_for(true), kPairBM);
         SkPlan plan;
-        cudaError_t e = run_gemm_pair<kWideBN, false, true, kWideStages, 1, EpiStoreF32>(
-            maps, ep, sh, status, st, sk_scratch, &plan);
+        const int split = proj_split(T_all, d, V);
+        if (split == 0) {
+            const GemmShape sh = make_shape(Tc, d, V, kWideBN, 1, band_for(true), kPairBM);
+            const cudaError_t e = run_gemm_pair<kWideBN, false, true, kWideStages, 1, EpiStoreF32>(
+                maps, ep, sh, status, st, sk_scratch, &plan);
+            if (e != cudaSuccess) return e;
+            return launch_sk_fixup<kWideBN>(plan, sh, sk_scratch, g, st);
+        }
+        const GemmShape sh = make_shape(Tc, d, V, kProjBN, 1, band_for(true), kPairBM);
+        const cudaError_t e = run_gemm_pair<kProjBN, false, true, kPairStages, 1, EpiStoreF32>(
+            maps, ep, sh, status, st, split > 1 ? sk_scratch : nullptr, &plan, split);
         if (e != cudaSuccess) return e;
-        return launch_sk_fixup<kWideBN>(plan, sh, sk_scratch, g, st);
+        return launch_sk_fixup<kProjBN>(plan, sh, sk_scratch, g, st);
     }
     if (use_pair())
         return run_gemm_pair<kProjBN, false, true, kPairStages, 1, EpiStoreF32>(

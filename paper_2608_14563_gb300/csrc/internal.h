@@ -61,10 +61,11 @@ cudaError_t launch_error_bf16(const void* yhat, const void* W_U, const int32_t* 
                               int Tc, int d, int V, float s, void* E, unsigned* status,
                               cudaStream_t st);
 
-// Projection: g[Tc, d] = E[Tc, V] W_U (fp32 out).  sk_scratch: proj_sk_scratch_bytes() of
-// device memory for the split-K tail of the 256 x 512 kernel (or null: whole tiles only).
-cudaError_t launch_proj_bf16(const void* E, const void* W_U, int Tc, int d, int V, float* g,
-                             float* sk_scratch, unsigned* status, cudaStream_t st);
+// Projection: g[Tc, d] = E[Tc, V] W_U (fp32 out).  T_all: the rows of the whole batch (the
+// split of K is chosen from it, whatever the chunking).  sk_scratch:
+// proj_sk_scratch_bytes() of device memory for the fp32 parts of split tiles.
+cudaError_t launch_proj_bf16(const void* E, const void* W_U, int Tc, int T_all, int d, int V,
+                             float* g, float* sk_scratch, unsigned* status, cudaStream_t st);
 size_t proj_sk_scratch_bytes();
 
 // Direct algorithm, logits pass anchored at c = anchor[t] (z never stored):
@@ -93,8 +94,8 @@ cudaError_t launch_fixup_logits_bf16(const void* yfix, const void* W_U, const in
 cudaError_t launch_proj_vjp_bf16(const void* P, const void* W_U, const int32_t* y,
                                  const float* alpha, const float* beta, const float* cv,
                                  const float* rho, const void* h, const void* w, float min_rms,
-                                 int Tc, int d, int V, void* g_tilde, float* sk_scratch,
-                                 unsigned* status, cudaStream_t st);
+                                 int Tc, int T_all, int d, int V, void* g_tilde,
+                                 float* sk_scratch, unsigned* status, cudaStream_t st);
 
 // Grouped pseudogradient update over n layers, layer l with signal g[l] (host array).
 cudaError_t launch_update_bf16(int n, int T, int d, int d_ff, const void* const* g,

@@ -277,3 +277,34 @@ def test_update_is_bitwise_identical_across_gemm_kernels(fpo, shape):
     for o in outs[1:]:
         for a, b in zip(outs[0], o):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("algo", [2, 3])  # stored logits, direct
+@pytest.mark.parametrize("shape", [(300, 520, 8200), (33, 264, 4104), (257, 256, 20000)])
+def test_projection_of_a_small_batch_split_over_k(fpo, algo, shape):
+    """Batches of fewer 256 x 512 projection tiles than pair clusters split every tile's K
+    loop into ranges of at least 32 k-blocks (2048 vocabulary entries) and sum them in the
+    fixup kernel: against whole tiles (the 256 x 256 kernel), the oracle, and across
+    chunkings (the split depends on the batch only); every third token is clamped."""
+    T, d, V = shape
+    wl = Workload("skb", T=T, d=d, d_ff=8, V=V, layers=1, targets="zipf")
+    inp = synth.make_all(wl)
+    h, w, W_U, y = inp["h"], inp["w"], inp["W_U"], inp["y"]
+    h[::3] *= 0.2
+    prev = fpo.set_gemm_variant(2)
+    try:
+        runs = [run(fpo, h, w, W_U, y, eps=wl.eps, algo=algo, t_chunk=c) for c in (0, 100, 31)]
+        fpo.set_gemm_variant(1)
+        whole = f64(run(fpo, h, w, W_U, y, eps=wl.eps, algo=algo)["g"])
+    finally:
+        fpo.set_gemm_variant(prev)
+    for r in runs[1:]:
+        assert torch.equal(runs[0]["g"], r["g"])
+    g = f64(runs[0]["g"])
+    # The fp32 sums reassociated: the tensor core adds 16 products at a time, each addition
+    # off by at most 2^-24 of the sum, so two orders differ by at most delta = V/16 2^-24 of
+    # it; a bf16 rounding (spacing 2^-8) then flips with probability delta / 2^-8 and changes
+    # the value by 2^-8 of itself: sqrt(delta 2^-8) in norm (a lost range would be O(1)).
+    assert rel_frob(g, whole) < np.sqrt(V / 16 * 2.0 ** -24 * 2.0 ** -8)
+    ref = reference(h, w, W_U, y, eps=wl.eps, s=wl.loss_scale)
+    assert rel_frob(g, ref["g_tilde"]) < TOL and cos(g, ref["g_tilde"]) >= COS_MIN
