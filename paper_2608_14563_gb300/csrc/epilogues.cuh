@@ -7,6 +7,16 @@
 // belong to the zero-filled tile overhang and are never written.  Dense
 // outputs go through the warp's swizzled staging buffers and TMA stores
 // (one 32-row x 128-byte box per store; the TMA engine clips the overhang).
+//
+// Epilogues that read or update matrices of the output's shape (the update, the
+// optimizer's first pass, the cosine, the gate / up signals, plain G) have 8 warps
+// (Epi::kWarps) and the form of epilogue_tile's second half: a chunk is staged in shared
+// memory and each lane takes 4 columns of 8 rows, so that every global access of a warp
+// covers whole row segments, and the operands of the next chunk (of the first chunk:
+// while the mainloop runs) are loaded as soon as their registers are free.  One row per
+// thread, as these epilogues had it with 4 warps, made every 16-byte access of a warp
+// touch 32 rows and kept 16 KB in flight per SM: AdamW with the step clip at T 4096,
+// d 4096, d_ff 11008, 8 layers took 4154 us in the GEMM for 1.5 ms of tensor work.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -26,6 +36,7 @@ namespace fpo {
 // the fp32 logits are also written to z [M, ldz] (stored-logits algorithm).
 template <bool kStoreZ>
 struct EpiLsePartialT {
+    static constexpr int kWarps = 4;
     struct Params {
         CUtensorMap zmap;  // fp32 logits [M, N], box 32 x 32 (kStoreZ only)
         float2* part;      // [M, part_ld]: (max, sum exp(z - max)) per vocabulary tile
@@ -109,6 +120,7 @@ using EpiLseStoreZ = EpiLsePartialT<true>;
 // per row) take a branch-free path on packed f32x2 arithmetic; two 32-column chunks
 // fill one 64-column bf16 staging row before each TMA store.
 struct EpiAnchorProb {
+    static constexpr int kWarps = 4;
     struct Params {
         CUtensorMap pmap;     // bf16 P [M, N], box 64 x 32
         float* su;            // [M, part_ld] sum of p~ over the tile
@@ -203,6 +215,7 @@ struct EpiAnchorProb {
 // sum of exponentials per (row, 256-column tile), written to part[row of the chunk,
 // tile], from which lse is formed before the second pass (EpiFixProb).
 struct EpiFixLse {
+    static constexpr int kWarps = 4;
     struct Params {
         float2* part;        // [T, part_ld] (max, sum exp(z - max))
         int part_ld;
@@ -251,6 +264,7 @@ struct EpiFixLse {
 // the row's sums over the tile of the rounded values and of the rounded values
 // times z go to sx[row, tile] and qz[row, tile], as EpiAnchorProb leaves them.
 struct EpiFixProb {
+    static constexpr int kWarps = 4;
     struct Params {
         __nv_bfloat16* P;    // [T, N] rows of the chunk, row stride N
         float* sx;           // [T, n_tiles]
@@ -310,6 +324,7 @@ struct EpiFixProb {
 // to bf16 into the error matrix E [M, N]; two 32-column chunks fill one
 // 64-column bf16 staging row before each TMA store.
 struct EpiError {
+    static constexpr int kWarps = 4;
     struct Params {
         CUtensorMap Emap;  // bf16 E [M, N], box 64 x 32
         const float* lse;  // [M]
@@ -356,6 +371,7 @@ struct EpiError {
 // ---------------------------------------------------------------------------
 // Plain fp32 store of C [M, N]: the projection g = E W_U (Eq. gproj).
 struct EpiStoreF32 {
+    static constexpr int kWarps = 4;
     struct Params {
         CUtensorMap Cmap;  // fp32 C [M, N], box 32 x 32
         int M, N;
@@ -394,6 +410,7 @@ struct EpiStoreF32 {
 // W_U[y] values of the next 32-column chunk are loaded while the current one is
 // processed; two chunks fill one 64-column bf16 staging row per TMA store.
 struct EpiProjVjp {
+    static constexpr int kWarps = 4;
     struct Params {
         CUtensorMap omap;           // bf16 g~ [M, N], box 64 x 32
         const float* alpha;         // [M]
@@ -504,11 +521,46 @@ struct EpiProjVjp {
     __device__ __forceinline__ void finish(const Params&, int) {}
 };
 
+// A lane's place in a warp's 32 rows of an 8-warp epilogue: its columns 4 (lane mod 8) ..
+// of the rows lane / 8, lane / 8 + 4, ... (8 of them), as element offsets into matrices
+// of row stride ld.
+struct QuadPos {
+    long long off;    // of the lane's first element
+    int rows, cols;   // rows from its first row, columns from its first column, in the matrix
+
+    __device__ __forceinline__ QuadPos(int M, int N, long long ld, int row0, int n0, int lane) {
+        const int r = row0 + (lane >> 3), c = n0 + 4 * (lane & 7);
+        off = r * ld + c;
+        rows = M - r;
+        cols = N - c;
+    }
+    // Row i of the lane (4 i rows below its first) and column offset co are inside
+    // (N is a multiple of 8, so the 4 columns are inside together).
+    __device__ __forceinline__ bool in(int i, int co) const { return 4 * i < rows && co < cols; }
+};
+
+// Slots of per-warp partial sums per (256-row block, 256-column tile): 8 blocks of 32 rows
+// times the two column halves of the 8-warp epilogues.
+constexpr int kColSlots = 16;
+
+__device__ __forceinline__ long long quad_slot(int g, int m256, int n_blocks, int nb, int row0,
+                                               int n0) {
+    return ((static_cast<long long>(g) * m256 + row0 / 256) * n_blocks + nb) * kColSlots +
+           ((n0 & 128) >> 4) + (row0 % 256) / 32;
+}
+
+__device__ __forceinline__ float warp_sum_f32(float x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
 // ---------------------------------------------------------------------------
 // Pseudogradient update (Eq. w3update, App. A): for group (layer) g,
 //   W_master[g] -= lr * G ;  W_out[g] = bf16(W_master[g]) ;  G_out[g] = bf16(G)
 // Any of the three pointers may be null for a layer.
 struct EpiUpdate {
+    static constexpr int kWarps = 8;
     struct Params {
         float* W_master[kMaxGroups];
         __nv_bfloat16* W_out[kMaxGroups];
@@ -517,129 +569,101 @@ struct EpiUpdate {
         int M, N;
         float neg_lr;
     };
-    int row, g;
-    bool valid;
+    QuadPos pos;
+    float* wm;
+    __nv_bfloat16* wo;
+    __nv_bfloat16* go;
+    float4 w[8];  // master values of the chunk that chunk() works on next
 
-    __device__ __forceinline__ EpiUpdate(const Params& p, int g_, int row_, int) : row(row_), g(g_) {
-        valid = row_ < p.M;
-    }
-
-    __device__ __forceinline__ void chunk(const Params& p, const float (&v)[32], int col0, int,
-                                          EpiIO&) {
-        const int lim = p.N - col0;
-        if (!valid || lim <= 0) return;
-        const long long off = row * p.ld + col0;
-        float* wm = p.W_master[g];
-        __nv_bfloat16* wo = p.W_out[g];
-        __nv_bfloat16* go = p.G_out[g];
+    __device__ __forceinline__ EpiUpdate(const Params& p, int g, int row0, int n0, int lane)
+        : pos(p.M, p.N, p.ld, row0, n0, lane) {
+        wm = p.W_master[g];
+        wo = p.W_out[g];
+        go = p.G_out[g];
         if (wm) {
-            float4* wp = reinterpret_cast<float4*>(wm + off);
-            uint4* op = reinterpret_cast<uint4*>(wo + off);
-            // every master load of the chunk is issued before the first store (which the
-            // compiler cannot reorder across, as W_out might alias W_master): one memory
-            // round trip per chunk instead of four
-            float4 ma[4], mb[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (q * 8 < lim) {
-                    ma[q] = wp[2 * q];
-                    mb[q] = wp[2 * q + 1];
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (q * 8 >= lim) break;
-                float4 a = ma[q], b = mb[q];
-                a.x = fmaf(p.neg_lr, v[8 * q + 0], a.x);
-                a.y = fmaf(p.neg_lr, v[8 * q + 1], a.y);
-                a.z = fmaf(p.neg_lr, v[8 * q + 2], a.z);
-                a.w = fmaf(p.neg_lr, v[8 * q + 3], a.w);
-                b.x = fmaf(p.neg_lr, v[8 * q + 4], b.x);
-                b.y = fmaf(p.neg_lr, v[8 * q + 5], b.y);
-                b.z = fmaf(p.neg_lr, v[8 * q + 6], b.z);
-                b.w = fmaf(p.neg_lr, v[8 * q + 7], b.w);
-                wp[2 * q] = a;
-                wp[2 * q + 1] = b;
-                if (wo)
-                    op[q] = make_uint4(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w),
-                                       pack_bf16x2(b.x, b.y), pack_bf16x2(b.z, b.w));
-            }
-        }
-        if (go) {
-            uint4* gp = reinterpret_cast<uint4*>(go + off);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (q * 8 < lim)
-                    gp[q] = make_uint4(pack_bf16x2(v[8 * q], v[8 * q + 1]),
-                                       pack_bf16x2(v[8 * q + 2], v[8 * q + 3]),
-                                       pack_bf16x2(v[8 * q + 4], v[8 * q + 5]),
-                                       pack_bf16x2(v[8 * q + 6], v[8 * q + 7]));
+            for (int i = 0; i < 8; ++i)
+                if (pos.in(i, 0)) w[i] = *reinterpret_cast<const float4*>(wm + pos.off + 4 * i * p.ld);
         }
     }
 
-    __device__ __forceinline__ void finish(const Params&, int) {}
+    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co,
+                                          bool more) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 v = out_read_quad(buf, lane, i);
+            const long long o = pos.off + 4 * i * p.ld + co;
+            const bool in = pos.in(i, co);
+            if (wm) {
+                float4 a = w[i];
+                a.x = fmaf(p.neg_lr, v.x, a.x);
+                a.y = fmaf(p.neg_lr, v.y, a.y);
+                a.z = fmaf(p.neg_lr, v.z, a.z);
+                a.w = fmaf(p.neg_lr, v.w, a.w);
+                if (in) {
+                    *reinterpret_cast<float4*>(wm + o) = a;
+                    if (wo)
+                        *reinterpret_cast<uint2*>(wo + o) =
+                            make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
+                }
+                if (more && pos.in(i, co + 32)) w[i] = *reinterpret_cast<const float4*>(wm + o + 32);
+            }
+            if (go && in)
+                *reinterpret_cast<uint2*>(go + o) =
+                    make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
+        }
+    }
+
+    __device__ __forceinline__ void finish(const Params&, int, int) {}
 };
 
 // ---------------------------------------------------------------------------
 // Pseudogradients with the layer-viability diagnostic's cosine (Sec. 2.2 Eq. (cosine),
 // Eq. (w3update)): for group (layer) g, G_out[g] = bf16(G), and the three sums of the
-// cosine of that stored G against Y[g] (<G, Y>, ||G||^2, ||Y||^2) over the thread's
-// row of the tile, summed over the warp's 32 rows (a fixed butterfly) and written as one
-// triple per (layer, 256-row block, column tile, 32-row slot):
-//   part[(((g m256 + row / 256) n_blocks + nb) 8 + (row mod 256) / 32) 3 + {0, 1, 2}]
-// so the cosine needs no second pass over G.  The Y values of the next 32-column chunk
-// are loaded while the current one is processed.
+// cosine of that stored G against Y[g] (<G, Y>, ||G||^2, ||Y||^2) over the warp's 32 rows
+// x 128 columns (fp32 per lane, then a fixed butterfly), one triple per quad_slot, so the
+// cosine needs no second pass over G.
 struct EpiGradCos {
+    static constexpr int kWarps = 8;
     struct Params {
         __nv_bfloat16* G_out[kMaxGroups];
         const __nv_bfloat16* Y[kMaxGroups];
-        float* part;     // [groups][m256][n_blocks][8][3]
+        float* part;     // [groups][m256][n_blocks][kColSlots][3]
         long long ld;
         int M, N;
         int m256, n_blocks;
     };
-    static constexpr int kTileN = 256;  // columns of the tiles it runs on (both GEMM kernels)
-    int row, g, n_end;
-    bool valid;
+    QuadPos pos;
+    int g, row0, n0;
     float2 s_gy, s_gg, s_yy;
-    uint4 uy[4];  // Y of the chunk the next chunk() call works on
+    uint2 y[8];  // Y of the chunk that chunk() works on next
 
-    __device__ __forceinline__ void fetch(const Params& p, int col0) {
-        const int lim = p.N - col0;
-        const uint4* py = reinterpret_cast<const uint4*>(p.Y[g] + row * p.ld + col0);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            uy[q] = (valid && q * 8 < lim) ? __ldg(py + q) : make_uint4(0, 0, 0, 0);
+    __device__ __forceinline__ uint2 load(const Params& p, int i, int co) const {
+        return pos.in(i, co) ? __ldg(reinterpret_cast<const uint2*>(p.Y[g] + pos.off + 4 * i * p.ld + co))
+                             : make_uint2(0, 0);
     }
 
-    __device__ __forceinline__ EpiGradCos(const Params& p, int g_, int row_, int n0)
-        : row(row_), g(g_) {
-        valid = row_ < p.M;
-        n_end = n0 + kTileN;
+    __device__ __forceinline__ EpiGradCos(const Params& p, int g_, int row0_, int n0_, int lane)
+        : pos(p.M, p.N, p.ld, row0_, n0_, lane), g(g_), row0(row0_), n0(n0_) {
         s_gy = s_gg = s_yy = make_float2(0.f, 0.f);
-        if (n0 < p.N) fetch(p, n0);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) y[i] = load(p, i, 0);
     }
 
-    __device__ __forceinline__ void chunk(const Params& p, const float (&v)[32], int col0, int,
-                                          EpiIO&) {
-        uint4 cy[4];
+    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co,
+                                          bool more) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) cy[q] = uy[q];
-        if (col0 + 32 < n_end && col0 + 32 < p.N) fetch(p, col0 + 32);
-        const int lim = p.N - col0;
-        if (!valid || lim <= 0) return;
-        uint4* gp = reinterpret_cast<uint4*>(p.G_out[g] + row * p.ld + col0);
+        for (int i = 0; i < 8; ++i) {
+            const float4 v = out_read_quad(buf, lane, i);
+            const uint32_t pk[2] = {pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w)};
+            // outside the matrix G is 0 (zero-filled operands) and Y was loaded as 0
+            const uint32_t yk[2] = {y[i].x, y[i].y};
+            if (pos.in(i, co))
+                *reinterpret_cast<uint2*>(p.G_out[g] + pos.off + 4 * i * p.ld + co) =
+                    make_uint2(pk[0], pk[1]);
+            if (more) y[i] = load(p, i, co + 32);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t pk[4] = {pack_bf16x2(v[8 * q], v[8 * q + 1]),
-                                    pack_bf16x2(v[8 * q + 2], v[8 * q + 3]),
-                                    pack_bf16x2(v[8 * q + 4], v[8 * q + 5]),
-                                    pack_bf16x2(v[8 * q + 6], v[8 * q + 7])};
-            if (q * 8 < lim) gp[q] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-            // columns >= N: G is 0 there (zero-filled operand) and Y was loaded as 0
-            const uint32_t yk[4] = {cy[q].x, cy[q].y, cy[q].z, cy[q].w};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
+            for (int k = 0; k < 2; ++k) {
                 const float2 gr = make_float2(__uint_as_float(pk[k] << 16),
                                               __uint_as_float(pk[k] & 0xffff0000u));
                 const float2 yr = make_float2(__uint_as_float(yk[k] << 16),
@@ -651,19 +675,11 @@ struct EpiGradCos {
         }
     }
 
-    __device__ __forceinline__ void finish(const Params& p, int nb) {
-        float gy = s_gy.x + s_gy.y, gg = s_gg.x + s_gg.y, yy = s_yy.x + s_yy.y;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            gy += __shfl_xor_sync(0xffffffffu, gy, o);
-            gg += __shfl_xor_sync(0xffffffffu, gg, o);
-            yy += __shfl_xor_sync(0xffffffffu, yy, o);
-        }
-        if ((threadIdx.x & 31) == 0) {
-            const long long slot =
-                ((static_cast<long long>(g) * p.m256 + row / 256) * p.n_blocks + nb) * 8 +
-                (row % 256) / 32;
-            float* o = p.part + slot * 3;
+    __device__ __forceinline__ void finish(const Params& p, int nb, int lane) {
+        const float gy = warp_sum_f32(s_gy.x + s_gy.y), gg = warp_sum_f32(s_gg.x + s_gg.y),
+                    yy = warp_sum_f32(s_yy.x + s_yy.y);
+        if (lane == 0) {
+            float* o = p.part + quad_slot(g, p.m256, p.n_blocks, nb, row0, n0) * 3;
             o[0] = gy;
             o[1] = gg;
             o[2] = yy;
@@ -675,30 +691,27 @@ struct EpiGradCos {
 // Pseudogradient only, fp32, one output per group (layer): G[g] = g~^T A_l, for
 // the optimizers that need the whole G (and its norm) before they step.
 struct EpiStoreGroupF32 {
+    static constexpr int kWarps = 8;
     struct Params {
         float* G[kMaxGroups];
         long long ld;
         int M, N;
     };
-    int row, g;
-    bool valid;
+    QuadPos pos;
+    float* G;
 
-    __device__ __forceinline__ EpiStoreGroupF32(const Params& p, int g_, int row_, int)
-        : row(row_), g(g_) {
-        valid = row_ < p.M;
-    }
+    __device__ __forceinline__ EpiStoreGroupF32(const Params& p, int g, int row0, int n0, int lane)
+        : pos(p.M, p.N, p.ld, row0, n0, lane), G(p.G[g]) {}
 
-    __device__ __forceinline__ void chunk(const Params& p, const float (&v)[32], int col0, int,
-                                          EpiIO&) {
-        const int lim = p.N - col0;
-        if (!valid || lim <= 0) return;
-        float4* dst = reinterpret_cast<float4*>(p.G[g] + row * p.ld + col0);
+    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co, bool) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            if (q * 4 < lim) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        for (int i = 0; i < 8; ++i) {
+            const float4 v = out_read_quad(buf, lane, i);
+            if (pos.in(i, co)) *reinterpret_cast<float4*>(G + pos.off + 4 * i * p.ld + co) = v;
+        }
     }
 
-    __device__ __forceinline__ void finish(const Params&, int) {}
+    __device__ __forceinline__ void finish(const Params&, int, int) {}
 };
 
 // ---------------------------------------------------------------------------
@@ -706,91 +719,95 @@ struct EpiStoreGroupF32 {
 // clip on the step (Sec. 3.1: SGD, SGD with momentum, AdamW on the fp32 masters; App. A:
 // ||dW|| <= clip_frac ||W||).  With G from the accumulator, each element's optimizer state
 // advances and its unclipped step d = opt_step(G, W, s1, s2) is stored (fp32, D[g]; the
-// state sees the unclipped gradient), and ||W||^2, ||d||^2 of the warp's 32 rows of the
-// tile are written as one pair per (layer, 256-row block, column tile, 32-row slot); a
-// kernel then scales each layer's steps by min(1, clip_frac ||W|| / ||d||) and applies
-// them (W is not written here, so its norm is the pre-step one).  Without a clip the
-// stand-alone passes are used: taking the whole step here made the update faster but
-// the power-capped step slower (its epilogue then held the tensor pipe back at full
-// draw).
+// state sees the unclipped gradient), and ||W||^2, ||d||^2 of the warp's 32 rows x 128
+// columns are written as one pair per quad_slot; a kernel then scales each layer's steps
+// by min(1, clip_frac ||W|| / ||d||) and applies them (W is not written here, so its norm
+// is the pre-step one).  Without a clip the stand-alone passes are used: taking the whole
+// step here made the update faster but the power-capped step slower (its epilogue then
+// held the tensor pipe back at full draw).
+// The operands of 4 of the chunk's 8 row quads are in flight at a time (48 registers).
 struct EpiOptStep {
+    static constexpr int kWarps = 8;
     struct Params {
         const float* W_master[kMaxGroups];
         float* s1[kMaxGroups];             // momentum / AdamW first moment (or null)
         float* s2[kMaxGroups];             // AdamW second moment (or null)
         float* D[kMaxGroups];              // the unclipped steps
-        float* part;                       // [groups][m256][n_blocks][8][2]
+        float* part;                       // [groups][m256][n_blocks][kColSlots][2]
         OptimParams op;
         long long ld;
         int M, N;
         int m256, n_blocks;
     };
-    int row, g;
-    bool valid;
+    static constexpr int kAhead = 4;
+    QuadPos pos;
+    int g, row0, n0;
+    const float* wm;
+    float* p1;
+    float* p2;
+    float* D;
     float s_ww, s_dd;
+    float4 w[kAhead], a[kAhead], b[kAhead];  // of the next kAhead row quads
 
-    __device__ __forceinline__ EpiOptStep(const Params& p, int g_, int row_, int)
-        : row(row_), g(g_), s_ww(0.f), s_dd(0.f) {
-        valid = row_ < p.M;
+    __device__ __forceinline__ void load(const Params& p, int k, int i, int co) {
+        w[k] = a[k] = b[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (!pos.in(i, co)) return;
+        const long long o = pos.off + 4 * i * p.ld + co;
+        w[k] = *reinterpret_cast<const float4*>(wm + o);
+        if (p1) a[k] = *reinterpret_cast<const float4*>(p1 + o);
+        if (p2) b[k] = *reinterpret_cast<const float4*>(p2 + o);
     }
 
-    __device__ __forceinline__ void chunk(const Params& p, const float (&v)[32], int col0, int,
-                                          EpiIO&) {
-        const int lim = p.N - col0;
-        if (!valid || lim <= 0) return;
-        const long long off = row * p.ld + col0;
-        const float4* wp = reinterpret_cast<const float4*>(p.W_master[g] + off);
-        float4* p1 = p.s1[g] ? reinterpret_cast<float4*>(p.s1[g] + off) : nullptr;
-        float4* p2 = p.s2[g] ? reinterpret_cast<float4*>(p.s2[g] + off) : nullptr;
+    __device__ __forceinline__ EpiOptStep(const Params& p, int g_, int row0_, int n0_, int lane)
+        : pos(p.M, p.N, p.ld, row0_, n0_, lane), g(g_), row0(row0_), n0(n0_), s_ww(0.f), s_dd(0.f) {
+        wm = p.W_master[g_];
+        p1 = p.s1[g_];
+        p2 = p.s2[g_];
+        D = p.D[g_];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {  // 16 columns at a time
-            if (h * 16 >= lim) break;
-            float w[16], a[16], b[16];
+        for (int k = 0; k < kAhead; ++k) load(p, k, k, 0);
+    }
+
+    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co,
+                                          bool more) {
+#pragma unroll 1
+        for (int h = 0; h < 8; h += kAhead) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int c4 = 4 * h + q;  // float4 index in the chunk
-                if (c4 * 4 < lim) {
-                    const float4 x = wp[c4];
-                    w[4 * q] = x.x; w[4 * q + 1] = x.y; w[4 * q + 2] = x.z; w[4 * q + 3] = x.w;
-                    const float4 y = p1 ? p1[c4] : make_float4(0.f, 0.f, 0.f, 0.f);
-                    a[4 * q] = y.x; a[4 * q + 1] = y.y; a[4 * q + 2] = y.z; a[4 * q + 3] = y.w;
-                    const float4 z = p2 ? p2[c4] : make_float4(0.f, 0.f, 0.f, 0.f);
-                    b[4 * q] = z.x; b[4 * q + 1] = z.y; b[4 * q + 2] = z.z; b[4 * q + 3] = z.w;
+            for (int k = 0; k < kAhead; ++k) {
+                const int i = h + k;
+                const float4 v4 = out_read_quad(buf, lane, i);
+                const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+                const float wv[4] = {w[k].x, w[k].y, w[k].z, w[k].w};
+                float av[4] = {a[k].x, a[k].y, a[k].z, a[k].w};
+                float bv[4] = {b[k].x, b[k].y, b[k].z, b[k].w};
+                float out[4];
+                const bool in = pos.in(i, co);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    out[e] = opt_step(p.op, v[e], wv[e], av[e], bv[e]);
+                    if (in) {
+                        s_ww = fmaf(wv[e], wv[e], s_ww);
+                        s_dd = fmaf(out[e], out[e], s_dd);
+                    }
                 }
-            }
-            float out[16];
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                out[e] = opt_step(p.op, v[16 * h + e], w[e], a[e], b[e]);
-                if (16 * h + e < lim) {  // (columns past N were not loaded)
-                    s_ww = fmaf(w[e], w[e], s_ww);
-                    s_dd = fmaf(out[e], out[e], s_dd);
+                if (in) {
+                    const long long o = pos.off + 4 * i * p.ld + co;
+                    *reinterpret_cast<float4*>(D + o) = make_float4(out[0], out[1], out[2], out[3]);
+                    if (p1) *reinterpret_cast<float4*>(p1 + o) = make_float4(av[0], av[1], av[2], av[3]);
+                    if (p2) *reinterpret_cast<float4*>(p2 + o) = make_float4(bv[0], bv[1], bv[2], bv[3]);
                 }
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int c4 = 4 * h + q;
-                if (c4 * 4 >= lim) break;
-                reinterpret_cast<float4*>(p.D[g] + off)[c4] =
-                    make_float4(out[4 * q], out[4 * q + 1], out[4 * q + 2], out[4 * q + 3]);
-                if (p1) p1[c4] = make_float4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]);
-                if (p2) p2[c4] = make_float4(b[4 * q], b[4 * q + 1], b[4 * q + 2], b[4 * q + 3]);
+                if (h == 0)
+                    load(p, k, i + kAhead, co);
+                else if (more)
+                    load(p, k, i - kAhead, co + 32);
             }
         }
     }
 
-    __device__ __forceinline__ void finish(const Params& p, int nb) {
-        float ww = s_ww, dd = s_dd;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            ww += __shfl_xor_sync(0xffffffffu, ww, o);
-            dd += __shfl_xor_sync(0xffffffffu, dd, o);
-        }
-        if ((threadIdx.x & 31) == 0) {
-            const long long slot =
-                ((static_cast<long long>(g) * p.m256 + row / 256) * p.n_blocks + nb) * 8 +
-                (row % 256) / 32;
-            float* o = p.part + slot * 2;
+    __device__ __forceinline__ void finish(const Params& p, int nb, int lane) {
+        const float ww = warp_sum_f32(s_ww), dd = warp_sum_f32(s_dd);
+        if (lane == 0) {
+            float* o = p.part + quad_slot(g, p.m256, p.n_blocks, nb, row0, n0) * 2;
             o[0] = ww;
             o[1] = dd;
         }
@@ -801,97 +818,66 @@ struct EpiOptStep {
 // Gate / up signals of a SwiGLU MLP (Sec. 3.1 step 5, Eq. errh): the GEMM gives
 // error_h = g W3_init; with the cached pre-activations a (gate) and b (up),
 //   dA = error_h (.) b (.) silu'(a),  dB = error_h (.) silu(a)   (bf16 out)
-// Each 64-column pair of chunks fills one dA and one dB staging buffer (the
-// warp's two buffers), stored by two TMA stores in one bulk group.
 struct EpiSwiglu {
+    static constexpr int kWarps = 8;
     struct Params {
-        CUtensorMap dAmap;  // bf16 [M, N], box 64 x 32
-        CUtensorMap dBmap;
+        __nv_bfloat16* dA;       // [M, N]
+        __nv_bfloat16* dB;
         const __nv_bfloat16* a;  // [M, N]
         const __nv_bfloat16* b;
         long long ld;
         int M, N;
     };
-    static constexpr int kTileN = 256;  // columns of the tiles it runs on (both GEMM kernels)
-    int row, n_end;
-    bool valid, pair_out;
-    // a and b of the chunk the next chunk() call works on: loaded one chunk ahead, so
-    // their latency overlaps the arithmetic of the chunk before (the first chunk's loads
-    // are issued by the constructor)
-    uint4 ua[4], ub[4];
+    QuadPos pos;
+    uint2 ua[8], ub[8];  // a and b of the chunk that chunk() works on next
 
-    __device__ __forceinline__ void fetch(const Params& p, int col0) {
-        const int lim = p.N - col0;
-        const uint4* pa = reinterpret_cast<const uint4*>(p.a + row * p.ld + col0);
-        const uint4* pb = reinterpret_cast<const uint4*>(p.b + row * p.ld + col0);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const bool in = valid && q * 8 < lim;
-            ua[q] = in ? pa[q] : make_uint4(0, 0, 0, 0);
-            ub[q] = in ? pb[q] : make_uint4(0, 0, 0, 0);
-        }
+    __device__ __forceinline__ void load(const Params& p, int i, int co) {
+        ua[i] = ub[i] = make_uint2(0, 0);
+        if (!pos.in(i, co)) return;
+        const long long o = pos.off + 4 * i * p.ld + co;
+        ua[i] = *reinterpret_cast<const uint2*>(p.a + o);
+        ub[i] = *reinterpret_cast<const uint2*>(p.b + o);
     }
 
-    __device__ __forceinline__ EpiSwiglu(const Params& p, int, int row_, int n0) : row(row_) {
-        valid = row_ < p.M;
-        pair_out = false;
-        n_end = n0 + kTileN;
-        fetch(p, n0);
+    __device__ __forceinline__ EpiSwiglu(const Params& p, int, int row0, int n0, int lane)
+        : pos(p.M, p.N, p.ld, row0, n0, lane) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) load(p, i, 0);
     }
 
-    __device__ __forceinline__ void chunk(const Params& p, const float (&v)[32], int col0, int c0,
-                                          EpiIO& io) {
-        const bool second = (c0 & 32) != 0;
-        uint4 ca[4], cb[4];
+    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co,
+                                          bool more) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            ca[q] = ua[q];
-            cb[q] = ub[q];
-        }
-        if (col0 + 32 < n_end) fetch(p, col0 + 32);
-        if (!second) {
-            pair_out = col0 >= p.N || io.row0 >= p.M;
-            if (pair_out) return;
-            if (io.lane == 0) bulk_wait_group_read<0>();  // both buffers free again
-            __syncwarp();
-        }
-        if (pair_out) return;
-        uint32_t wa[16], wb[16];
+        for (int i = 0; i < 8; ++i) {
+            const float4 v4 = out_read_quad(buf, lane, i);
+            const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+            const float xa[4] = {__uint_as_float(ua[i].x << 16), __uint_as_float(ua[i].x & 0xffff0000u),
+                                 __uint_as_float(ua[i].y << 16), __uint_as_float(ua[i].y & 0xffff0000u)};
+            const float xb[4] = {__uint_as_float(ub[i].x << 16), __uint_as_float(ub[i].x & 0xffff0000u),
+                                 __uint_as_float(ub[i].y << 16), __uint_as_float(ub[i].y & 0xffff0000u)};
+            if (more) load(p, i, co + 32);
+            float da[4], db[4];
 #pragma unroll
-        for (int j = 0; j < 32; j += 2) {
-            const __nv_bfloat162 ha = reinterpret_cast<const __nv_bfloat162*>(&ca[j / 8])[(j % 8) / 2];
-            const __nv_bfloat162 hb = reinterpret_cast<const __nv_bfloat162*>(&cb[j / 8])[(j % 8) / 2];
-            const float2 fa = __bfloat1622float2(ha), fb = __bfloat1622float2(hb);
-            const float xa[2] = {fa.x, fa.y}, xb[2] = {fb.x, fb.y};
-            float da[2], db[2];
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
+            for (int k = 0; k < 4; ++k) {
                 // sigmoid with the fast intrinsic divide: its few-ulp fp32 error is far
                 // below the bf16 rounding of dA and dB (for x < -87 it gives 0, as the
                 // exact value is below bf16's range there too)
                 const float x = xa[k];
                 const float sg = __fdividef(1.f, 1.f + __expf(-x));
-                da[k] = v[j + k] * xb[k] * sg * fmaf(x, 1.f - sg, 1.f);
-                db[k] = v[j + k] * x * sg;
+                da[k] = v[k] * xb[k] * sg * fmaf(x, 1.f - sg, 1.f);
+                db[k] = v[k] * x * sg;
             }
-            wa[j / 2] = pack_bf16x2(da[0], da[1]);
-            wb[j / 2] = pack_bf16x2(db[0], db[1]);
-        }
-        const uint32_t bufA = io.out, bufB = io.out + kOutBufBytes;
-        out_stage_half(bufA, io.lane, second ? 1 : 0, wa);
-        out_stage_half(bufB, io.lane, second ? 1 : 0, wb);
-        if (second) {
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (io.lane == 0) {
-                tma_store_2d(&p.dAmap, bufA, col0 - 32, io.row0);
-                tma_store_2d(&p.dBmap, bufB, col0 - 32, io.row0);
-                bulk_commit_group();
+            if (pos.in(i, co)) {
+                const long long o = pos.off + 4 * i * p.ld + co;
+                *reinterpret_cast<uint2*>(p.dA + o) =
+                    make_uint2(pack_bf16x2(da[0], da[1]), pack_bf16x2(da[2], da[3]));
+                *reinterpret_cast<uint2*>(p.dB + o) =
+                    make_uint2(pack_bf16x2(db[0], db[1]), pack_bf16x2(db[2], db[3]));
             }
         }
     }
 
-    __device__ __forceinline__ void finish(const Params&, int) {}
+    __device__ __forceinline__ void finish(const Params&, int, int) {}
 };
 
 }  // namespace fpo

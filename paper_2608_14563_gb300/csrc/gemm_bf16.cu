@@ -112,7 +112,7 @@ cudaError_t run_gemm(const GemmMaps<MAXG>& maps, const typename Epi::Params& ep,
     DevInfo di;
     if (!current_device_info(&di)) return cudaErrorUnknown;
     const long long grid = sh.tiles < di.sm_count ? sh.tiles : di.sm_count;
-    kern<<<static_cast<unsigned>(grid), kGemmThreads, L::kBytes, st>>>(maps, ep, sh, status,
+    kern<<<static_cast<unsigned>(grid), gemm_threads<Epi>(), L::kBytes, st>>>(maps, ep, sh, status,
                                                                       wait_limit_ns()),
         ::fpo::note_launch();
     return cudaGetLastError();
@@ -121,10 +121,10 @@ cudaError_t run_gemm(const GemmMaps<MAXG>& maps, const typename Epi::Params& ep,
 // Clusters (of `cta` CTAs, the kernel's cluster size) that can be resident at once for a
 // pair-kernel instantiation.
 template <class Kern>
-int pair_clusters(Kern kern, int smem_bytes, int sm_count, int cta) {
+int pair_clusters(Kern kern, int threads, int smem_bytes, int sm_count, int cta) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(sm_count / cta * cta), 1, 1);
-    cfg.blockDim = dim3(kGemmThreads, 1, 1);
+    cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
     cfg.dynamicSmemBytes = static_cast<size_t>(smem_bytes);
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
@@ -137,13 +137,13 @@ int pair_clusters(Kern kern, int smem_bytes, int sm_count, int cta) {
 // pair_clusters for the current device, computed once per device (after the kernel's
 // shared-memory limit is raised there).
 template <auto Kern>
-int resident_clusters(int smem_bytes, int sm_count, int cta) {
+int resident_clusters(int threads, int smem_bytes, int sm_count, int cta) {
     static std::atomic<int> cache[kMaxDevices];
     const int dev = current_device();
     if (dev < 0) return sm_count / cta;
     int n = cache[dev].load(std::memory_order_relaxed);
     if (n > 0) return n;
-    n = pair_clusters(Kern, smem_bytes, sm_count, cta);
+    n = pair_clusters(Kern, threads, smem_bytes, sm_count, cta);
     cache[dev].store(n, std::memory_order_relaxed);
     return n;
 }
@@ -195,7 +195,7 @@ cudaError_t run_gemm_pair(const GemmMaps<MAXG>& maps, const typename Epi::Params
     if (attr_err != cudaSuccess) return attr_err;
     DevInfo di;
     if (!current_device_info(&di)) return cudaErrorUnknown;
-    const int max_clusters = resident_clusters<kern>(L::kBytes, di.sm_count, 2);
+    const int max_clusters = resident_clusters<kern>(gemm_threads<Epi>(), L::kBytes, di.sm_count, 2);
     const long long units = split > 1 ? sh_in.tiles * split : sh_in.tiles;
     const long long clusters = units < max_clusters ? units : max_clusters;
     GemmShape sh = sh_in;
@@ -214,8 +214,8 @@ cudaError_t run_gemm_pair(const GemmMaps<MAXG>& maps, const typename Epi::Params
             if (plan) *plan = p;
         }
     }
-    kern<<<static_cast<unsigned>(2 * clusters), kGemmThreads, L::kBytes, st>>>(maps, ep, sh, status,
-                                                                              wait_limit_ns()),
+    kern<<<static_cast<unsigned>(2 * clusters), gemm_threads<Epi>(), L::kBytes, st>>>(
+        maps, ep, sh, status, wait_limit_ns()),
         ::fpo::note_launch();
     return cudaGetLastError();
 }
@@ -386,7 +386,7 @@ int proj_clusters() {
     DevInfo di;
     int c = 128;
     if (current_device_info(&di) && set_smem_limit<kern>(L::kBytes) == cudaSuccess)
-        c = resident_clusters<kern>(L::kBytes, di.sm_count, 2);
+        c = resident_clusters<kern>(gemm_threads<EpiProjVjp>(), L::kBytes, di.sm_count, 2);
     cudaGetLastError();
     return c;
 }
@@ -746,6 +746,12 @@ cudaError_t launch_opt_step_bf16(int n, int T, int d, int d_ff, const void* cons
     ep.N = d_ff;
     ep.m256 = (d + 255) / 256;
     ep.n_blocks = (d_ff + kUpdBN - 1) / kUpdBN;
+    // single-CTA 128-row tiles leave the upper half of a last, short 256-row block of slots
+    // unwritten: start from zeros
+    if (!use_pair()) {
+        const cudaError_t e = cudaMemsetAsync(part, 0, n * opt_step_partial_bytes(1, d, d_ff), st);
+        if (e != cudaSuccess) return e;
+    }
     if (use_pair())
         return run_gemm_pair<kUpdBN, true, true, kPairStages, kMaxGroups, EpiOptStep>(
             maps, ep, make_shape(d, d_ff, T, kUpdBN, n, band_for(true), kPairBM), status, st);
@@ -754,8 +760,8 @@ cudaError_t launch_opt_step_bf16(int n, int T, int d, int d_ff, const void* cons
 }
 
 size_t opt_step_partial_bytes(int n_layers, int d, int d_ff) {
-    return static_cast<size_t>(n_layers) * ((d + 255) / 256) * ((d_ff + kUpdBN - 1) / kUpdBN) * 8 *
-           2 * sizeof(float);
+    return static_cast<size_t>(n_layers) * ((d + 255) / 256) * ((d_ff + kUpdBN - 1) / kUpdBN) *
+           kColSlots * 2 * sizeof(float);
 }
 
 // Second pass of the fused cosine: one block per layer adds the layer's slot triples in a
@@ -808,7 +814,7 @@ __global__ void __launch_bounds__(kCosFinalThreads)
 size_t grad_cosine_partial_bytes(int n, int d, int d_ff) {
     const size_t m256 = (static_cast<size_t>(d) + 255) / 256;
     const size_t nb = (static_cast<size_t>(d_ff) + kUpdBN - 1) / kUpdBN;
-    return static_cast<size_t>(n) * m256 * nb * 8 * 3 * sizeof(float);
+    return static_cast<size_t>(n) * m256 * nb * kColSlots * 3 * sizeof(float);
 }
 
 cudaError_t launch_grad_cosine_bf16(int n, int T, int d, int d_ff, const void* const* g,
@@ -841,10 +847,10 @@ cudaError_t launch_grad_cosine_bf16(int n, int T, int d, int d_ff, const void* c
     ep.N = d_ff;
     ep.m256 = (d + 255) / 256;
     ep.n_blocks = (d_ff + kUpdBN - 1) / kUpdBN;
-    static_assert(EpiGradCos::kTileN == kUpdBN, "the cosine epilogue prefetches 256-column tiles");
     // every slot is written by a tile (pair kernel), but single-CTA 128-row tiles leave
     // the upper half of a last, short 256-row block unwritten: start from zeros
-    cudaError_t e = cudaMemsetAsync(part, 0, grad_cosine_partial_bytes(n, d, d_ff), st);
+    cudaError_t e = cudaSuccess;
+    if (!use_pair()) e = cudaMemsetAsync(part, 0, grad_cosine_partial_bytes(n, d, d_ff), st);
     if (e != cudaSuccess) return e;
     if (use_pair())
         e = run_gemm_pair<kUpdBN, true, true, kPairStages, kMaxGroups, EpiGradCos>(
@@ -853,7 +859,7 @@ cudaError_t launch_grad_cosine_bf16(int n, int T, int d, int d_ff, const void* c
         e = run_gemm<kUpdBN, true, true, kUpdStages, kMaxGroups, EpiGradCos>(
             maps, ep, make_shape(d, d_ff, T, kUpdBN, n, band_for(false)), status, st);
     if (e != cudaSuccess) return e;
-    grad_cosine_final_kernel<<<n, kCosFinalThreads, 0, st>>>(part, ep.m256 * ep.n_blocks * 8, out),
+    grad_cosine_final_kernel<<<n, kCosFinalThreads, 0, st>>>(part, ep.m256 * ep.n_blocks * kColSlots, out),
         ::fpo::note_launch();
     return cudaGetLastError();
 }
@@ -864,10 +870,9 @@ cudaError_t launch_swiglu_bf16(int T, int d, int d_ff, const void* g, const void
     GemmMaps<1> maps;
     if (!map_kmajor(&maps.a[0], g, T, d, kBM) || !map_mnmajor(&maps.b[0], W3, d, d_ff))
         return cudaErrorInvalidValue;
-    static_assert(EpiSwiglu::kTileN == 256, "the SwiGLU epilogue prefetches 256-column tiles");
     EpiSwiglu::Params ep;
-    if (!map_out_bf16(&ep.dAmap, dA, T, d_ff) || !map_out_bf16(&ep.dBmap, dB, T, d_ff))
-        return cudaErrorInvalidValue;
+    ep.dA = static_cast<__nv_bfloat16*>(dA);
+    ep.dB = static_cast<__nv_bfloat16*>(dB);
     ep.a = static_cast<const __nv_bfloat16*>(a);
     ep.b = static_cast<const __nv_bfloat16*>(b);
     ep.ld = d_ff;

@@ -2,13 +2,14 @@
 //
 //   C[g][m, n] = sum_k A(m, k) * B[g](n, k)      (bf16 inputs, fp32 accumulate)
 //
-// One CTA per SM (persistent over output tiles), 192 threads:
+// One CTA per SM (persistent over output tiles), 192 or 320 threads:
 //   warp 0      TMA producer: streams A/B k-blocks into a STAGES-deep ring of
 //               128-byte-swizzled shared-memory buffers (mbarrier full/empty).
 //   warp 1      allocates TMEM; lane 0 issues tcgen05.mma (128 x BN x 16) and
 //               commits stage releases / accumulator-ready signals.
-//   warps 2..5  epilogue: tcgen05.ld of the fp32 accumulator (one row per
-//               thread), hand the values to the Epilogue functor.
+//   warps 2..   epilogue (Epi::kWarps of them, 4 or 8): tcgen05.ld of the fp32
+//               accumulator (one row per thread), hand the values to the
+//               Epilogue functor.
 // The accumulator is double-buffered in TMEM (2 x BN columns) so the epilogue
 // of tile i overlaps the mainloop of tile i+1.
 //
@@ -27,7 +28,11 @@ namespace fpo {
 constexpr int kBM = 128;       // UMMA M (one TMEM lane per output row)
 constexpr int kBK = 64;        // k-block: 64 bf16 = one 128-byte swizzle row
 constexpr int kUmmaK = 16;     // K of one tcgen05.mma.kind::f16
-constexpr int kGemmThreads = 192;
+// Threads of a GEMM kernel: the producer and MMA warps, then the epilogue's.
+template <class Epi>
+constexpr int gemm_threads() {
+    return 64 + 32 * Epi::kWarps;
+}
 constexpr int kMaxGroups = 64;
 // Limit of the teardown waits for copies and MMAs already issued (they complete in
 // microseconds); fixed, so that a short wait limit cannot cut them off.
@@ -154,6 +159,62 @@ __device__ __forceinline__ void out_stage_half(uint32_t buf, int r, int h, const
                      w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
 }
 
+// A 32 x 32 fp32 chunk staged by out_stage_row, read back with 8 lanes to a row: the 4
+// columns 4 (lane mod 8) .. of row 4 i + lane / 8 (i in [0, 8)), so that a warp's global
+// accesses cover whole 128-byte row segments.
+__device__ __forceinline__ float4 out_read_quad(uint32_t buf, int lane, int i) {
+    const uint32_t r = 4u * static_cast<uint32_t>(i) + static_cast<uint32_t>(lane >> 3);
+    return ld_shared_f4(buf + r * 128u + ((static_cast<uint32_t>(lane & 7) ^ (r & 7u)) << 4));
+}
+
+// The epilogue's warps.  With Epi::kWarps = 4 each warp owns 32 rows of the CTA's 128 and
+// walks all BN columns, one row per thread (Epi(params, group, row, n0); chunk(params,
+// v[32], column, offset in the tile, io); finish(params, n_block)).  With 8, two warps
+// share the rows and take half of the columns each, and every 32 x 32 chunk goes through
+// the warp's staging buffer (Epi(params, group, first row, first column, lane);
+// chunk(params, staged chunk, lane, offset, another chunk follows); finish(params,
+// n_block, lane)).  The functor is made before the accumulator is awaited, so that what
+// its constructor loads arrives during the mainloop.  `ready` waits for the accumulator
+// (false: give up), `release` gives it back once its last columns are in registers.
+template <int BN, class Epi, class Ready, class Release>
+__device__ __forceinline__ bool epilogue_tile(const typename Epi::Params& ep, int g, int row0,
+                                              int nb, int warp_half, uint32_t t_row, EpiIO& io,
+                                              Ready ready, Release release) {
+    if constexpr (Epi::kWarps == 4) {
+        const int n0 = nb * BN;
+        io.row0 = row0;
+        Epi epi(ep, g, row0 + io.lane, n0);
+        if (!ready()) return false;
+#pragma unroll 1
+        for (int c = 0; c < BN / 32; ++c) {
+            float v[32];
+            tmem_ld_32x32b_x32(t_row + c * 32, v);
+            if (c == BN / 32 - 1) release();
+            epi.chunk(ep, v, n0 + c * 32, c * 32, io);
+        }
+        epi.finish(ep, nb);
+    } else {
+        constexpr int kCols = BN / 2;
+        Epi epi(ep, g, row0, nb * BN + warp_half * kCols, io.lane);
+        if (!ready()) return false;
+#pragma unroll 1
+        for (int c = 0; c < kCols / 32; ++c) {
+            float v[32];
+            tmem_ld_32x32b_x32(t_row + warp_half * kCols + c * 32, v);
+            if (c == kCols / 32 - 1) release();
+            uint32_t w[32];
+#pragma unroll
+            for (int j = 0; j < 32; ++j) w[j] = __float_as_uint(v[j]);
+            out_stage_row(io.out, io.lane, w);
+            __syncwarp();
+            epi.chunk(ep, io.out, io.lane, c * 32, c + 1 < kCols / 32);
+            __syncwarp();
+        }
+        epi.finish(ep, nb, io.lane);
+    }
+    return true;
+}
+
 // Store a filled staging buffer to (x, y) of `map` (rows/columns outside the
 // tensor are clipped by the TMA engine).
 __device__ __forceinline__ void out_commit(EpiIO& io, const CUtensorMap* map, uint32_t buf, int x,
@@ -168,7 +229,7 @@ __device__ __forceinline__ void out_commit(EpiIO& io, const CUtensorMap* map, ui
 }
 
 template <int BN, bool A_MN, bool B_MN, int STAGES, int MAXG, class Epi>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
     tc_gemm_kernel(const __grid_constant__ GemmMaps<MAXG> maps,
                    const __grid_constant__ typename Epi::Params ep, const GemmShape sh,
                    unsigned int* status, unsigned long long wait_limit_ns) {
@@ -201,7 +262,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(tfull_bar(a), 1);
-            mbar_init(tempty_bar(a), 4);
+            mbar_init(tempty_bar(a), Epi::kWarps);
         }
         mbar_init(drain_bar, 1);
         *abort_flag = 0;
@@ -293,32 +354,29 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     } else {
         // ------------------------------------------------------- epilogue
         const int q = warp & 3;  // TMEM lane quarter this warp may access
-        const int r_in_tile = q * 32 + lane;
-        EpiIO io{sbase + L::kOutOffset + static_cast<uint32_t>((warp - 2) * kOutBytesPerWarp), lane,
-                 0, 0u};
+        constexpr int kOutPerWarp = 4 * kOutBytesPerWarp / Epi::kWarps;
+        EpiIO io{sbase + L::kOutOffset + static_cast<uint32_t>((warp - 2) * kOutPerWarp), lane, 0,
+                 0u};
         int acc = 0;
         uint32_t acc_phase = 0;
         for (long long t = blockIdx.x; t < sh.tiles; t += gridDim.x) {
             int g, mb, nb;
             tile_coords(t, sh, g, mb, nb);
-            if (!mbar_wait(tfull_bar(acc), acc_phase, guard)) break;
-            tc_fence_after();
-            const int row = mb * kBM + r_in_tile;
-            const int n0 = nb * BN;
-            io.row0 = mb * kBM + q * 32;
-            Epi epi(ep, g, row, n0);
             const uint32_t t_row = tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
                                    static_cast<uint32_t>(acc * BN);
-#pragma unroll 1
-            for (int c = 0; c < BN / 32; ++c) {
-                float v[32];
-                tmem_ld_32x32b_x32(t_row + c * 32, v);
-                epi.chunk(ep, v, n0 + c * 32, c * 32, io);
-            }
-            epi.finish(ep, nb);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(tempty_bar(acc));
+            const bool ok = epilogue_tile<BN, Epi>(
+                ep, g, mb * kBM + q * 32, nb, (warp - 2) / 4, t_row, io,
+                [&] {
+                    if (!mbar_wait(tfull_bar(acc), acc_phase, guard)) return false;
+                    tc_fence_after();
+                    return true;
+                },
+                [&] {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(tempty_bar(acc));
+                });
+            if (!ok) break;
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
         if (lane == 0) bulk_wait_group_all();  // stores done before shared memory goes away

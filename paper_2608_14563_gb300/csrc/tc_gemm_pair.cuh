@@ -26,8 +26,8 @@
 //                       on the LEADER's (rank 0) full barrier
 //   leader, warp 1      issues the pair MMAs and commits to the empty /
 //                       accumulator-ready barriers of BOTH CTAs (multicast)
-//   both CTAs, warps 2-5  epilogue on the CTA's 128 rows; arrive on the
-//                       leader's accumulator-empty barrier (8 arrivals)
+//   both CTAs, warps 2-   epilogue on the CTA's 128 rows (Epi::kWarps warps); arrive
+//                       on the leader's accumulator-empty barrier
 // TMEM (512 columns) is allocated collectively by warp 1 of both CTAs.
 //
 // BN is 256 (two accumulator buffers of 256 columns: the epilogue of one tile
@@ -218,7 +218,7 @@ __device__ __forceinline__ void pair_drain_copies(uint32_t bar0, long long n_sel
 }
 
 template <int BN, bool A_MN, bool B_MN, int STAGES, int MAXG, class Epi>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<Epi>(), 1)
     tc_gemm_pair_kernel(const __grid_constant__ GemmMaps<MAXG> maps,
                         const __grid_constant__ typename Epi::Params ep, const GemmShape sh_in,
                         unsigned int* status, unsigned long long wait_limit_ns) {
@@ -279,7 +279,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(tfull_bar(a), 1);
-            mbar_init(tempty_bar(a), 8);  // leader's: 4 epilogue warps x 2 CTAs
+            mbar_init(tempty_bar(a), 2 * Epi::kWarps);  // leader's: the epilogue warps of both CTAs
         }
         mbar_init(drain_bar, 1);
         *abort_flag = 0;
@@ -391,47 +391,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
     } else {
         // ------------------------------------------------------- epilogue (both CTAs)
         const int q = warp & 3;
-        const int r_in_tile = 128 * static_cast<int>(rank) + q * 32 + lane;
-        EpiIO io{sbase + L::kOutOffset + static_cast<uint32_t>((warp - 2) * kOutBytesPerWarp), lane,
-                 0, 0u};
+        const int half = (warp - 2) / 4;  // with 8 epilogue warps: the warp's columns
+        constexpr int kOutPerWarp = 4 * kOutBytesPerWarp / Epi::kWarps;
+        constexpr int kPartCols = BN / (Epi::kWarps / 4);
+        EpiIO io{sbase + L::kOutOffset + static_cast<uint32_t>((warp - 2) * kOutPerWarp), lane, 0,
+                 0u};
         int acc = 0;
         uint32_t acc_phase = 0;
-        SegCursor seg(sh, cluster, n_clusters);
-        long long t;
-        int kb0, kb1, part, slot;
-        while (seg.next(sh, t, kb0, kb1, part, slot)) {
-            int g, mp, nb;
-            tile_coords(t, sh, g, mp, nb);
-            if (!mbar_wait_cl(tfull_bar(acc), acc_phase, guard)) break;
+        auto ready = [&] {
+            if (!mbar_wait_cl(tfull_bar(acc), acc_phase, guard)) return false;
             tc_fence_after();
-            const uint32_t t_row = tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
-                                   static_cast<uint32_t>(acc * BN);
-            if (part < 0) {
-                const int tile_row0 = mp * kPairBM;
-                const int row = tile_row0 + r_in_tile;
-                const int n0 = nb * BN;
-                io.row0 = tile_row0 + 128 * static_cast<int>(rank) + q * 32;
-                Epi epi(ep, g, row, n0);
-#pragma unroll 1
-                for (int c = 0; c < BN / 32; ++c) {
-                    float v[32];
-                    tmem_ld_32x32b_x32(t_row + c * 32, v);
-                    epi.chunk(ep, v, n0 + c * 32, c * 32, io);
-                }
-                epi.finish(ep, nb);
-            } else {
-                // one k range of a split tile: its raw fp32 sums, row r_in_tile, to its slot
-                float* dst = sh.sk_scratch + (static_cast<size_t>(slot) * kPairBM + r_in_tile) * BN;
-#pragma unroll 1
-                for (int c = 0; c < BN / 32; ++c) {
-                    float v[32];
-                    tmem_ld_32x32b_x32(t_row + c * 32, v);
-                    float4* d4 = reinterpret_cast<float4*>(dst + c * 32);
-#pragma unroll
-                    for (int q4 = 0; q4 < 8; ++q4)
-                        d4[q4] = make_float4(v[4 * q4], v[4 * q4 + 1], v[4 * q4 + 2], v[4 * q4 + 3]);
-                }
-            }
+            return true;
+        };
+        auto release = [&] {
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {
@@ -439,6 +411,35 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
                     mbar_arrive(tempty_bar(acc));
                 else
                     mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));
+            }
+        };
+        SegCursor seg(sh, cluster, n_clusters);
+        long long t;
+        int kb0, kb1, part, slot;
+        while (seg.next(sh, t, kb0, kb1, part, slot)) {
+            int g, mp, nb;
+            tile_coords(t, sh, g, mp, nb);
+            const uint32_t t_row = tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
+                                   static_cast<uint32_t>(acc * BN);
+            const int r0 = 128 * static_cast<int>(rank) + q * 32;  // first row in the tile
+            if (part < 0) {
+                if (!epilogue_tile<BN, Epi>(ep, g, mp * kPairBM + r0, nb, half, t_row, io, ready,
+                                            release))
+                    break;
+            } else {
+                // one k range of a split tile: its raw fp32 sums, row r0 + lane, to its slot
+                if (!ready()) break;
+                float* dst = sh.sk_scratch + (static_cast<size_t>(slot) * kPairBM + r0 + lane) * BN;
+#pragma unroll 1
+                for (int c = half * (kPartCols / 32); c < (half + 1) * (kPartCols / 32); ++c) {
+                    float v[32];
+                    tmem_ld_32x32b_x32(t_row + c * 32, v);
+                    float4* d4 = reinterpret_cast<float4*>(dst + c * 32);
+#pragma unroll
+                    for (int q4 = 0; q4 < 8; ++q4)
+                        d4[q4] = make_float4(v[4 * q4], v[4 * q4 + 1], v[4 * q4 + 2], v[4 * q4 + 3]);
+                }
+                release();
             }
             if (++acc == kAccBufs) { acc = 0; acc_phase ^= 1u; }
         }
