@@ -13,7 +13,7 @@
 // (Epi::kWarps) and the form of epilogue_tile's second half: a chunk is staged in shared
 // memory and each lane takes 4 columns of 8 rows, so that every global access of a warp
 // covers whole row segments, and the operands of the next chunk (of the first chunk:
-// while the mainloop runs) are loaded as soon as their registers are free.  One row per
+// while the mainloop runs) are loaded ahead.  One row per
 // thread, as these epilogues had it with 4 warps, made every 16-byte access of a warp
 // touch 32 rows and kept 16 KB in flight per SM: AdamW with the step clip at T 4096,
 // d 4096, d_ff 11008, 8 layers took 4154 us in the GEMM for 1.5 ms of tensor work.
@@ -521,32 +521,49 @@ struct EpiProjVjp {
     __device__ __forceinline__ void finish(const Params&, int) {}
 };
 
-// A lane's place in a warp's 32 rows of an 8-warp epilogue: its columns 4 (lane mod 8) ..
-// of the rows lane / 8, lane / 8 + 4, ... (8 of them), as element offsets into matrices
-// of row stride ld.
+// A lane's place in a warp's 32 rows of an 8-warp epilogue: its columns
+// 4 (lane mod kLanes) .. of every kRows-th row from lane / kLanes, as element offsets into
+// matrices of row stride ld.
 struct QuadPos {
+    using Q = QuadChunk;
     long long off;    // of the lane's first element
     int rows, cols;   // rows from its first row, columns from its first column, in the matrix
 
     __device__ __forceinline__ QuadPos(int M, int N, long long ld, int row0, int n0, int lane) {
-        const int r = row0 + (lane >> 3), c = n0 + 4 * (lane & 7);
+        const int r = row0 + lane / Q::kLanes, c = n0 + 4 * (lane % Q::kLanes);
         off = r * ld + c;
         rows = M - r;
         cols = N - c;
     }
-    // Row i of the lane (4 i rows below its first) and column offset co are inside
+    // Quad i of the lane (kRows i rows below its first) and column offset co are inside
     // (N is a multiple of 8, so the 4 columns are inside together).
-    __device__ __forceinline__ bool in(int i, int co) const { return 4 * i < rows && co < cols; }
+    __device__ __forceinline__ bool in(int i, int co) const { return Q::kRows * i < rows && co < cols; }
+    __device__ __forceinline__ long long at(long long ld, int i, int co) const {
+        return off + Q::kRows * i * ld + co;
+    }
+    // That element of a matrix m, or m itself outside the matrix: always readable, so that
+    // a batch of loads has no branches between them.
+    template <typename TT>
+    __device__ __forceinline__ const TT* src(const TT* m, long long ld, int i, int co) const {
+        return in(i, co) ? m + at(ld, i, co) : m;
+    }
 };
 
+// The operands of a chunk are loaded as one batch when the chunk before is done, with
+// nothing that waits between its loads: loads issued one by one between the uses of the
+// batch before shared the warp's few scoreboards with it, and each use waited for the
+// newest load (the update of T 512, d 2048, d_ff 8264, 4 layers: 278 us, 230 of them with
+// the loads alone, 115 without; 200 us with batches.  Two batches in flight gave nothing
+// more, nor did 16 warps, L2 prefetches of the next tile or streaming cache hints).
+
 // Slots of per-warp partial sums per (256-row block, 256-column tile): 8 blocks of 32 rows
-// times the two column halves of the 8-warp epilogues.
+// times the two column halves.
 constexpr int kColSlots = 16;
 
 __device__ __forceinline__ long long quad_slot(int g, int m256, int n_blocks, int nb, int row0,
                                                int n0) {
     return ((static_cast<long long>(g) * m256 + row0 / 256) * n_blocks + nb) * kColSlots +
-           ((n0 & 128) >> 4) + (row0 % 256) / 32;
+           ((n0 % 256) / QuadChunk::kTileCols) * 8 + (row0 % 256) / 32;
 }
 
 __device__ __forceinline__ float warp_sum_f32(float x) {
@@ -569,30 +586,33 @@ struct EpiUpdate {
         int M, N;
         float neg_lr;
     };
+    using Q = QuadChunk;
     QuadPos pos;
     float* wm;
     __nv_bfloat16* wo;
     __nv_bfloat16* go;
-    float4 w[8];  // master values of the chunk that chunk() works on next
+    float4 w[Q::kQuads];  // master values of the next chunk
+
+    __device__ __forceinline__ void load(const Params& p, int co) {
+        if (!wm) return;
+#pragma unroll
+        for (int i = 0; i < Q::kQuads; ++i)
+            w[i] = *reinterpret_cast<const float4*>(pos.src(wm, p.ld, i, co));
+    }
 
     __device__ __forceinline__ EpiUpdate(const Params& p, int g, int row0, int n0, int lane)
         : pos(p.M, p.N, p.ld, row0, n0, lane) {
         wm = p.W_master[g];
         wo = p.W_out[g];
         go = p.G_out[g];
-        if (wm) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if (pos.in(i, 0)) w[i] = *reinterpret_cast<const float4*>(wm + pos.off + 4 * i * p.ld);
-        }
+        load(p, 0);
     }
 
-    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co,
-                                          bool more) {
+    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float4 v = out_read_quad(buf, lane, i);
-            const long long o = pos.off + 4 * i * p.ld + co;
+        for (int i = 0; i < Q::kQuads; ++i) {
+            const float4 v = Q::read(buf, lane, i);
+            const long long o = pos.at(p.ld, i, co);
             const bool in = pos.in(i, co);
             if (wm) {
                 float4 a = w[i];
@@ -606,12 +626,12 @@ struct EpiUpdate {
                         *reinterpret_cast<uint2*>(wo + o) =
                             make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
                 }
-                if (more && pos.in(i, co + 32)) w[i] = *reinterpret_cast<const float4*>(wm + o + 32);
             }
             if (go && in)
                 *reinterpret_cast<uint2*>(go + o) =
                     make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
         }
+        if (co + Q::kCols < Q::kTileCols) load(p, co + Q::kCols);
     }
 
     __device__ __forceinline__ void finish(const Params&, int, int) {}
@@ -633,35 +653,34 @@ struct EpiGradCos {
         int M, N;
         int m256, n_blocks;
     };
+    using Q = QuadChunk;
     QuadPos pos;
     int g, row0, n0;
     float2 s_gy, s_gg, s_yy;
-    uint2 y[8];  // Y of the chunk that chunk() works on next
+    uint2 y[Q::kQuads];  // Y of the next chunk
 
-    __device__ __forceinline__ uint2 load(const Params& p, int i, int co) const {
-        return pos.in(i, co) ? __ldg(reinterpret_cast<const uint2*>(p.Y[g] + pos.off + 4 * i * p.ld + co))
-                             : make_uint2(0, 0);
+    __device__ __forceinline__ void load(const Params& p, int co) {
+#pragma unroll
+        for (int i = 0; i < Q::kQuads; ++i)
+            y[i] = __ldg(reinterpret_cast<const uint2*>(pos.src(p.Y[g], p.ld, i, co)));
     }
 
     __device__ __forceinline__ EpiGradCos(const Params& p, int g_, int row0_, int n0_, int lane)
         : pos(p.M, p.N, p.ld, row0_, n0_, lane), g(g_), row0(row0_), n0(n0_) {
         s_gy = s_gg = s_yy = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) y[i] = load(p, i, 0);
+        load(p, 0);
     }
 
-    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co,
-                                          bool more) {
+    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float4 v = out_read_quad(buf, lane, i);
+        for (int i = 0; i < Q::kQuads; ++i) {
+            const float4 v = Q::read(buf, lane, i);
             const uint32_t pk[2] = {pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w)};
-            // outside the matrix G is 0 (zero-filled operands) and Y was loaded as 0
-            const uint32_t yk[2] = {y[i].x, y[i].y};
-            if (pos.in(i, co))
-                *reinterpret_cast<uint2*>(p.G_out[g] + pos.off + 4 * i * p.ld + co) =
-                    make_uint2(pk[0], pk[1]);
-            if (more) y[i] = load(p, i, co + 32);
+            if (!pos.in(i, co)) continue;
+            const uint2 yv = y[i];
+            const uint32_t yk[2] = {yv.x, yv.y};
+            *reinterpret_cast<uint2*>(p.G_out[g] + pos.at(p.ld, i, co)) =
+                make_uint2(pk[0], pk[1]);
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 const float2 gr = make_float2(__uint_as_float(pk[k] << 16),
@@ -673,6 +692,7 @@ struct EpiGradCos {
                 s_yy = __ffma2_rn(yr, yr, s_yy);
             }
         }
+        if (co + Q::kCols < Q::kTileCols) load(p, co + Q::kCols);
     }
 
     __device__ __forceinline__ void finish(const Params& p, int nb, int lane) {
@@ -697,17 +717,18 @@ struct EpiStoreGroupF32 {
         long long ld;
         int M, N;
     };
+    using Q = QuadChunk;
     QuadPos pos;
     float* G;
 
     __device__ __forceinline__ EpiStoreGroupF32(const Params& p, int g, int row0, int n0, int lane)
         : pos(p.M, p.N, p.ld, row0, n0, lane), G(p.G[g]) {}
 
-    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co, bool) {
+    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float4 v = out_read_quad(buf, lane, i);
-            if (pos.in(i, co)) *reinterpret_cast<float4*>(G + pos.off + 4 * i * p.ld + co) = v;
+        for (int i = 0; i < Q::kQuads; ++i) {
+            const float4 v = Q::read(buf, lane, i);
+            if (pos.in(i, co)) *reinterpret_cast<float4*>(G + pos.at(p.ld, i, co)) = v;
         }
     }
 
@@ -725,7 +746,9 @@ struct EpiStoreGroupF32 {
 // is the pre-step one).  Without a clip the stand-alone passes are used: taking the whole
 // step here made the update faster but the power-capped step slower (its epilogue then
 // held the tensor pipe back at full draw).
-// The operands of 4 of the chunk's 8 row quads are in flight at a time (48 registers).
+// The operands of the next 4 quads are loaded as each quad is done: its arithmetic hides
+// the wait that the batches of the other epilogues avoid (2362 us; batches of a whole or
+// half a chunk 3006 and 2500, 2 quads ahead 2561, 8 ahead 2840, 16 warps 2990).
 struct EpiOptStep {
     static constexpr int kWarps = 8;
     struct Params {
@@ -739,6 +762,7 @@ struct EpiOptStep {
         int M, N;
         int m256, n_blocks;
     };
+    using Q = QuadChunk;
     static constexpr int kAhead = 4;
     QuadPos pos;
     int g, row0, n0;
@@ -747,12 +771,12 @@ struct EpiOptStep {
     float* p2;
     float* D;
     float s_ww, s_dd;
-    float4 w[kAhead], a[kAhead], b[kAhead];  // of the next kAhead row quads
+    float4 w[kAhead], a[kAhead], b[kAhead];  // of the next kAhead quads
 
     __device__ __forceinline__ void load(const Params& p, int k, int i, int co) {
         w[k] = a[k] = b[k] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (!pos.in(i, co)) return;
-        const long long o = pos.off + 4 * i * p.ld + co;
+        const long long o = pos.at(p.ld, i, co);
         w[k] = *reinterpret_cast<const float4*>(wm + o);
         if (p1) a[k] = *reinterpret_cast<const float4*>(p1 + o);
         if (p2) b[k] = *reinterpret_cast<const float4*>(p2 + o);
@@ -768,14 +792,13 @@ struct EpiOptStep {
         for (int k = 0; k < kAhead; ++k) load(p, k, k, 0);
     }
 
-    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co,
-                                          bool more) {
+    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co) {
 #pragma unroll 1
-        for (int h = 0; h < 8; h += kAhead) {
+        for (int h = 0; h < Q::kQuads; h += kAhead) {
 #pragma unroll
             for (int k = 0; k < kAhead; ++k) {
                 const int i = h + k;
-                const float4 v4 = out_read_quad(buf, lane, i);
+                const float4 v4 = Q::read(buf, lane, i);
                 const float v[4] = {v4.x, v4.y, v4.z, v4.w};
                 const float wv[4] = {w[k].x, w[k].y, w[k].z, w[k].w};
                 float av[4] = {a[k].x, a[k].y, a[k].z, a[k].w};
@@ -791,15 +814,15 @@ struct EpiOptStep {
                     }
                 }
                 if (in) {
-                    const long long o = pos.off + 4 * i * p.ld + co;
+                    const long long o = pos.at(p.ld, i, co);
                     *reinterpret_cast<float4*>(D + o) = make_float4(out[0], out[1], out[2], out[3]);
                     if (p1) *reinterpret_cast<float4*>(p1 + o) = make_float4(av[0], av[1], av[2], av[3]);
                     if (p2) *reinterpret_cast<float4*>(p2 + o) = make_float4(bv[0], bv[1], bv[2], bv[3]);
                 }
-                if (h == 0)
+                if (i + kAhead < Q::kQuads)
                     load(p, k, i + kAhead, co);
-                else if (more)
-                    load(p, k, i - kAhead, co + 32);
+                else if (co + Q::kCols < Q::kTileCols)
+                    load(p, k, i + kAhead - Q::kQuads, co + Q::kCols);
             }
         }
     }
@@ -828,34 +851,33 @@ struct EpiSwiglu {
         long long ld;
         int M, N;
     };
+    using Q = QuadChunk;
     QuadPos pos;
-    uint2 ua[8], ub[8];  // a and b of the chunk that chunk() works on next
+    uint2 ua[Q::kQuads], ub[Q::kQuads];  // a and b of the next chunk
 
-    __device__ __forceinline__ void load(const Params& p, int i, int co) {
-        ua[i] = ub[i] = make_uint2(0, 0);
-        if (!pos.in(i, co)) return;
-        const long long o = pos.off + 4 * i * p.ld + co;
-        ua[i] = *reinterpret_cast<const uint2*>(p.a + o);
-        ub[i] = *reinterpret_cast<const uint2*>(p.b + o);
+    __device__ __forceinline__ void load(const Params& p, int co) {
+#pragma unroll
+        for (int i = 0; i < Q::kQuads; ++i) {
+            ua[i] = *reinterpret_cast<const uint2*>(pos.src(p.a, p.ld, i, co));
+            ub[i] = *reinterpret_cast<const uint2*>(pos.src(p.b, p.ld, i, co));
+        }
     }
 
     __device__ __forceinline__ EpiSwiglu(const Params& p, int, int row0, int n0, int lane)
         : pos(p.M, p.N, p.ld, row0, n0, lane) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) load(p, i, 0);
+        load(p, 0);
     }
 
-    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co,
-                                          bool more) {
+    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float4 v4 = out_read_quad(buf, lane, i);
+        for (int i = 0; i < Q::kQuads; ++i) {
+            const float4 v4 = Q::read(buf, lane, i);
             const float v[4] = {v4.x, v4.y, v4.z, v4.w};
-            const float xa[4] = {__uint_as_float(ua[i].x << 16), __uint_as_float(ua[i].x & 0xffff0000u),
-                                 __uint_as_float(ua[i].y << 16), __uint_as_float(ua[i].y & 0xffff0000u)};
-            const float xb[4] = {__uint_as_float(ub[i].x << 16), __uint_as_float(ub[i].x & 0xffff0000u),
-                                 __uint_as_float(ub[i].y << 16), __uint_as_float(ub[i].y & 0xffff0000u)};
-            if (more) load(p, i, co + 32);
+            const uint2 a2 = ua[i], b2 = ub[i];
+            const float xa[4] = {__uint_as_float(a2.x << 16), __uint_as_float(a2.x & 0xffff0000u),
+                                 __uint_as_float(a2.y << 16), __uint_as_float(a2.y & 0xffff0000u)};
+            const float xb[4] = {__uint_as_float(b2.x << 16), __uint_as_float(b2.x & 0xffff0000u),
+                                 __uint_as_float(b2.y << 16), __uint_as_float(b2.y & 0xffff0000u)};
             float da[4], db[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -868,13 +890,14 @@ struct EpiSwiglu {
                 db[k] = v[k] * x * sg;
             }
             if (pos.in(i, co)) {
-                const long long o = pos.off + 4 * i * p.ld + co;
+                const long long o = pos.at(p.ld, i, co);
                 *reinterpret_cast<uint2*>(p.dA + o) =
                     make_uint2(pack_bf16x2(da[0], da[1]), pack_bf16x2(da[2], da[3]));
                 *reinterpret_cast<uint2*>(p.dB + o) =
                     make_uint2(pack_bf16x2(db[0], db[1]), pack_bf16x2(db[2], db[3]));
             }
         }
+        if (co + Q::kCols < Q::kTileCols) load(p, co + Q::kCols);
     }
 
     __device__ __forceinline__ void finish(const Params&, int, int) {}

@@ -149,33 +149,33 @@ __device__ __forceinline__ void out_stage_row(uint32_t buf, int r, const uint32_
                      w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
 }
 
-// Write 16 words (64 bytes) of row r into half `h` (pieces 4h..4h+3) of a
-// staging buffer, same swizzle as out_stage_row.
-__device__ __forceinline__ void out_stage_half(uint32_t buf, int r, int h, const uint32_t (&w)[16]) {
-    const uint32_t row = buf + static_cast<uint32_t>(r) * 128u;
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-        st_shared_v4(row + (((static_cast<uint32_t>(4 * h + c)) ^ (static_cast<uint32_t>(r) & 7u)) << 4),
-                     w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
-}
+// Chunks of the 8-warp epilogues: 32 rows x 32 fp32 columns, staged in the warp's 4 KB of
+// output staging with one row per lane and read back with 8 lanes to a row, 4 columns each,
+// so that a warp's global accesses cover whole row segments.  16-byte pieces are swizzled
+// (out_stage_row), so neither side has bank conflicts.
+struct QuadChunk {
+    static constexpr int kCols = 32;
+    static constexpr int kLanes = 8;        // lanes sharing a row
+    static constexpr int kRows = 4;         // rows of one access of the warp
+    static constexpr int kQuads = 8;        // accesses per chunk
+    static constexpr int kTileCols = 128;   // of a 256-column tile, per warp
 
-// A 32 x 32 fp32 chunk staged by out_stage_row, read back with 8 lanes to a row: the 4
-// columns 4 (lane mod 8) .. of row 4 i + lane / 8 (i in [0, 8)), so that a warp's global
-// accesses cover whole 128-byte row segments.
-__device__ __forceinline__ float4 out_read_quad(uint32_t buf, int lane, int i) {
-    const uint32_t r = 4u * static_cast<uint32_t>(i) + static_cast<uint32_t>(lane >> 3);
-    return ld_shared_f4(buf + r * 128u + ((static_cast<uint32_t>(lane & 7) ^ (r & 7u)) << 4));
-}
+    // Columns 4 (lane mod kLanes) .. of row kRows i + lane / kLanes, i in [0, kQuads).
+    static __device__ __forceinline__ float4 read(uint32_t buf, int lane, int i) {
+        const uint32_t r = static_cast<uint32_t>(kRows * i + lane / kLanes);
+        return ld_shared_f4(buf + r * 128u + ((static_cast<uint32_t>(lane % kLanes) ^ (r & 7u)) << 4));
+    }
+};
 
 // The epilogue's warps.  With Epi::kWarps = 4 each warp owns 32 rows of the CTA's 128 and
 // walks all BN columns, one row per thread (Epi(params, group, row, n0); chunk(params,
 // v[32], column, offset in the tile, io); finish(params, n_block)).  With 8, two warps
-// share the rows and take half of the columns each, and every 32 x 32 chunk goes through
-// the warp's staging buffer (Epi(params, group, first row, first column, lane);
-// chunk(params, staged chunk, lane, offset, another chunk follows); finish(params,
-// n_block, lane)).  The functor is made before the accumulator is awaited, so that what
-// its constructor loads arrives during the mainloop.  `ready` waits for the accumulator
-// (false: give up), `release` gives it back once its last columns are in registers.
+// share the rows and take half of the columns each, and every chunk goes through the warp's
+// staging buffer (QuadChunk; Epi(params, group, first row, first column, lane);
+// chunk(params, staged chunk, lane, offset); finish(params, n_block, lane)).  The functor
+// is made before the accumulator is awaited, so that what its constructor loads arrives
+// during the mainloop.  `ready` waits for the accumulator (false: give up), `release`
+// gives it back once its last columns are in registers.
 template <int BN, class Epi, class Ready, class Release>
 __device__ __forceinline__ bool epilogue_tile(const typename Epi::Params& ep, int g, int row0,
                                               int nb, int warp_half, uint32_t t_row, EpiIO& io,
@@ -194,20 +194,23 @@ __device__ __forceinline__ bool epilogue_tile(const typename Epi::Params& ep, in
         }
         epi.finish(ep, nb);
     } else {
-        constexpr int kCols = BN / 2;
-        Epi epi(ep, g, row0, nb * BN + warp_half * kCols, io.lane);
+        using Q = QuadChunk;
+        static_assert(BN == 256, "the 8-warp epilogues split 256 columns");
+        const int c0 = warp_half * Q::kTileCols;
+        Epi epi(ep, g, row0, nb * BN + c0, io.lane);
         if (!ready()) return false;
+        constexpr int kChunks = Q::kTileCols / Q::kCols;
 #pragma unroll 1
-        for (int c = 0; c < kCols / 32; ++c) {
+        for (int c = 0; c < kChunks; ++c) {
             float v[32];
-            tmem_ld_32x32b_x32(t_row + warp_half * kCols + c * 32, v);
-            if (c == kCols / 32 - 1) release();
+            tmem_ld_32x32b_x32(t_row + c0 + c * Q::kCols, v);
+            if (c == kChunks - 1) release();
             uint32_t w[32];
 #pragma unroll
             for (int j = 0; j < 32; ++j) w[j] = __float_as_uint(v[j]);
             out_stage_row(io.out, io.lane, w);
             __syncwarp();
-            epi.chunk(ep, io.out, io.lane, c * 32, c + 1 < kCols / 32);
+            epi.chunk(ep, io.out, io.lane, c * Q::kCols);
             __syncwarp();
         }
         epi.finish(ep, nb, io.lane);
