@@ -709,38 +709,74 @@ struct EpiGradCos {
 
 // ---------------------------------------------------------------------------
 // Pseudogradient only, fp32, one output per group (layer): G[g] = g~^T A_l, for
-// the optimizers that need the whole G (and its norm) before they step.
+// the optimizers that need the whole G before they step.  With W_master set (the relative
+// clip on the gradient) also ||W||^2 and ||G||^2 of the warp's 32 rows x 128 columns, one
+// pair per quad_slot, so that the clip factor needs no pass over W and G of its own
+// (448 us of 1823 for 3 layers of 3072 x 23040).
 struct EpiStoreGroupF32 {
     static constexpr int kWarps = 8;
     struct Params {
         float* G[kMaxGroups];
+        const float* W_master[kMaxGroups];  // or null: no norms
+        float* part;                        // [groups][m256][n_blocks][kColSlots][2]
         long long ld;
         int M, N;
+        int m256, n_blocks;
     };
     using Q = QuadChunk;
     QuadPos pos;
+    int g, row0, n0;
     float* G;
+    const float* wm;
+    float s_ww, s_gg;
+    float4 w[Q::kQuads];  // master values of the next chunk
 
-    __device__ __forceinline__ EpiStoreGroupF32(const Params& p, int g, int row0, int n0, int lane)
-        : pos(p.M, p.N, p.ld, row0, n0, lane), G(p.G[g]) {}
+    __device__ __forceinline__ void load(const Params& p, int co) {
+        if (!wm) return;
+#pragma unroll
+        for (int i = 0; i < Q::kQuads; ++i)
+            w[i] = *reinterpret_cast<const float4*>(pos.src(wm, p.ld, i, co));
+    }
+
+    __device__ __forceinline__ EpiStoreGroupF32(const Params& p, int g_, int row0_, int n0_,
+                                                int lane)
+        : pos(p.M, p.N, p.ld, row0_, n0_, lane), g(g_), row0(row0_), n0(n0_), G(p.G[g_]),
+          wm(p.W_master[g_]), s_ww(0.f), s_gg(0.f) {
+        load(p, 0);
+    }
 
     __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co) {
 #pragma unroll
         for (int i = 0; i < Q::kQuads; ++i) {
             const float4 v = Q::read(buf, lane, i);
-            if (pos.in(i, co)) *reinterpret_cast<float4*>(G + pos.at(p.ld, i, co)) = v;
+            if (!pos.in(i, co)) continue;
+            *reinterpret_cast<float4*>(G + pos.at(p.ld, i, co)) = v;
+            if (wm) {
+                s_gg = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, s_gg))));
+                s_ww = fmaf(w[i].x, w[i].x,
+                            fmaf(w[i].y, w[i].y, fmaf(w[i].z, w[i].z, fmaf(w[i].w, w[i].w, s_ww))));
+            }
         }
+        if (co + Q::kCols < Q::kTileCols) load(p, co + Q::kCols);
     }
 
-    __device__ __forceinline__ void finish(const Params&, int, int) {}
+    __device__ __forceinline__ void finish(const Params& p, int nb, int lane) {
+        if (!wm) return;
+        const float ww = warp_sum_f32(s_ww), gg = warp_sum_f32(s_gg);
+        if (lane == 0) {
+            float* o = p.part + quad_slot(g, p.m256, p.n_blocks, nb, row0, n0) * 2;
+            o[0] = ww;
+            o[1] = gg;
+        }
+    }
 };
 
 // ---------------------------------------------------------------------------
 // The optimizer's first pass in the pseudogradient GEMM's epilogue, for the relative
 // clip on the step (Sec. 3.1: SGD, SGD with momentum, AdamW on the fp32 masters; App. A:
 // ||dW|| <= clip_frac ||W||).  With G from the accumulator, each element's optimizer state
-// advances and its unclipped step d = opt_step(G, W, s1, s2) is stored (fp32, D[g]; the
-// state sees the unclipped gradient), and ||W||^2, ||d||^2 of the warp's 32 rows x 128
+// advances and its unclipped step d = opt_step(G, W, s1, s2) is stored (fp32, D[g], null
+// for momentum, whose step -lr s1 the state holds; the state sees the unclipped gradient), and ||W||^2, ||d||^2 of the warp's 32 rows x 128
 // columns are written as one pair per quad_slot; a kernel then scales each layer's steps
 // by min(1, clip_frac ||W|| / ||d||) and applies them (W is not written here, so its norm
 // is the pre-step one).  Without a clip the stand-alone passes are used: taking the whole
@@ -755,7 +791,7 @@ struct EpiOptStep {
         const float* W_master[kMaxGroups];
         float* s1[kMaxGroups];             // momentum / AdamW first moment (or null)
         float* s2[kMaxGroups];             // AdamW second moment (or null)
-        float* D[kMaxGroups];              // the unclipped steps
+        float* D[kMaxGroups];              // the unclipped steps (not for momentum: -lr s1)
         float* part;                       // [groups][m256][n_blocks][kColSlots][2]
         OptimParams op;
         long long ld;
@@ -815,7 +851,9 @@ struct EpiOptStep {
                 }
                 if (in) {
                     const long long o = pos.at(p.ld, i, co);
-                    *reinterpret_cast<float4*>(D + o) = make_float4(out[0], out[1], out[2], out[3]);
+                    if (D)
+                        *reinterpret_cast<float4*>(D + o) =
+                            make_float4(out[0], out[1], out[2], out[3]);
                     if (p1) *reinterpret_cast<float4*>(p1 + o) = make_float4(av[0], av[1], av[2], av[3]);
                     if (p2) *reinterpret_cast<float4*>(p2 + o) = make_float4(bv[0], bv[1], bv[2], bv[3]);
                 }

@@ -598,28 +598,37 @@ int32_t fpo_layer_optimize_grouped(int32_t n_layers, int64_t T, int64_t d, int64
     float* const* s1 = opt->kind != FPO_OPT_SGD ? state1 : nullptr;
     float* const* s2 = opt->kind == FPO_OPT_ADAMW ? state2 : nullptr;
 
+    // norms summed in the GEMM's epilogue (bf16 with a clip)
+    float* part = reinterpret_cast<float*>(partials);
+    const int slots = static_cast<int>(
+        opt_step_partial_bytes(1, static_cast<int>(d), static_cast<int>(d_ff)) / (2 * sizeof(float)));
     if (dtype == FPO_BF16 && T > 0 && opt->clip == FPO_CLIP_STEP) {
         // the step clip's first pass in the GEMM's epilogue: the state advanced, the
         // unclipped steps (in the G buffer) and their norm partials; then a scale and an
         // apply pass (measured: the AdamW + step-clip step 0.6% faster than with G stored
         // and three passes; without a clip the stand-alone passes are faster overall)
-        float* part = reinterpret_cast<float*>(partials);
+        const bool momentum = op.kind == FPO_OPT_SGD_MOMENTUM;  // its step is -lr s1
         FPO_TRY(launch_opt_step_bf16(n_layers, static_cast<int>(T), static_cast<int>(d),
-                                     static_cast<int>(d_ff), g, A, op, W_master, s1, s2, G, part,
-                                     status, st));
-        const int slots = static_cast<int>(opt_step_partial_bytes(1, static_cast<int>(d),
-                                                                  static_cast<int>(d_ff)) /
-                                           (2 * sizeof(float)));
-        return cuda_status(launch_opt_step_clip(n_layers, n, op, part, slots, G, W_master, W_out,
-                                                scales, st));
+                                     static_cast<int>(d_ff), g, A, op, W_master, s1, s2,
+                                     momentum ? nullptr : G, part, status, st));
+        FPO_TRY(launch_opt_scale(n_layers, op, part, slots, scales, st));
+        return cuda_status(launch_opt_step_apply(n_layers, n, op, G, momentum ? s1 : nullptr,
+                                                 W_master, W_out, scales, st));
     }
 
     // 1. G_l = g_l^T A_l (fp32)
+    bool norms_done = false;
     if (T == 0) {
         FPO_TRY(cudaMemsetAsync(Gbuf, 0, n_layers * n * 4, st));
     } else if (dtype == FPO_BF16) {
+        const bool norms = opt->clip == FPO_CLIP_GRADIENT;
         FPO_TRY(launch_grad_bf16(n_layers, static_cast<int>(T), static_cast<int>(d),
-                                 static_cast<int>(d_ff), g, A, G, status, st));
+                                 static_cast<int>(d_ff), g, A, G, norms ? W_master : nullptr, part,
+                                 status, st));
+        if (norms) {
+            FPO_TRY(launch_opt_scale(n_layers, op, part, slots, scales, st));
+            norms_done = true;
+        }
     } else {
         FPO_TRY(launch_update_f32(n_layers, static_cast<int>(T), static_cast<int>(d),
                                   static_cast<int>(d_ff), reinterpret_cast<const float* const*>(g),
@@ -628,7 +637,7 @@ int32_t fpo_layer_optimize_grouped(int32_t n_layers, int64_t T, int64_t d, int64
     }
     // 2. clip factor and optimizer step on the fp32 masters
     return cuda_status(launch_optimizer(dtype, n_layers, n, op, G, W_master, W_out, s1, s2,
-                                        partials, scales, st));
+                                        partials, scales, norms_done, st));
 }
 
 int32_t fpo_gate_up_signals(int64_t T, int64_t d, int64_t d_ff, int32_t dtype, const void* g,

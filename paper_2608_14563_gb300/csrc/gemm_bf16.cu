@@ -683,7 +683,8 @@ cudaError_t launch_update_bf16(int n, int T, int d, int d_ff, const void* const*
 }
 
 cudaError_t launch_grad_bf16(int n, int T, int d, int d_ff, const void* const* g,
-                             const void* const* A, float* const* G_out, unsigned* status,
+                             const void* const* A, float* const* G_out,
+                             float* const* W_master, float* part, unsigned* status,
                              cudaStream_t st) {
     if (n < 1 || n > kMaxGroups) return cudaErrorInvalidValue;
     static GemmMaps<kMaxGroups> maps;
@@ -697,15 +698,24 @@ cudaError_t launch_grad_bf16(int n, int T, int d, int d_ff, const void* const* g
             return cudaErrorInvalidValue;
         if (!map_mnmajor(&maps.b[l], A[l], T, d_ff)) return cudaErrorInvalidValue;
         ep.G[l] = G_out[l];
+        ep.W_master[l] = W_master ? W_master[l] : nullptr;
     }
     for (int l = n; l < kMaxGroups; ++l) {
         maps.a[l] = maps.a[0];
         maps.b[l] = maps.b[0];
         ep.G[l] = G_out[0];
+        ep.W_master[l] = ep.W_master[0];
     }
+    ep.part = part;
     ep.ld = d_ff;
     ep.M = d;
     ep.N = d_ff;
+    ep.m256 = (d + 255) / 256;
+    ep.n_blocks = (d_ff + kUpdBN - 1) / kUpdBN;
+    if (W_master && !use_pair()) {  // as in launch_opt_step_bf16
+        const cudaError_t e = cudaMemsetAsync(part, 0, n * opt_step_partial_bytes(1, d, d_ff), st);
+        if (e != cudaSuccess) return e;
+    }
     if (use_pair())
         return run_gemm_pair<kUpdBN, true, true, kPairStages, kMaxGroups, EpiStoreGroupF32>(
             maps, ep, make_shape(d, d_ff, T, kUpdBN, n, band_for(true), kPairBM), status, st);
@@ -859,7 +869,8 @@ cudaError_t launch_grad_cosine_bf16(int n, int T, int d, int d_ff, const void* c
         e = run_gemm<kUpdBN, true, true, kUpdStages, kMaxGroups, EpiGradCos>(
             maps, ep, make_shape(d, d_ff, T, kUpdBN, n, band_for(false)), status, st);
     if (e != cudaSuccess) return e;
-    grad_cosine_final_kernel<<<n, kCosFinalThreads, 0, st>>>(part, ep.m256 * ep.n_blocks * kColSlots, out),
+    grad_cosine_final_kernel<<<n, kCosFinalThreads, 0, st>>>(
+        part, ep.m256 * ep.n_blocks * kColSlots, out),
         ::fpo::note_launch();
     return cudaGetLastError();
 }

@@ -103,10 +103,12 @@ cudaError_t launch_update_bf16(int n, int T, int d, int d_ff, const void* const*
                                void* const* W_out, void* const* G_out, unsigned* status,
                                cudaStream_t st);
 
-// Grouped pseudogradients only: G_out[l] (fp32 [d, d_ff]) = g[l]^T A[l].
+// Grouped pseudogradients only: G_out[l] (fp32 [d, d_ff]) = g[l]^T A[l].  With W_master (the
+// clip on the gradient) also (||W||^2, ||G||^2) per slot in part, as launch_opt_step_bf16
+// leaves its pairs, for launch_opt_scale.
 cudaError_t launch_grad_bf16(int n, int T, int d, int d_ff, const void* const* g,
-                             const void* const* A, float* const* G_out, unsigned* status,
-                             cudaStream_t st);
+                             const void* const* A, float* const* G_out, float* const* W_master,
+                             float* part, unsigned* status, cudaStream_t st);
 
 // Grouped pseudogradients with the diagnostic's cosine: G_out[l] (bf16 [d, d_ff]) =
 // g[l]^T A[l], and out[4 l ..] = <G_l, Y_l>, ||G_l||^2, ||Y_l||^2, cos_l of the stored
@@ -137,20 +139,25 @@ struct OptimParams {
 size_t optim_partials_bytes(int n_layers);
 // The step clip's first optimizer pass fused into the pseudogradient GEMM (bf16): the
 // state advanced, the unclipped steps in D and (||W||^2, ||d||^2) per (layer, 256 rows,
-// column tile, 32 rows) in part, for launch_opt_step_clip.
+// column tile half, 32 rows) in part, for launch_opt_scale and launch_opt_step_apply.  D is
+// not written for momentum (the step is -lr s1).
 cudaError_t launch_opt_step_bf16(int n, int T, int d, int d_ff, const void* const* g,
                                  const void* const* A, const OptimParams& op,
                                  float* const* W_master, float* const* s1, float* const* s2,
                                  float* const* D, float* part, unsigned* status, cudaStream_t st);
 size_t opt_step_partial_bytes(int n_layers, int d, int d_ff);
-cudaError_t launch_opt_step_clip(int n_layers, size_t n_elem, const OptimParams& op,
-                                 const float* part, int slots, float* const* D,
-                                 float* const* W_master, void* const* W_out, float* scales,
-                                 cudaStream_t st);
+// scales[l] = min(1, clip_frac ||W|| / ||x||) from the slot pairs (||W||^2, ||x||^2).
+cudaError_t launch_opt_scale(int n_layers, const OptimParams& op, const float* part, int slots,
+                             float* scales, cudaStream_t st);
+// W += scales[l] d with d = D, or -lr s1 where s1 is given; W_out = bf16(W).
+cudaError_t launch_opt_step_apply(int n_layers, size_t n_elem, const OptimParams& op,
+                                  float* const* D, float* const* s1, float* const* W_master,
+                                  void* const* W_out, const float* scales, cudaStream_t st);
+// The optimizer from G: the clip factors (norms_done: already in scales), then the step.
 cudaError_t launch_optimizer(int dtype, int n_layers, size_t n_elem, const OptimParams& op,
                              float* const* G, float* const* W_master, void* const* W_out,
                              float* const* s1, float* const* s2, double* partials, float* scales,
-                             cudaStream_t st);
+                             bool norms_done, cudaStream_t st);
 
 // Which tcgen05 GEMM kernel the launchers use: 0 = single-CTA 128 x 256 tiles,
 // 1 = CTA-pair 256 x 256 tiles.

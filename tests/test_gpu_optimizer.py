@@ -155,3 +155,40 @@ def test_adamw_step_clip_full_size(fpo):
         s = np.sum(got * step) / np.sum(step * step)                       # common factor
         assert 0.0 < s < 1.0
         assert rel_frob(got, s * step) < 2e-3
+
+
+@pytest.mark.parametrize("kind", list(KINDS))
+@pytest.mark.parametrize("clip", list(CLIPS))
+@pytest.mark.parametrize("size", [("f32", 12, 9, 28), ("bf16", 40, 256, 136), ("bf16", 33, 392, 520)])
+def test_optimizer_pass_edges(fpo, kind, clip, size):
+    """fp32 layers of a multiple of 4 elements (16-byte passes; the odd ones above take 4-byte
+    ones) and bf16 layers whose last column half, or 32-row block, is partly or wholly outside
+    the matrix (norm slots that only part of a warp, or none, adds to)."""
+    dtype, T, d, d_ff = size
+    wl = Workload("opt-edges", T=T, d=d, d_ff=d_ff, V=8, layers=3, dtype=dtype, seed=5)
+    g = synth.normal((T, d), std=1e-2, seed=5, tensor="h").to(wl.torch_dtype)
+    A = [synth.make_A(wl, l) for l in range(3)]
+    W = [synth.make_W_master(wl, l) for l in range(3)]
+    Gs = [oracle.pseudograd(synth.to_numpy_exact(g), synth.to_numpy_exact(a)) for a in A]
+    s1, s2 = _states(wl, Gs, kind, 3)
+    lr = {"sgd": 0.5, "sgdm": 0.05, "adamw": 2e-3}[kind]
+    opt = fpo.optimizer_desc(KINDS[kind], lr=lr, clip=CLIPS[clip], step=3)
+    Wm = [w.cuda() for w in W]
+    Wo = [torch.empty(w.shape, dtype=wl.torch_dtype, device="cuda") for w in W]
+    S1 = [torch.from_numpy(x).cuda() for x in s1] if kind != "sgd" else None
+    S2 = [torch.from_numpy(x).cuda() for x in s2] if kind == "adamw" else None
+    ws = fpo.layer_optimize_grouped([g.cuda()] * 3, [a.cuda() for a in A], opt, Wm, W_outs=Wo,
+                                    states1=S1, states2=S2)
+    assert fpo.get_device_status(ws) == fpo.OK
+    tol = 2e-2 if dtype == "bf16" else 1e-5
+    for l in range(3):
+        ref = oracle.optimizer_step(W[l].numpy(), Gs[l], kind=KINDS[kind], lr=lr, t=3,
+                                    clip=CLIPS[clip], s1=s1[l], s2=s2[l])
+        W0 = W[l].double().numpy()
+        d_ref = ref["W"].astype(np.float64) - W0
+        # dW is read back from fp32 W': resolved to fp32 ulps of W'
+        ulp = np.spacing(np.abs(ref["W"]).astype(np.float32)).astype(np.float64)
+        assert rel_frob(f64(Wm[l]) - W0, d_ref) < tol + np.linalg.norm(ulp) / np.linalg.norm(d_ref)
+        if kind != "sgd":
+            assert rel_frob(f64(S1[l]), ref["s1"]) < tol
+        assert rel_frob(f64(Wo[l]), ref["W"]) < max(tol, 4e-3 if dtype == "bf16" else 0)
