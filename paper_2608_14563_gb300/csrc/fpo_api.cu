@@ -129,14 +129,18 @@ EsLayout es_layout(const fpo_error_signal_desc* d) {
     L.Tc = d->T == 0 ? 0 : (chunk < d->T ? chunk : d->T);
     L.ldv = d->dtype == FPO_BF16 ? d->V : (d->V + 7) / 8 * 8;
     const size_t ldv = static_cast<size_t>(L.ldv);
+    // the chunks' fixup row counts follow the status word: one memset clears both
     size_t off = kStatusBytes;
+    L.algo = es_algo(d);
+    L.fix_count = off;
+    if (L.algo == FPO_ES_DIRECT && L.Tc > 0)
+        off = align_up(off + static_cast<size_t>((d->T + L.Tc - 1) / L.Tc) * 4);
     L.yhat = off; off = align_up(off + T * D * esz);
     L.rho = off;  off = align_up(off + T * 4);
     L.lse = off;  off = align_up(off + T * 4);
     L.zy = off;   off = align_up(off + T * 4);
     L.ce = off;   off = align_up(off + T * 4);
     L.part = off; off = align_up(off + T * static_cast<size_t>(L.n_tiles) * 8);
-    L.algo = es_algo(d);
     const bool stored = L.algo == FPO_ES_STORED_LOGITS, direct = L.algo == FPO_ES_DIRECT;
     // g in fp32 for the separate VJP (the direct algorithm writes g~ from the projection)
     L.g = off;    off = align_up(off + (direct ? 0 : T * D * 4));
@@ -152,7 +156,6 @@ EsLayout es_layout(const fpo_error_signal_desc* d) {
     L.cv = off;        off = align_up(off + Tdir * 4);
     L.fix = off;       off = align_up(off + Tcdir * 4);
     L.yfix = off;      off = align_up(off + Tcdir * D * esz);
-    L.fix_count = off; off = align_up(off + (direct ? 4 : 0));
     // the projection's split-K tail (the fp32 partial sums of the last wave's split tiles)
     L.sk = off;        off = align_up(off + (d->dtype == FPO_BF16 ? proj_sk_scratch_bytes() : 0));
     L.total = off;
@@ -218,7 +221,7 @@ int32_t fpo_error_signal(const fpo_error_signal_desc* desc, const void* h, const
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     unsigned* status = reinterpret_cast<unsigned*>(ws);
-    FPO_TRY(cudaMemsetAsync(status, 0, sizeof(unsigned), st));
+    FPO_TRY(cudaMemsetAsync(status, 0, L.yhat, st));  // and the fixup counts behind it
     const int T = static_cast<int>(desc->T), d = static_cast<int>(desc->d),
               V = static_cast<int>(desc->V);
     if (T == 0) {
@@ -272,7 +275,7 @@ int32_t fpo_error_signal(const fpo_error_signal_desc* desc, const void* h, const
         float* beta = reinterpret_cast<float*>(ws + L.beta);
         float* cv = reinterpret_cast<float*>(ws + L.cv);
         int* fix = reinterpret_cast<int*>(ws + L.fix);
-        int* fix_count = reinterpret_cast<int*>(ws + L.fix_count);
+        int* fix_counts = reinterpret_cast<int*>(ws + L.fix_count);
         void* yfix = ws + L.yfix;
         for (int64_t c0 = 0, ci = 0; c0 < T; c0 += L.Tc, ++ci) {
             const int tc = static_cast<int>(L.Tc < T - c0 ? L.Tc : T - c0);
@@ -283,7 +286,7 @@ int32_t fpo_error_signal(const fpo_error_signal_desc* desc, const void* h, const
             float* sxc = sx + static_cast<size_t>(c0) * L.n_tiles;
             float* qc = qz + static_cast<size_t>(c0) * L.n_tiles;
             float* cec = ce ? ce + c0 : nullptr;
-            FPO_TRY(cudaMemsetAsync(fix_count, 0, sizeof(int), st));
+            int* fix_count = fix_counts + ci;
             FPO_TRY(launch_anchor_prob_bf16(yh, W_U, targets + c0, anchor + c0, tc, d, V, suc, sxc,
                                             qc, L.n_tiles, E, status, st));
             FPO_TRY(cmark(ci, 2));
@@ -857,7 +860,8 @@ int64_t fpo_testing_direct_fixup_rows(const fpo_error_signal_desc* desc, const v
     if (L.algo != FPO_ES_DIRECT) return -1;
     if (cudaStreamSynchronize(static_cast<cudaStream_t>(stream)) != cudaSuccess) return -1;
     int n = 0;
-    if (cudaMemcpy(&n, static_cast<const uint8_t*>(workspace) + L.fix_count, sizeof n,
+    const int64_t last = (desc->T + L.Tc - 1) / L.Tc - 1;
+    if (cudaMemcpy(&n, static_cast<const uint8_t*>(workspace) + L.fix_count + 4 * last, sizeof n,
                    cudaMemcpyDeviceToHost) != cudaSuccess)
         return -1;
     return n;

@@ -21,6 +21,7 @@
 
 #include "epilogues.cuh"
 #include "internal.h"
+#include "slot_sum.cuh"
 #include "tc_gemm.cuh"
 #include "tc_gemm_pair.cuh"
 
@@ -112,10 +113,8 @@ cudaError_t run_gemm(const GemmMaps<MAXG>& maps, const typename Epi::Params& ep,
     DevInfo di;
     if (!current_device_info(&di)) return cudaErrorUnknown;
     const long long grid = sh.tiles < di.sm_count ? sh.tiles : di.sm_count;
-    kern<<<static_cast<unsigned>(grid), gemm_threads<Epi>(), L::kBytes, st>>>(maps, ep, sh, status,
-                                                                      wait_limit_ns()),
-        ::fpo::note_launch();
-    return cudaGetLastError();
+    return launch_chained(kern, dim3(static_cast<unsigned>(grid)), gemm_threads<Epi>(), L::kBytes, st,
+                          maps, ep, sh, status, wait_limit_ns());
 }
 
 // Clusters (of `cta` CTAs, the kernel's cluster size) that can be resident at once for a
@@ -214,10 +213,8 @@ cudaError_t run_gemm_pair(const GemmMaps<MAXG>& maps, const typename Epi::Params
             if (plan) *plan = p;
         }
     }
-    kern<<<static_cast<unsigned>(2 * clusters), gemm_threads<Epi>(), L::kBytes, st>>>(
-        maps, ep, sh, status, wait_limit_ns()),
-        ::fpo::note_launch();
-    return cudaGetLastError();
+    return launch_chained(kern, dim3(static_cast<unsigned>(2 * clusters)), gemm_threads<Epi>(),
+                          L::kBytes, st, maps, ep, sh, status, wait_limit_ns());
 }
 
 // Fixups of the split-K tail: sum the tail_split k-range partials of every split tail
@@ -258,6 +255,8 @@ __device__ __forceinline__ bool sk_tail_sum(const GemmShape& sh, const float* __
 template <int BN>
 __global__ void __launch_bounds__(kFixupThreads)
     sk_fixup_kernel(const GemmShape sh, const float* __restrict__ scratch, float* __restrict__ C) {
+    grid_dependency_trigger();
+    grid_dependency_wait();
     int row, n;
     float s4[4];
     if (!sk_tail_sum<BN>(sh, scratch, row, n, s4)) return;
@@ -284,6 +283,8 @@ template <int BN>
 __global__ void __launch_bounds__(kFixupThreads)
     sk_fixup_vjp_kernel(const GemmShape sh, const float* __restrict__ scratch,
                         __nv_bfloat16* __restrict__ out, const VjpArgs va) {
+    grid_dependency_trigger();
+    grid_dependency_wait();
     int row, n;
     float s4[4];
     if (!sk_tail_sum<BN>(sh, scratch, row, n, s4)) return;
@@ -326,19 +327,16 @@ template <int BN>
 cudaError_t launch_sk_fixup(const SkPlan& plan, const GemmShape& sh, const float* scratch,
                             float* C, cudaStream_t st) {
     if (plan.tail_tiles <= 0) return cudaSuccess;
-    sk_fixup_kernel<BN><<<sk_fixup_grid<BN>(plan), kFixupThreads, 0, st>>>(
-        sk_fixup_shape(plan, sh), scratch, C), ::fpo::note_launch();
-    return cudaGetLastError();
+    return launch_chained(sk_fixup_kernel<BN>, sk_fixup_grid<BN>(plan), kFixupThreads, 0, st,
+                          sk_fixup_shape(plan, sh), scratch, C);
 }
 
 template <int BN>
 cudaError_t launch_sk_fixup_vjp(const SkPlan& plan, const GemmShape& sh, const float* scratch,
                                 void* out, const VjpArgs& va, cudaStream_t st) {
     if (plan.tail_tiles <= 0) return cudaSuccess;
-    sk_fixup_vjp_kernel<BN><<<sk_fixup_grid<BN>(plan), kFixupThreads, 0, st>>>(
-        sk_fixup_shape(plan, sh), scratch, static_cast<__nv_bfloat16*>(out), va),
-        ::fpo::note_launch();
-    return cudaGetLastError();
+    return launch_chained(sk_fixup_vjp_kernel<BN>, sk_fixup_grid<BN>(plan), kFixupThreads, 0, st,
+                          sk_fixup_shape(plan, sh), scratch, static_cast<__nv_bfloat16*>(out), va);
 }
 
 constexpr int kProjBN = 256;     // projection tiles where 512 columns are too wide
@@ -774,51 +772,20 @@ size_t opt_step_partial_bytes(int n_layers, int d, int d_ff) {
            kColSlots * 2 * sizeof(float);
 }
 
-// Second pass of the fused cosine: one block per layer adds the layer's slot triples in a
-// fixed order (thread-strided fp64 sums, a fixed butterfly per warp, then the warps' sums
-// in warp order) and writes <G, Y>, ||G||^2, ||Y||^2 and the cosine.
-constexpr int kCosFinalThreads = 256;
-
-__device__ __forceinline__ double warp_sum_f64(double x) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-}
-
-__global__ void __launch_bounds__(kCosFinalThreads)
+// Second pass of the fused cosine: a cluster per layer adds the layer's slot triples in a
+// fixed order and writes <G, Y>, ||G||^2, ||Y||^2 and the cosine.
+__global__ void __cluster_dims__(kSlotBlocks, 1, 1) __launch_bounds__(kSlotThreads)
     grad_cosine_final_kernel(const float* __restrict__ part, int slots, double* __restrict__ out) {
-    const int layer = blockIdx.x;
-    const float* p = part + static_cast<size_t>(layer) * slots * 3;
-    double gy = 0.0, gg = 0.0, yy = 0.0;
-#pragma unroll 4
-    for (int i = threadIdx.x; i < slots; i += kCosFinalThreads) {
-        gy += p[3 * i];
-        gg += p[3 * i + 1];
-        yy += p[3 * i + 2];
-    }
-    gy = warp_sum_f64(gy);
-    gg = warp_sum_f64(gg);
-    yy = warp_sum_f64(yy);
-    __shared__ double sh[3][kCosFinalThreads / 32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) {
-        sh[0][wid] = gy;
-        sh[1][wid] = gg;
-        sh[2][wid] = yy;
-    }
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    gy = gg = yy = 0.0;
-    for (int k = 0; k < kCosFinalThreads / 32; ++k) {
-        gy += sh[0][k];
-        gg += sh[1][k];
-        yy += sh[2][k];
-    }
+    grid_dependency_trigger();
+    grid_dependency_wait();
+    const int layer = blockIdx.x / kSlotBlocks;
+    double t[3];
+    if (!slot_sum<3>(part + static_cast<size_t>(layer) * slots * 3, slots, t)) return;
     double* o = out + 4 * layer;
-    o[0] = gy;
-    o[1] = gg;
-    o[2] = yy;
-    o[3] = (gg > 0.0 && yy > 0.0) ? gy / (sqrt(gg) * sqrt(yy)) : 0.0;
+    o[0] = t[0];
+    o[1] = t[1];
+    o[2] = t[2];
+    o[3] = (t[1] > 0.0 && t[2] > 0.0) ? t[0] / (sqrt(t[1]) * sqrt(t[2])) : 0.0;
 }
 
 size_t grad_cosine_partial_bytes(int n, int d, int d_ff) {
@@ -869,10 +836,8 @@ cudaError_t launch_grad_cosine_bf16(int n, int T, int d, int d_ff, const void* c
         e = run_gemm<kUpdBN, true, true, kUpdStages, kMaxGroups, EpiGradCos>(
             maps, ep, make_shape(d, d_ff, T, kUpdBN, n, band_for(false)), status, st);
     if (e != cudaSuccess) return e;
-    grad_cosine_final_kernel<<<n, kCosFinalThreads, 0, st>>>(
-        part, ep.m256 * ep.n_blocks * kColSlots, out),
-        ::fpo::note_launch();
-    return cudaGetLastError();
+    return launch_chained(grad_cosine_final_kernel, dim3(kSlotBlocks * n), kSlotThreads, 0, st, part,
+                          ep.m256 * ep.n_blocks * kColSlots, out);
 }
 
 cudaError_t launch_swiglu_bf16(int T, int d, int d_ff, const void* g, const void* W3,

@@ -77,6 +77,7 @@ template <typename TG, typename TW, bool kDot>
 __global__ void __launch_bounds__(kNrThreads)
     grouped_partial_kernel(const __grid_constant__ NrPtrs ptrs, int64_t n,
                            double* __restrict__ partial) {
+    grid_dependency_wait();
     const int layer = blockIdx.y;
     const TG* G = static_cast<const TG*>(ptrs.G[layer]);
     const TW* W = static_cast<const TW*>(ptrs.W[layer]);
@@ -144,6 +145,7 @@ __global__ void __launch_bounds__(kNrThreads)
             gw += g * w;
         }
     }
+    grid_dependency_trigger();
     __shared__ double sh[3][kNrThreads / 32];
     const double s0 = warp_sum_d(gg), s1 = warp_sum_d(ww), s2 = warp_sum_d(gw);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -180,6 +182,7 @@ __device__ __forceinline__ double warp_sum_f64(double x) {
 __global__ void grouped_final_kernel(const double* __restrict__ partial, int blocks,
                                      int n_layers, int mode, double rel,
                                      double* __restrict__ out) {
+    grid_dependency_wait();
     const int layer = blockIdx.x;
     const int lane = threadIdx.x;
     const double* p = partial + static_cast<size_t>(layer) * blocks * 3;
@@ -211,14 +214,13 @@ __global__ void grouped_final_kernel(const double* __restrict__ partial, int blo
 template <typename TG, typename TW, bool kDot>
 cudaError_t run(const NrPtrs& ptrs, int n_layers, int64_t n, int blocks, int mode, double rel,
                 double* partial, double* out, cudaStream_t st) {
-    grouped_partial_kernel<TG, TW, kDot>
-        <<<dim3(static_cast<unsigned>(blocks), static_cast<unsigned>(n_layers)), kNrThreads, 0,
-           st>>>(ptrs, n, partial), ::fpo::note_launch();
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_chained(
+        grouped_partial_kernel<TG, TW, kDot>,
+        dim3(static_cast<unsigned>(blocks), static_cast<unsigned>(n_layers)), kNrThreads, 0, st, ptrs,
+        n, partial);
     if (e != cudaSuccess) return e;
-    grouped_final_kernel<<<n_layers, 32, 0, st>>>(partial, blocks, n_layers, mode, rel, out),
-        ::fpo::note_launch();
-    return cudaGetLastError();
+    return launch_chained(grouped_final_kernel, dim3(n_layers), 32, 0, st, partial, blocks, n_layers,
+                          mode, rel, out);
 }
 
 NrPtrs pack(int n_layers, const void* const* G, const void* const* W) {

@@ -48,6 +48,41 @@ uint64_t wait_limit_ns();
 void note_launch();
 uint64_t launches();
 
+// Launches a kernel so that it may become resident while the kernel before it in the stream
+// is still running (programmatic dependent launch).  Every such kernel calls
+// grid_dependency_wait() in every thread before it touches memory that another kernel reads
+// or writes, and before any block of it exits: the wait ends when the kernel before has
+// completed and its writes are visible.  It calls grid_dependency_trigger() where the next
+// kernel may start taking its place: at once in short kernels, near the end in the GEMMs,
+// whose SMs would otherwise be shared with waiting blocks for milliseconds.
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem,
+                           cudaStream_t st, A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    note_launch();
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_dependency_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void grid_dependency_trigger() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 // ------------------------------------------------------------ bf16 (tcgen05)
 // Logits pass: part[T, n_tiles] (max, sum exp), zy[T] (target logits) and, when z is
 // non-null, the fp32 logits z[T, V] (stored-logits algorithm).

@@ -22,6 +22,7 @@
 
 #include "internal.h"
 #include "optim_math.cuh"
+#include "slot_sum.cuh"
 
 namespace fpo {
 namespace {
@@ -197,40 +198,18 @@ __global__ void __launch_bounds__(kOptThreads)
 }
 
 // Clip after an epilogue that summed the norms (EpiOptStep: d the unclipped step,
-// EpiStoreGroupF32: d the gradient): one block per layer adds the layer's
-// (||W||^2, ||d||^2) slot pairs in a fixed order (thread-strided fp64 sums, a fixed
-// butterfly per warp, then the warps' sums in warp order; 256 threads keep many loads
-// in flight, where one warp waited on one load at a time) and writes the layer's scale
+// EpiStoreGroupF32: d the gradient): a cluster per layer adds the layer's
+// (||W||^2, ||d||^2) slot pairs in a fixed order and writes the layer's scale
 // min(1, clip_frac ||W|| / ||d||).
-__global__ void __launch_bounds__(kScaleThreads)
+__global__ void __cluster_dims__(kSlotBlocks, 1, 1) __launch_bounds__(kSlotThreads)
     opt_scale_kernel(const float* __restrict__ part, int slots, const OptimParams op,
-                          float* __restrict__ scales) {
-    const int layer = blockIdx.x;
-    const float2* p = reinterpret_cast<const float2*>(part) + static_cast<size_t>(layer) * slots;
-    double ww = 0.0, dd = 0.0;
-#pragma unroll 4
-    for (int i = threadIdx.x; i < slots; i += kScaleThreads) {
-        const float2 v = p[i];
-        ww += v.x;
-        dd += v.y;
-    }
-    ww = warp_sum_d(ww);
-    dd = warp_sum_d(dd);
-    __shared__ double sh[2][kScaleThreads / 32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) {
-        sh[0][wid] = ww;
-        sh[1][wid] = dd;
-    }
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    ww = dd = 0.0;
-    for (int k = 0; k < kScaleThreads / 32; ++k) {
-        ww += sh[0][k];
-        dd += sh[1][k];
-    }
-    const double lim = static_cast<double>(op.clip_frac) * sqrt(ww);
-    scales[layer] = static_cast<float>(sqrt(dd) > lim ? lim / sqrt(dd) : 1.0);
+                     float* __restrict__ scales) {
+    grid_dependency_wait();
+    const int layer = blockIdx.x / kSlotBlocks;
+    double t[2];
+    if (!slot_sum<2>(part + static_cast<size_t>(layer) * slots * 2, slots, t)) return;
+    const double lim = static_cast<double>(op.clip_frac) * sqrt(t[0]);
+    scales[layer] = static_cast<float>(sqrt(t[1]) > lim ? lim / sqrt(t[1]) : 1.0);
 }
 
 // W <- W + s d with the layer's scale, and W_out = bf16(W) (16-byte vectors); d = D, or
@@ -258,6 +237,9 @@ __global__ void __launch_bounds__(kOptThreads)
     }
 }
 
+// Blocks per layer of the element-wise passes: all of them resident at once, which a launch
+// beside the end of a GEMM (launch_chained) would spoil: their blocks then crowd the SMs
+// that are free first (apply pass 790 -> 1040 us).
 int blocks_per_layer(int n_layers) {
     DevInfo di;
     const int sms = current_device_info(&di) ? di.sm_count : 148;
@@ -331,9 +313,8 @@ cudaError_t launch_optimizer(int dtype, int n_layers, size_t n_elem, const Optim
 cudaError_t launch_opt_scale(int n_layers, const OptimParams& op, const float* part, int slots,
                              float* scales, cudaStream_t st) {
     if (n_layers < 1 || n_layers > kMaxLayers) return cudaErrorInvalidValue;
-    opt_scale_kernel<<<n_layers, kScaleThreads, 0, st>>>(part, slots, op, scales),
-        ::fpo::note_launch();
-    return cudaGetLastError();
+    return launch_chained(opt_scale_kernel, dim3(kSlotBlocks * n_layers), kSlotThreads, 0, st, part, slots, op,
+                          scales);
 }
 
 cudaError_t launch_opt_step_apply(int n_layers, size_t n_elem, const OptimParams& op,

@@ -110,6 +110,8 @@ __global__ void __launch_bounds__(kRowThreads)
                        TT* __restrict__ yhat, float* __restrict__ rho, const int32_t* __restrict__ y,
                        int V, unsigned* status, const TT* __restrict__ W_U,
                        float* __restrict__ anchor) {
+    grid_dependency_trigger();
+    grid_dependency_wait();
     const int lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
     for (int row = blockIdx.x * wpb + (threadIdx.x >> 5); row < T; row += gridDim.x * wpb) {
@@ -186,6 +188,8 @@ __global__ void __launch_bounds__(kBlkThreads)
                            float* __restrict__ rho, const int32_t* __restrict__ y, int V,
                            unsigned* status, const __nv_bfloat16* __restrict__ W_U,
                            float* __restrict__ anchor) {
+    grid_dependency_trigger();
+    grid_dependency_wait();
     constexpr int NV = EPT / 8;
     // h row r and, for an in-range target, the target's unembedding row (the anchor's
     // operand); the next row's are loaded before the current row is computed
@@ -263,6 +267,8 @@ __global__ void __launch_bounds__(kBlkThreads)
     rmsnorm_vjp_row_kernel(const float* __restrict__ g, const __nv_bfloat16* __restrict__ h,
                            const __nv_bfloat16* __restrict__ w, const float* __restrict__ rho,
                            int T, int d, float min_rms, __nv_bfloat16* __restrict__ out) {
+    grid_dependency_trigger();
+    grid_dependency_wait();
     constexpr int NV = EPT / 8;
     for (int row = blockIdx.x; row < T; row += gridDim.x) {
         const float r = rho[row];
@@ -326,6 +332,8 @@ __global__ void __launch_bounds__(kRowThreads)
     rmsnorm_vjp_kernel(const float* __restrict__ g, const TT* __restrict__ h,
                        const TT* __restrict__ w, const float* __restrict__ rho, int T, int d,
                        float min_rms, TT* __restrict__ out) {
+    grid_dependency_trigger();
+    grid_dependency_wait();
     const int lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
     for (int row = blockIdx.x * wpb + (threadIdx.x >> 5); row < T; row += gridDim.x * wpb) {
@@ -361,6 +369,8 @@ __global__ void __launch_bounds__(kRowThreads)
 __global__ void __launch_bounds__(kRowThreads)
     lse_combine_kernel(const float2* __restrict__ part, int n_tiles, int T,
                        const float* __restrict__ zy, float* __restrict__ lse, float* __restrict__ ce) {
+    grid_dependency_trigger();
+    grid_dependency_wait();
     const int lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
     for (int row = blockIdx.x * wpb + (threadIdx.x >> 5); row < T; row += gridDim.x * wpb) {
@@ -406,6 +416,8 @@ __global__ void __launch_bounds__(kRowThreads)
                           float* __restrict__ ce, float* __restrict__ alpha,
                           float* __restrict__ beta, float* __restrict__ cv,
                           int* __restrict__ fix, int* __restrict__ fix_count) {
+    grid_dependency_trigger();
+    grid_dependency_wait();
     const int lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
     for (int row = blockIdx.x * wpb + (threadIdx.x >> 5); row < T; row += gridDim.x * wpb) {
@@ -452,6 +464,8 @@ __global__ void __launch_bounds__(kRowThreads)
 __global__ void __launch_bounds__(kRowThreads)
     gather_rows_kernel(const uint4* __restrict__ src, const int* __restrict__ fix,
                        const int* __restrict__ count, int v8, uint4* __restrict__ dst) {
+    grid_dependency_trigger();
+    grid_dependency_wait();
     const long long n = static_cast<long long>(*count) * v8;
     for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -467,6 +481,8 @@ __global__ void __launch_bounds__(kRowThreads)
                             const int* __restrict__ fix_count, int n_tiles,
                             const float* __restrict__ anchor, float* __restrict__ lse,
                             float* __restrict__ ce) {
+    grid_dependency_trigger();
+    grid_dependency_wait();
     const int lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
     const int n = *fix_count;
@@ -498,6 +514,8 @@ __global__ void __launch_bounds__(kRowThreads)
                                 int n_tiles, const float* __restrict__ anchor, float s,
                                 float* __restrict__ alpha, float* __restrict__ beta,
                                 float* __restrict__ cv) {
+    grid_dependency_trigger();
+    grid_dependency_wait();
     const int lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
     const int n = *fix_count;
@@ -520,14 +538,17 @@ __global__ void __launch_bounds__(kRowThreads)
     }
 }
 
-constexpr int kMeanThreads = 1024;
+// Mean of x[0, n) by one block, in a fixed order: thread i adds x[i], x[i + kMeanThreads],
+// ..., its loads issued kBatch at a time (the loop waits once per batch), then a fixed
+// butterfly per warp and the warps' sums in warp order.
+constexpr int kMeanThreads = 512;
 
 __global__ void __launch_bounds__(kMeanThreads) mean_kernel(const float* __restrict__ x, int n,
                                                             float* __restrict__ out) {
-    __shared__ double buf[kMeanThreads];
-    // thread i adds x[i], x[i + kMeanThreads], ... in that order; eight loads are issued
-    // before their adds, so the loop waits once per eight elements, not once per element
-    constexpr int kBatch = 8;
+    grid_dependency_trigger();
+    grid_dependency_wait();
+    __shared__ double buf[kMeanThreads / 32];
+    constexpr int kBatch = 16;
     double acc = 0.0;
     long long i = threadIdx.x;
     for (; i + (kBatch - 1) * static_cast<long long>(kMeanThreads) < n; i += kBatch * kMeanThreads) {
@@ -538,13 +559,16 @@ __global__ void __launch_bounds__(kMeanThreads) mean_kernel(const float* __restr
         for (int k = 0; k < kBatch; ++k) acc += static_cast<double>(v[k]);
     }
     for (; i < n; i += kMeanThreads) acc += static_cast<double>(x[i]);
-    buf[threadIdx.x] = acc;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = acc;
     __syncthreads();
-    for (int s = kMeanThreads / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) buf[threadIdx.x] += buf[threadIdx.x + s];
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+#pragma unroll
+        for (int k = 0; k < kMeanThreads / 32; ++k) t += buf[k];
+        out[0] = static_cast<float>(t / static_cast<double>(n));
     }
-    if (threadIdx.x == 0) out[0] = static_cast<float>(buf[0] / static_cast<double>(n));
 }
 
 __global__ void cast_f32_kernel(const float* __restrict__ src, size_t n, __nv_bfloat16* __restrict__ dst) {
@@ -562,6 +586,8 @@ __global__ void __launch_bounds__(kErrThreads)
     error_from_logits_kernel(const float* __restrict__ z, const float* __restrict__ lse,
                              const int32_t* __restrict__ y, int M, int V, long long ld, float s,
                              void* __restrict__ E) {
+    grid_dependency_trigger();
+    grid_dependency_wait();
     for (int row = blockIdx.x; row < M; row += gridDim.x) {
         const float l = lse[row];
         const float l2 = l * kLog2e;
@@ -974,31 +1000,31 @@ cudaError_t launch_rmsnorm_fwd(int dtype, const void* h, const void* w, int T, i
         auto* yy = static_cast<__nv_bfloat16*>(yhat);
         const auto* wu = static_cast<const __nv_bfloat16*>(W_U);
         if (ept == 8)
-            rmsnorm_fwd_row_kernel<8><<<blk_grid(T), kBlkThreads, 0, st>>>(
-                hh, ww, T, d, eps, yy, rho, y, V, status, wu, anchor), ::fpo::note_launch();
+            return launch_chained(rmsnorm_fwd_row_kernel<8>, dim3(blk_grid(T)), kBlkThreads, 0, st,
+                                  hh, ww, T, d, eps, yy, rho, y, V, status, wu, anchor);
         else if (ept == 16)
-            rmsnorm_fwd_row_kernel<16><<<blk_grid(T), kBlkThreads, 0, st>>>(
-                hh, ww, T, d, eps, yy, rho, y, V, status, wu, anchor), ::fpo::note_launch();
+            return launch_chained(rmsnorm_fwd_row_kernel<16>, dim3(blk_grid(T)), kBlkThreads, 0,
+                                  st, hh, ww, T, d, eps, yy, rho, y, V, status, wu, anchor);
         else
-            rmsnorm_fwd_row_kernel<32><<<blk_grid(T), kBlkThreads, 0, st>>>(
-                hh, ww, T, d, eps, yy, rho, y, V, status, wu, anchor), ::fpo::note_launch();
+            return launch_chained(rmsnorm_fwd_row_kernel<32>, dim3(blk_grid(T)), kBlkThreads, 0,
+                                  st, hh, ww, T, d, eps, yy, rho, y, V, status, wu, anchor);
     } else if (dtype == 1) {
-        rmsnorm_fwd_kernel<__nv_bfloat16, 8><<<grid, kRowThreads, 0, st>>>(
-            static_cast<const __nv_bfloat16*>(h), static_cast<const __nv_bfloat16*>(w), T, d, eps,
-            static_cast<__nv_bfloat16*>(yhat), rho, y, V, status,
-            static_cast<const __nv_bfloat16*>(W_U), anchor), ::fpo::note_launch();
+        return launch_chained(rmsnorm_fwd_kernel<__nv_bfloat16, 8>, dim3(grid), kRowThreads, 0, st,
+                              static_cast<const __nv_bfloat16*>(h),
+                              static_cast<const __nv_bfloat16*>(w), T, d, eps,
+                              static_cast<__nv_bfloat16*>(yhat), rho, y, V, status,
+                              static_cast<const __nv_bfloat16*>(W_U), anchor);
     } else if (d % 4 == 0) {
-        rmsnorm_fwd_kernel<float, 4><<<grid, kRowThreads, 0, st>>>(
-            static_cast<const float*>(h), static_cast<const float*>(w), T, d, eps,
-            static_cast<float*>(yhat), rho, y, V, status, static_cast<const float*>(W_U), anchor),
-            ::fpo::note_launch();
+        return launch_chained(rmsnorm_fwd_kernel<float, 4>, dim3(grid), kRowThreads, 0, st,
+                              static_cast<const float*>(h), static_cast<const float*>(w), T, d,
+                              eps, static_cast<float*>(yhat), rho, y, V, status,
+                              static_cast<const float*>(W_U), anchor);
     } else {
-        rmsnorm_fwd_kernel<float, 1><<<grid, kRowThreads, 0, st>>>(
-            static_cast<const float*>(h), static_cast<const float*>(w), T, d, eps,
-            static_cast<float*>(yhat), rho, y, V, status, static_cast<const float*>(W_U), anchor),
-            ::fpo::note_launch();
+        return launch_chained(rmsnorm_fwd_kernel<float, 1>, dim3(grid), kRowThreads, 0, st,
+                              static_cast<const float*>(h), static_cast<const float*>(w), T, d,
+                              eps, static_cast<float*>(yhat), rho, y, V, status,
+                              static_cast<const float*>(W_U), anchor);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_direct_combine(const float* su, const float* sx, const float* qz, int n_tiles,
@@ -1006,20 +1032,17 @@ cudaError_t launch_direct_combine(const float* su, const float* sx, const float*
                                   float* lse, float* ce, float* alpha, float* beta, float* cv,
                                   int* fix, int* fix_count, cudaStream_t st) {
     if (T <= 0) return cudaSuccess;
-    direct_combine_kernel<<<row_grid(T), kRowThreads, 0, st>>>(
-        su, sx, qz, n_tiles, T, V, y, anchor, s, lse, ce, alpha, beta, cv, fix, fix_count),
-        ::fpo::note_launch();
-    return cudaGetLastError();
+    return launch_chained(direct_combine_kernel, dim3(row_grid(T)), kRowThreads, 0, st, su, sx, qz,
+                          n_tiles, T, V, y, anchor, s, lse, ce, alpha, beta, cv, fix, fix_count);
 }
 
 cudaError_t launch_gather_rows(const void* yhat, const int* fix, const int* fix_count, int d,
                                void* out, cudaStream_t st) {
     DevInfo di;
     const int sms = current_device_info(&di) ? di.sm_count : 148;
-    gather_rows_kernel<<<4 * sms, kRowThreads, 0, st>>>(static_cast<const uint4*>(yhat), fix,
-                                                        fix_count, d / 8, static_cast<uint4*>(out)),
-        ::fpo::note_launch();
-    return cudaGetLastError();
+    return launch_chained(gather_rows_kernel, dim3(4 * sms), kRowThreads, 0, st,
+                          static_cast<const uint4*>(yhat), fix, fix_count, d / 8,
+                          static_cast<uint4*>(out));
 }
 
 cudaError_t launch_direct_fixup_lse(const float2* part, const int* fix, const int* fix_count,
@@ -1027,9 +1050,8 @@ cudaError_t launch_direct_fixup_lse(const float2* part, const int* fix, const in
                                     cudaStream_t st) {
     DevInfo di;
     const int sms = current_device_info(&di) ? di.sm_count : 148;
-    direct_fixup_lse_kernel<<<sms, kRowThreads, 0, st>>>(part, fix, fix_count, n_tiles, anchor,
-                                                        lse, ce), ::fpo::note_launch();
-    return cudaGetLastError();
+    return launch_chained(direct_fixup_lse_kernel, dim3(sms), kRowThreads, 0, st, part, fix,
+                          fix_count, n_tiles, anchor, lse, ce);
 }
 
 cudaError_t launch_direct_fixup_factors(const float* sx, const float* qz, const int* fix,
@@ -1038,10 +1060,8 @@ cudaError_t launch_direct_fixup_factors(const float* sx, const float* qz, const 
                                         cudaStream_t st) {
     DevInfo di;
     const int sms = current_device_info(&di) ? di.sm_count : 148;
-    direct_fixup_factors_kernel<<<sms, kRowThreads, 0, st>>>(sx, qz, fix, fix_count, n_tiles,
-                                                            anchor, s, alpha, beta, cv),
-        ::fpo::note_launch();
-    return cudaGetLastError();
+    return launch_chained(direct_fixup_factors_kernel, dim3(sms), kRowThreads, 0, st, sx, qz, fix,
+                          fix_count, n_tiles, anchor, s, alpha, beta, cv);
 }
 
 cudaError_t launch_rmsnorm_vjp(int dtype, const float* g, const void* h, const void* w,
@@ -1055,31 +1075,28 @@ cudaError_t launch_rmsnorm_vjp(int dtype, const float* g, const void* h, const v
         const auto* ww = static_cast<const __nv_bfloat16*>(w);
         auto* oo = static_cast<__nv_bfloat16*>(out);
         if (ept == 8)
-            rmsnorm_vjp_row_kernel<8><<<blk_grid(T), kBlkThreads, 0, st>>>(g, hh, ww, rho, T, d,
-                                                                        min_rms, oo),
-                ::fpo::note_launch();
+            return launch_chained(rmsnorm_vjp_row_kernel<8>, dim3(blk_grid(T)), kBlkThreads, 0, st,
+                                  g, hh, ww, rho, T, d, min_rms, oo);
         else if (ept == 16)
-            rmsnorm_vjp_row_kernel<16><<<blk_grid(T), kBlkThreads, 0, st>>>(g, hh, ww, rho, T, d,
-                                                                         min_rms, oo),
-                ::fpo::note_launch();
+            return launch_chained(rmsnorm_vjp_row_kernel<16>, dim3(blk_grid(T)), kBlkThreads, 0,
+                                  st, g, hh, ww, rho, T, d, min_rms, oo);
         else
-            rmsnorm_vjp_row_kernel<32><<<blk_grid(T), kBlkThreads, 0, st>>>(g, hh, ww, rho, T, d,
-                                                                         min_rms, oo),
-                ::fpo::note_launch();
+            return launch_chained(rmsnorm_vjp_row_kernel<32>, dim3(blk_grid(T)), kBlkThreads, 0,
+                                  st, g, hh, ww, rho, T, d, min_rms, oo);
     } else if (dtype == 1) {
-        rmsnorm_vjp_kernel<__nv_bfloat16, 8><<<grid, kRowThreads, 0, st>>>(
-            g, static_cast<const __nv_bfloat16*>(h), static_cast<const __nv_bfloat16*>(w), rho, T,
-            d, min_rms, static_cast<__nv_bfloat16*>(out)), ::fpo::note_launch();
+        return launch_chained(rmsnorm_vjp_kernel<__nv_bfloat16, 8>, dim3(grid), kRowThreads, 0, st,
+                              g, static_cast<const __nv_bfloat16*>(h),
+                              static_cast<const __nv_bfloat16*>(w), rho, T, d, min_rms,
+                              static_cast<__nv_bfloat16*>(out));
     } else if (d % 4 == 0) {
-        rmsnorm_vjp_kernel<float, 4><<<grid, kRowThreads, 0, st>>>(
-            g, static_cast<const float*>(h), static_cast<const float*>(w), rho, T, d, min_rms,
-            static_cast<float*>(out)), ::fpo::note_launch();
+        return launch_chained(rmsnorm_vjp_kernel<float, 4>, dim3(grid), kRowThreads, 0, st, g,
+                              static_cast<const float*>(h), static_cast<const float*>(w), rho, T,
+                              d, min_rms, static_cast<float*>(out));
     } else {
-        rmsnorm_vjp_kernel<float, 1><<<grid, kRowThreads, 0, st>>>(
-            g, static_cast<const float*>(h), static_cast<const float*>(w), rho, T, d, min_rms,
-            static_cast<float*>(out)), ::fpo::note_launch();
+        return launch_chained(rmsnorm_vjp_kernel<float, 1>, dim3(grid), kRowThreads, 0, st, g,
+                              static_cast<const float*>(h), static_cast<const float*>(w), rho, T,
+                              d, min_rms, static_cast<float*>(out));
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_cast_f32(int dtype, const float* src, size_t n, void* dst, cudaStream_t st) {
@@ -1098,12 +1115,11 @@ cudaError_t launch_error_from_logits(int dtype, const float* z, const float* lse
     const int sms = current_device_info(&di) ? di.sm_count : 148;
     const int grid = M < sms * 8 ? M : sms * 8;
     if (dtype == 1)
-        error_from_logits_kernel<true><<<grid, kErrThreads, 0, st>>>(z, lse, y, M, V, ld, s, E),
-            ::fpo::note_launch();
+        return launch_chained(error_from_logits_kernel<true>, dim3(grid), kErrThreads, 0, st, z,
+                              lse, y, M, V, ld, s, E);
     else
-        error_from_logits_kernel<false><<<grid, kErrThreads, 0, st>>>(z, lse, y, M, V, ld, s, E),
-            ::fpo::note_launch();
-    return cudaGetLastError();
+        return launch_chained(error_from_logits_kernel<false>, dim3(grid), kErrThreads, 0, st, z,
+                              lse, y, M, V, ld, s, E);
 }
 
 cudaError_t launch_wait_timeout(unsigned* status, uint64_t limit_ns, cudaStream_t st) {
@@ -1196,15 +1212,13 @@ cudaError_t launch_layer_signals(int dtype, int n_layers, const void* g, const v
 cudaError_t launch_lse_combine(const float2* part, int n_tiles, int T, const float* zy, float* lse,
                                float* ce, cudaStream_t st) {
     if (T <= 0) return cudaSuccess;
-    lse_combine_kernel<<<row_grid(T), kRowThreads, 0, st>>>(part, n_tiles, T, zy, lse, ce),
-        ::fpo::note_launch();
-    return cudaGetLastError();
+    return launch_chained(lse_combine_kernel, dim3(row_grid(T)), kRowThreads, 0, st, part, n_tiles,
+                          T, zy, lse, ce);
 }
 
 cudaError_t launch_mean(const float* x, int n, float* out, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    mean_kernel<<<1, kMeanThreads, 0, st>>>(x, n, out), ::fpo::note_launch();
-    return cudaGetLastError();
+    return launch_chained(mean_kernel, dim3(1), kMeanThreads, 0, st, x, n, out);
 }
 
 }  // namespace fpo

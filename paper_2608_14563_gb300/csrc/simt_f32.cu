@@ -180,6 +180,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
         for (int j = 0; j < 2 * kH; ++j) acc[i][j] = make_float2(0.f, 0.f);
 
+    grid_dependency_wait();
     SliceLoader<BT, kAKC> la;
     SliceLoader<BT, kBKC> lb;
     if (s0 < s1) {
@@ -230,6 +231,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
     }
 
+    grid_dependency_trigger();
     // k ranges of the cluster: every block leaves its sums in shared memory, thread by
     // thread, and block `rank` adds the rows i with i mod S = rank in rank order
     if (S > 1) {
@@ -403,15 +405,19 @@ cudaError_t run_tile(SimtOps ops, const Epi& ep, int groups, cudaStream_t st) {
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = static_cast<size_t>(smem);
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 1;
-    at[0].val.clusterDim.y = static_cast<unsigned>(ops.splits);
-    at[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_chained
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 1;
+    at[1].val.clusterDim.y = static_cast<unsigned>(ops.splits);
+    at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = ops.splits > 1 ? 1 : 0;
+    cfg.numAttrs = ops.splits > 1 ? 2 : 1;
     note_launch();
-    return cudaLaunchKernelEx(&cfg, kern, ops, ep);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, ops, ep);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 // Tiles of 128 or 64, whichever simt_cost estimates faster (the same sums either way).

@@ -280,6 +280,7 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
+    grid_dependency_wait();
 
     const WaitGuard guard{abort_flag, status, wait_limit_ns};
 
@@ -308,6 +309,7 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
             }
+            grid_dependency_trigger();  // only the last tiles' MMAs and epilogues are left
             // Do not leave copies landing in shared memory after exit: the last copy of
             // every stage is awaited (at once when it was consumed), also when another
             // role gave up first.

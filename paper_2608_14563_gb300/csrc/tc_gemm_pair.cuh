@@ -238,7 +238,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<Epi>(),
     // reach past K; its loads read zeros there)
     sh.k_blocks = (sh.k_blocks + kSub - 1) / kSub;
     if (sh.m_dev) {  // rows counted on the device (every thread reads the same value)
-        const int m = min(*sh.m_dev, sh.M);
+        grid_dependency_wait();
+        const int m = min(*static_cast<const volatile int*>(sh.m_dev), sh.M);
         if (m <= 0) return;
         sh.M = m;
         sh.m_blocks = (m + kPairBM - 1) / kPairBM;
@@ -296,6 +297,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<Epi>(),
     cluster_sync();  // barrier initialisation and TMEM allocation visible to the pair
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
+    // the set-up above ran beside the end of the kernel before; its results are read from here
+    grid_dependency_wait();
 
     const WaitGuard guard{abort_flag, status, wait_limit_ns};
 
@@ -337,6 +340,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<Epi>(),
                 }
             }
             *issued_word = issued;  // read by the leader at teardown
+            grid_dependency_trigger();  // only the last tiles' MMAs and epilogues are left
         }
         __syncwarp();
     } else if (warp == 1) {
