@@ -179,18 +179,22 @@ def _dtype_code(t: torch.Tensor) -> int:
 
 
 def _ptr(t):
+    # an int: ctypes passes it through a c_void_p argument or array slot
     if t is None:
         return None
     if not t.is_cuda:
         raise ValueError("libfpo takes CUDA tensors")
     if not t.is_contiguous():
         raise ValueError("libfpo takes contiguous tensors")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    # the current stream's handle without building a torch Stream object (3 us a call, a
+    # tenth of the host time of a small step)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _nbytes(t: torch.Tensor) -> int:
@@ -241,9 +245,8 @@ def error_signal(h, norm_w, W_U, targets, g_out, *, eps=1e-6, min_rms=0.5, loss_
     desc = error_signal_desc(T, d, V, _dtype_code(h), eps=eps, min_rms=min_rms,
                              loss_scale=loss_scale, t_chunk=t_chunk, stage_events=stage_events,
                              algo=algo, per_chunk_events=per_chunk_events)
-    need = error_signal_workspace(desc)
     if workspace is None:
-        workspace = _workspace(need, h.device)
+        workspace = _workspace(error_signal_workspace(desc), h.device)
     rc = _lib.fpo_error_signal(ctypes.byref(desc), _ptr(h), _ptr(norm_w), _ptr(W_U), _ptr(targets),
                                _ptr(g_out), _ptr(lse_out), _ptr(loss_out), _ptr(workspace),
                                _nbytes(workspace), _stream(stream))
@@ -281,10 +284,7 @@ def layer_update(g, A, lr, *, W_master=None, W_out=None, G_out=None, workspace=N
 def _ptr_array(ts, n):
     if ts is None:
         return None
-    arr = (_vp * n)()
-    for i, t in enumerate(ts):
-        arr[i] = None if t is None else _ptr(t).value
-    return arr
+    return (_vp * n)(*[_ptr(t) for t in ts])
 
 
 def layer_update_grouped(g, As, lr, *, W_masters=None, W_outs=None, G_outs=None, workspace=None,
@@ -502,7 +502,7 @@ def h2d_copy(dsts, srcs, *, stream=None):
     for c in range(0, len(srcs), MAX_COPY_BUFFERS):
         ds, ss = dsts[c:c + MAX_COPY_BUFFERS], srcs[c:c + MAX_COPY_BUFFERS]
         n = len(ss)
-        darr = (_vp * n)(*[_ptr(t).value for t in ds])
+        darr = (_vp * n)(*[_ptr(t) for t in ds])
         sarr = (_vp * n)(*[t.data_ptr() for t in ss])
         barr = (_sz * n)(*[t.numel() * t.element_size() for t in ss])
         _check(_lib.fpo_h2d_copy(n, darr, sarr, barr, _stream(stream)), "fpo_h2d_copy")
