@@ -651,25 +651,36 @@ struct LayerSignalPtrs {
     void* out[kNrMaxLayers];
 };
 
-// Block-wide sums of N values (warp butterflies, then the warps' partials in order).
-template <int N, int THREADS>
-__device__ __forceinline__ void block_sum_n(float (&v)[N]) {
-    __shared__ float red[THREADS / 32][N];
+// Block-wide sums of five values (every thread gets them), with one barrier: `phase`
+// alternates between calls, so that the readers of one call need not be done before the
+// writers of the next.  The warp step halves the values with the lanes instead of running
+// five butterflies (8 shuffles, not 25); the warps' partials are added in order.
+template <int THREADS>
+__device__ __forceinline__ void block_sum5(float (&v)[5], int phase) {
+    constexpr int kW = THREADS / 32;
+    static_assert(kW == 8, "two 16-byte reads per value");
+    __shared__ __align__(16) float red[2][5][kW];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < N; ++i) v[i] = warp_sum(v[i]);
-    __syncthreads();  // the previous call's readers are done with red
-    if (lane == 0) {
-#pragma unroll
-        for (int i = 0; i < N; ++i) red[wid][i] = v[i];
-    }
+    const bool b16 = lane & 16, b8 = lane & 8, b4 = lane & 4;
+    auto both = [&](float lo, float hi, bool upper, int o) {
+        return (upper ? hi : lo) + __shfl_xor_sync(0xffffffffu, upper ? lo : hi, o);
+    };
+    const float a = both(v[0], v[1], b16, 16), b = both(v[2], v[3], b16, 16);
+    float c = v[4] + __shfl_xor_sync(0xffffffffu, v[4], 16);
+    const float d = both(a, b, b8, 8);
+    c += __shfl_xor_sync(0xffffffffu, c, 8);
+    float e = both(d, c, b4, 4);
+    e += __shfl_xor_sync(0xffffffffu, e, 2);
+    e += __shfl_xor_sync(0xffffffffu, e, 1);
+    // value 4 ended in lane 4, value 2 b8 + b16 in lanes 0, 16, 8, 24
+    if ((lane & 7) == 0) red[phase][(b16 ? 1 : 0) + (b8 ? 2 : 0)][wid] = e;
+    if (lane == 4) red[phase][4][wid] = e;
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < N; ++i) {
-        float t = 0.f;
-#pragma unroll
-        for (int w = 0; w < THREADS / 32; ++w) t += red[w][i];
-        v[i] = t;
+    for (int i = 0; i < 5; ++i) {
+        const float4 p = *reinterpret_cast<const float4*>(&red[phase][i][0]);
+        const float4 q = *reinterpret_cast<const float4*>(&red[phase][i][4]);
+        v[i] = ((p.x + p.y) + (p.z + p.w)) + ((q.x + q.y) + (q.z + q.w));
     }
 }
 
@@ -767,6 +778,17 @@ __global__ void __launch_bounds__(THREADS)
     uint4 gp[NV], gq[NV];  // the layer's norm weights, loaded once
     if constexpr (POST) ld_row_raw<NV, THREADS>(static_cast<const __nv_bfloat16*>(p.gp[l]), d, gp);
     if constexpr (PRE) ld_row_raw<NV, THREADS>(static_cast<const __nv_bfloat16*>(p.gq[l]), d, gq);
+    // with both norms they are held as fp32 (converting them again for every row was a
+    // third of the kernel's instructions, which bound it: 638 us of T 16384, d 4096, 8 layers)
+    float2 gpf[POST && PRE ? EPT / 2 : 1], gqf[POST && PRE ? EPT / 2 : 1];
+    if constexpr (POST && PRE) {
+#pragma unroll
+        for (int j = 0; j < EPT / 2; ++j) {
+            gpf[j] = bf16x2_at(gp[j / 4], j % 4);
+            gqf[j] = bf16x2_at(gq[j / 4], j % 4);
+        }
+    }
+    const float inv_min = 1.0f / min_rms;  // 1 / max(rho, min_rms) below the clamp
     const uint32_t sbase = smem_u32(sig_smem);
     const uint32_t row_bytes = static_cast<uint32_t>(d) * 2u;  // a multiple of 16
     auto stage_row = [&](int s, int t) { return sbase + static_cast<uint32_t>(s * NT + t) * row_bytes; };
@@ -821,7 +843,7 @@ __global__ void __launch_bounds__(THREADS)
             // Both stages from one block reduction: with a = gp (.) g and
             // u = (a - m inv1 kd1) pref1, the pre-MLP stage's sum <x, gq (.) u> is
             // pref1 (<x gq, a> - inv1 kd1 <x gq, m>), so all five sums are taken in one
-            // pass over the row (one barrier round per row instead of two).
+            // pass over the row (one barrier per row); a stays in u.
             float2 S[5];
 #pragma unroll
             for (int i = 0; i < 5; ++i) S[i] = make_float2(0.f, 0.f);
@@ -830,8 +852,10 @@ __global__ void __launch_bounds__(THREADS)
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const float2 m2 = bf16x2_at(mraw[v], k), x2 = bf16x2_at(xraw[v], k);
-                    const float2 a2 = __fmul2_rn(bf16x2_at(gp[v], k), bf16x2_at(graw[v], k));
-                    const float2 b2 = __fmul2_rn(x2, bf16x2_at(gq[v], k));
+                    const float2 a2 = __fmul2_rn(gpf[4 * v + k], bf16x2_at(graw[v], k));
+                    const float2 b2 = __fmul2_rn(x2, gqf[4 * v + k]);
+                    u[8 * v + 2 * k] = a2.x;
+                    u[8 * v + 2 * k + 1] = a2.y;
                     S[0] = __ffma2_rn(m2, m2, S[0]);
                     S[1] = __ffma2_rn(m2, a2, S[1]);
                     S[2] = __ffma2_rn(x2, x2, S[2]);
@@ -842,27 +866,33 @@ __global__ void __launch_bounds__(THREADS)
             float s5[5];
 #pragma unroll
             for (int i = 0; i < 5; ++i) s5[i] = S[i].x + S[i].y;
-            block_sum_n<5, THREADS>(s5);
-            const float r1 = sqrtf(s5[0] / static_cast<float>(d) + eps);
-            const float inv1 = 1.0f / r1;
+            block_sum5<THREADS>(s5, k_it & 1);
+            // rho, 1 / rho and the clamped prefactor of the post-FFN norm in the even lanes,
+            // of the pre-MLP one in the odd
+            const bool odd = threadIdx.x & 1;
+            const float r = sqrtf((odd ? s5[2] : s5[0]) / static_cast<float>(d) + eps);
+            const float inv = 1.0f / r;
+            const float pref = r >= min_rms ? inv : inv_min;
+            const float inv_o = __shfl_xor_sync(0xffffffffu, inv, 1);
+            const float pref_o = __shfl_xor_sync(0xffffffffu, pref, 1);
+            const float inv1 = odd ? inv_o : inv, inv2 = odd ? inv : inv_o;
+            const float pref1 = odd ? pref_o : pref, pref2 = odd ? pref : pref_o;
             const float kd1 = (s5[1] * inv1) / static_cast<float>(d);
-            const float pref1 = 1.0f / fmaxf(r1, min_rms);
-            const float r2 = sqrtf(s5[2] / static_cast<float>(d) + eps);
-            const float inv2 = 1.0f / r2;
             const float xu = pref1 * (s5[3] - (inv1 * kd1) * s5[4]);
             const float kd2 = (xu * inv2) / static_cast<float>(d);
-            const float pref2 = 1.0f / fmaxf(r2, min_rms);
-            // u = a pref1 - m (inv1 kd1 pref1);  out = (gq (.) u) pref2 - x (inv2 kd2 pref2)
-            const float2 P1 = make_float2(pref1, pref1), P2 = make_float2(pref2, pref2);
-            const float c1 = -(inv1 * kd1) * pref1, c2 = -(inv2 * kd2) * pref2;
-            const float2 C1 = make_float2(c1, c1), C2 = make_float2(c2, c2);
+            // u = a pref1 - m (inv1 kd1 pref1);  out = (gq (.) u) pref2 - x (inv2 kd2 pref2),
+            // with pref2 taken into the factors of a and m
+            const float p12 = pref1 * pref2, c12 = -((inv1 * kd1) * pref1) * pref2,
+                        c2 = -(inv2 * kd2) * pref2;
+            const float2 P = make_float2(p12, p12), C1 = make_float2(c12, c12),
+                         C2 = make_float2(c2, c2);
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const float2 a2 = __fmul2_rn(bf16x2_at(gp[v], k), bf16x2_at(graw[v], k));
-                    const float2 u2 = __ffma2_rn(a2, P1, __fmul2_rn(bf16x2_at(mraw[v], k), C1));
-                    const float2 o2 = __ffma2_rn(__fmul2_rn(bf16x2_at(gq[v], k), u2), P2,
+                    const float2 a2 = make_float2(u[8 * v + 2 * k], u[8 * v + 2 * k + 1]);
+                    const float2 u2 = __ffma2_rn(a2, P, __fmul2_rn(bf16x2_at(mraw[v], k), C1));
+                    const float2 o2 = __ffma2_rn(gqf[4 * v + k], u2,
                                                  __fmul2_rn(bf16x2_at(xraw[v], k), C2));
                     u[8 * v + 2 * k] = o2.x;
                     u[8 * v + 2 * k + 1] = o2.y;
