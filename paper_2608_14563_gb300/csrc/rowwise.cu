@@ -641,8 +641,6 @@ __global__ void wait_timeout_kernel(unsigned* status, unsigned long long limit_n
 //   out = (gq (.) u - xhat <xhat, gq (.) u> / d) / max(rho_x, rho_min)    (PRE)
 // Each stage's sums in fp32; u stays in registers (fp32) between the stages.  Grid x
 // runs over the layers, grid y over the rows.
-constexpr int kSigThreads = 256;  // block size of the block-per-row kernel (512: slower)
-
 struct LayerSignalPtrs {
     const void* m[kNrMaxLayers];
     const void* gp[kNrMaxLayers];
@@ -658,7 +656,7 @@ struct LayerSignalPtrs {
 template <int THREADS>
 __device__ __forceinline__ void block_sum5(float (&v)[5], int phase) {
     constexpr int kW = THREADS / 32;
-    static_assert(kW == 8, "two 16-byte reads per value");
+    static_assert(kW == 2 || kW == 4 || kW == 8, "8- or 16-byte reads of a value's partials");
     __shared__ __align__(16) float red[2][5][kW];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const bool b16 = lane & 16, b8 = lane & 8, b4 = lane & 4;
@@ -678,9 +676,17 @@ __device__ __forceinline__ void block_sum5(float (&v)[5], int phase) {
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        const float4 p = *reinterpret_cast<const float4*>(&red[phase][i][0]);
-        const float4 q = *reinterpret_cast<const float4*>(&red[phase][i][4]);
-        v[i] = ((p.x + p.y) + (p.z + p.w)) + ((q.x + q.y) + (q.z + q.w));
+        if constexpr (kW == 2) {
+            const float2 p = *reinterpret_cast<const float2*>(&red[phase][i][0]);
+            v[i] = p.x + p.y;
+        } else {
+            const float4 p = *reinterpret_cast<const float4*>(&red[phase][i][0]);
+            v[i] = (p.x + p.y) + (p.z + p.w);
+            if constexpr (kW == 8) {
+                const float4 q = *reinterpret_cast<const float4*>(&red[phase][i][4]);
+                v[i] += (q.x + q.y) + (q.z + q.w);
+            }
+        }
     }
 }
 
@@ -1160,16 +1166,16 @@ cudaError_t launch_wait_timeout(unsigned* status, uint64_t limit_ns, cudaStream_
 namespace {
 
 // The block-per-row kernel with its shared-memory size; the limit is raised once per
-// instantiation and device to the largest staging it can need (rows of EPT x kSigThreads
+// instantiation and device to the largest staging it can need (rows of EPT x THREADS
 // elements).
-template <int EPT, bool POST, bool PRE>
+template <int EPT, int THREADS, bool POST, bool PRE>
 cudaError_t launch_sig_rows(dim3 grid, size_t smem, cudaStream_t st, const __nv_bfloat16* g,
                             const LayerSignalPtrs& p, int T, int d, float eps, float min_rms) {
-    constexpr auto kern = layer_signal_row_kernel<EPT, kSigThreads, POST, PRE>;
+    constexpr auto kern = layer_signal_row_kernel<EPT, THREADS, POST, PRE>;
     constexpr int kNT = 1 + (POST ? 1 : 0) + (PRE ? 1 : 0);
-    const cudaError_t attr = set_smem_limit<kern>(kSigStages * kNT * EPT * kSigThreads * 2);
+    const cudaError_t attr = set_smem_limit<kern>(kSigStages * kNT * EPT * THREADS * 2);
     if (attr != cudaSuccess) return attr;
-    kern<<<grid, kSigThreads, smem, st>>>(g, p, T, d, eps, min_rms);
+    kern<<<grid, THREADS, smem, st>>>(g, p, T, d, eps, min_rms);
     return cudaSuccess;
 }
 
@@ -1179,25 +1185,30 @@ cudaError_t run_layer_signals(int dtype, int n_layers, const void* g, const Laye
     DevInfo di;
     const int sms = current_device_info(&di) ? di.sm_count : 148;
     const int per_layer = (sms * 8 + n_layers - 1) / n_layers;  // ~8 blocks per SM in all
-    // bf16 rows up to 32 x kSigThreads elements: block per row, the rows in registers
-    const int ept = dtype != 1             ? 0
-                    : d <= 8 * kSigThreads  ? 8
-                    : d <= 16 * kSigThreads ? 16
-                    : d <= 32 * kSigThreads ? 32
-                                            : 0;
-    if (ept) {
+    // bf16 rows up to 8192 elements: block per row, the rows in registers.  16 elements per
+    // thread keep what every thread does for itself (the norms' scalars) in proportion, so
+    // shorter rows take smaller blocks, and as many more of them (256 threads for any row
+    // up to 2048 left half or more of them idle: T 9000, d 1024, 9 layers, both norms 231 us,
+    // 84 us with 64).
+    if (dtype == 1 && d <= 8192) {
+        const int threads = d <= 1024 ? 64 : d <= 2048 ? 128 : 256;
+        const int blocks = per_layer * (256 / threads);
         const dim3 grid(static_cast<unsigned>(n_layers),
-                        static_cast<unsigned>(T < per_layer ? T : per_layer));
+                        static_cast<unsigned>(T < blocks ? T : blocks));
         const auto* gg = static_cast<const __nv_bfloat16*>(g);
         constexpr int kNT = 1 + (POST ? 1 : 0) + (PRE ? 1 : 0);
         const size_t smem = static_cast<size_t>(kSigStages) * kNT * d * 2;
         cudaError_t e = cudaSuccess;
-        if (ept == 8)
-            e = launch_sig_rows<8, POST, PRE>(grid, smem, st, gg, p, T, d, eps, min_rms);
-        else if (ept == 16)
-            e = launch_sig_rows<16, POST, PRE>(grid, smem, st, gg, p, T, d, eps, min_rms);
+        if (d <= 512)
+            e = launch_sig_rows<8, 64, POST, PRE>(grid, smem, st, gg, p, T, d, eps, min_rms);
+        else if (d <= 1024)
+            e = launch_sig_rows<16, 64, POST, PRE>(grid, smem, st, gg, p, T, d, eps, min_rms);
+        else if (d <= 2048)
+            e = launch_sig_rows<16, 128, POST, PRE>(grid, smem, st, gg, p, T, d, eps, min_rms);
+        else if (d <= 4096)
+            e = launch_sig_rows<16, 256, POST, PRE>(grid, smem, st, gg, p, T, d, eps, min_rms);
         else
-            e = launch_sig_rows<32, POST, PRE>(grid, smem, st, gg, p, T, d, eps, min_rms);
+            e = launch_sig_rows<32, 256, POST, PRE>(grid, smem, st, gg, p, T, d, eps, min_rms);
         if (e != cudaSuccess) return e;
     } else {
         const int wpb = kRowThreads / 32;

@@ -187,3 +187,19 @@ def test_layer_signals_full_size_sampled_rows(fpo, post):
         got = f64(outs[l][rows])
         for r in range(len(rows)):
             assert rel_frob(got[r], ref[r]) < 2e-2
+
+
+@pytest.mark.parametrize("d", [8, 504, 512, 1024, 1032, 2048, 2056, 4104])
+@pytest.mark.parametrize("min_rms", [0.5, 0.0])
+def test_block_per_row_widths(fpo, d, min_rms):
+    """bf16 rows around the widths where the block size or the elements per thread change
+    (512, 1024, 2048, 4096), with more rows than one wave of blocks and without the clamp."""
+    wl = Workload("sigw", T=2600 if d < 600 else 260, d=d, d_ff=8, V=8, layers=2)
+    g, m, gp, x, gq = _case(wl, 2)
+    for mode, (post, pre) in MODES.items():
+        outs = _run(fpo, g, m, gp, x, gq, post, pre, min_rms=min_rms)
+        for l in range(2):
+            ref = _ref(g, m, gp, x, gq, post, pre, l, min_rms=min_rms)
+            row = np.linalg.norm(f64(outs[l]) - ref, axis=1) / np.linalg.norm(ref, axis=1)
+            # bf16 results of fp32 arithmetic: half an ulp (2^-9) per element
+            assert np.max(row) < 2.0 ** -8, (mode, l, int(np.argmax(row)))
