@@ -353,6 +353,17 @@ std::atomic<int> g_gemm_variant{2};
 std::atomic<int> g_band_override{0};  // > 0: rasterisation band height (tests / tuning)
 
 bool use_pair() { return g_gemm_variant.load(std::memory_order_relaxed) >= 1; }
+
+// Whether the GEMMs over the vocabulary of a chunk of T tokens run on CTA pairs: not, by
+// default, when an odd number of 128-row blocks, at most 5, leaves half of a pair's 256 rows
+// empty.  The single-CTA kernel is 10-25% slower per row but wastes at most 127 of them.
+// Logits pass, d 4096, V 100352, pair against single: T 128 167 and 145 us, 333 251 and
+// 224, 600 347 and 333 (seven blocks, T 900, V 50304: 237 and 268).  Same sums either way.
+bool use_pair_rows(int T) {
+    const int blocks = (T + kBM - 1) / kBM;
+    return use_pair() &&
+           !(g_gemm_variant.load(std::memory_order_relaxed) == 2 && blocks % 2 == 1 && blocks <= 5);
+}
 bool wide_proj() { return g_gemm_variant.load(std::memory_order_relaxed) >= 2; }
 
 // Rasterisation band in tile rows, unless overridden: 16 tile rows, i.e. 2048
@@ -396,8 +407,8 @@ int proj_clusters() {
 // that costs least.  Measured, in ns: a 64-deep k-block 344 (at the clock the tensor cores
 // hold under load), with a split the fixup's launch 4000 and its read of the fp32 parts
 // 4.3 bytes a ns.  Ranges have at least 32 k-blocks, and the units fit the scratch.  T is
-// the whole batch, not a token chunk, so that the sums do not depend on the chunking.
-// Projection with its fixup, T x d x V: 333 x 4096 x 100352 (16 tiles of 512 columns on 76
+// the whole batch where that is small, so that its sums do not depend on the chunking, and
+// otherwise the chunk (the last one of T 9000 has 808 tokens).  Projection with its fixup, T x d x V: 333 x 4096 x 100352 (16 tiles of 512 columns on 76
 // clusters) 887 us whole, 246 us in 7 ranges; 2048 x 2048 x 50304 (32 tiles) 434 and 276.
 int proj_split(int T, int d, int V) {
     const long long clusters = proj_clusters();
@@ -435,7 +446,7 @@ int lse_tile_n_bf16() { return kLseBN; }
 cudaError_t launch_lse_partial_bf16(const void* yhat, const void* W_U, const int32_t* y, int T,
                                     int d, int V, float2* part, int part_ld, float* zy, float* z,
                                     unsigned* status, cudaStream_t st) {
-    const bool pair = use_pair();
+    const bool pair = use_pair_rows(T);
     GemmMaps<1> maps;
     if (!map_kmajor(&maps.a[0], yhat, T, d, kBM) ||
         !map_kmajor(&maps.b[0], W_U, V, d, pair ? kLseBN / 2 : kLseBN))
@@ -472,7 +483,7 @@ cudaError_t launch_lse_partial_bf16(const void* yhat, const void* W_U, const int
 cudaError_t launch_error_bf16(const void* yhat, const void* W_U, const int32_t* y, const float* lse,
                               int Tc, int d, int V, float s, void* E, unsigned* status,
                               cudaStream_t st) {
-    const bool pair = use_pair();
+    const bool pair = use_pair_rows(Tc);
     GemmMaps<1> maps;
     if (!map_kmajor(&maps.a[0], yhat, Tc, d, kBM) ||
         !map_kmajor(&maps.b[0], W_U, V, d, pair ? kLseBN / 2 : kLseBN))
@@ -495,7 +506,7 @@ cudaError_t launch_anchor_prob_bf16(const void* yhat, const void* W_U, const int
                                     const float* anchor, int T, int d, int V, float* su, float* sx,
                                     float* qz, int part_ld, void* P, unsigned* status,
                                     cudaStream_t st) {
-    const bool pair = use_pair();
+    const bool pair = use_pair_rows(T);
     GemmMaps<1> maps;
     if (!map_kmajor(&maps.a[0], yhat, T, d, kBM) ||
         !map_kmajor(&maps.b[0], W_U, V, d, pair ? kLseBN / 2 : kLseBN))
@@ -584,7 +595,8 @@ cudaError_t launch_proj_vjp_bf16(const void* P, const void* W_U, const int32_t* 
     ep.N = d;
     if (wide_proj()) {
         SkPlan plan;
-        const int split = proj_split(T_all, d, V);
+        int split = proj_split(T_all, d, V);
+        if (split == 0) split = proj_split(Tc, d, V);  // a short chunk of a large batch
         if (split == 0) {
             ep.tile_n = kWideBN;
             const GemmShape sh = make_shape(Tc, d, V, kWideBN, 1, band_for(true), kPairBM);
@@ -619,7 +631,8 @@ cudaError_t launch_proj_bf16(const void* E, const void* W_U, int Tc, int T_all, 
     ep.N = d;
     if (wide_proj()) {
         SkPlan plan;
-        const int split = proj_split(T_all, d, V);
+        int split = proj_split(T_all, d, V);
+        if (split == 0) split = proj_split(Tc, d, V);  // a short chunk of a large batch
         if (split == 0) {
             const GemmShape sh = make_shape(Tc, d, V, kWideBN, 1, band_for(true), kPairBM);
             const cudaError_t e = run_gemm_pair<kWideBN, false, true, kWideStages, 1, EpiStoreF32>(

@@ -97,7 +97,7 @@ cudaError_t launch_error_bf16(const void* yhat, const void* W_U, const int32_t* 
                               cudaStream_t st);
 
 // Projection: g[Tc, d] = E[Tc, V] W_U (fp32 out).  T_all: the rows of the whole batch (the
-// split of K is chosen from it, whatever the chunking).  sk_scratch:
+// split of K is chosen from it when it is small, whatever the chunking).  sk_scratch:
 // proj_sk_scratch_bytes() of device memory for the fp32 parts of split tiles.
 cudaError_t launch_proj_bf16(const void* E, const void* W_U, int Tc, int T_all, int d, int V,
                              float* g, float* sk_scratch, unsigned* status, cudaStream_t st);

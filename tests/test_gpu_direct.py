@@ -308,3 +308,24 @@ def test_projection_of_a_small_batch_split_over_k(fpo, algo, shape):
     assert rel_frob(g, whole) < np.sqrt(V / 16 * 2.0 ** -24 * 2.0 ** -8)
     ref = reference(h, w, W_U, y, eps=wl.eps, s=wl.loss_scale)
     assert rel_frob(g, ref["g_tilde"]) < TOL and cos(g, ref["g_tilde"]) >= COS_MIN
+
+
+@pytest.mark.parametrize("T", [1, 127, 128, 129, 257, 384, 385, 513, 640, 641])
+def test_logits_kernel_by_row_blocks(fpo, T):
+    """Batches of an odd number (at most 5) of 128-row blocks run the logits pass on single
+    CTAs, the others on CTA pairs: the same bits as either kernel throughout, around every
+    change of the rule."""
+    wl = Workload("rows", T=T, d=136, d_ff=8, V=520, layers=1, targets="zipf")
+    inp = synth.make_all(wl)
+    prev = fpo.set_gemm_variant(2)
+    outs = []
+    try:
+        for v in (2, 1, 0):
+            fpo.set_gemm_variant(v)
+            outs.append(run(fpo, inp["h"], inp["w"], inp["W_U"], inp["y"], eps=wl.eps,
+                            algo=fpo.ES_DIRECT))
+    finally:
+        fpo.set_gemm_variant(prev)
+    for o in outs[1:]:
+        for k in ("g", "lse", "loss"):
+            assert torch.equal(outs[0][k], o[k]), k
