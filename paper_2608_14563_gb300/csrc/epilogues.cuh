@@ -11,8 +11,8 @@
 // Epilogues that read or update matrices of the output's shape (the update, the
 // optimizer's first pass, the cosine, the gate / up signals, plain G) have 8 warps
 // (Epi::kWarps) and the form of epilogue_tile's second half: a chunk is staged in shared
-// memory and each lane takes 4 columns of 8 rows, so that every global access of a warp
-// covers whole row segments, and the operands of the next chunk (of the first chunk:
+// memory and each lane takes 4 columns of 8 of its rows, so that every global access of a
+// warp covers 256 bytes of two rows, and the operands of the next chunk (of the first chunk:
 // while the mainloop runs) are loaded ahead.  One row per
 // thread, as these epilogues had it with 4 warps, made every 16-byte access of a warp
 // touch 32 rows and kept 16 KB in flight per SM: AdamW with the step clip at T 4096,
@@ -521,31 +521,35 @@ struct EpiProjVjp {
     __device__ __forceinline__ void finish(const Params&, int) {}
 };
 
-// A lane's place in a warp's 32 rows of an 8-warp epilogue: its columns
-// 4 (lane mod kLanes) .. of every kRows-th row from lane / kLanes, as element offsets into
-// matrices of row stride ld.
-struct QuadPos {
-    using Q = QuadChunk;
-    long long off;    // of the lane's first element
-    int rows, cols;   // rows from its first row, columns from its first column, in the matrix
+// A lane's place in a warp's 32 rows x 128 columns of an 8-warp epilogue: the 4 columns of
+// access i of chunk c (numbered j = kAcc c + i over the whole block), as element offsets
+// into matrices of row stride ld.
+struct RowPos {
+    using R = RowChunk;
+    long long off;    // of the lane's columns in its first row
+    int rows, cols;   // rows from the lane's first, columns from its first, inside
 
-    __device__ __forceinline__ QuadPos(int M, int N, long long ld, int row0, int n0, int lane) {
-        const int r = row0 + lane / Q::kLanes, c = n0 + 4 * (lane % Q::kLanes);
+    __device__ __forceinline__ RowPos(int M, int N, long long ld, int row0, int n0, int lane) {
+        const int r = row0 + lane / R::kLanes, c = n0 + 4 * (lane % R::kLanes);
         off = r * ld + c;
         rows = M - r;
         cols = N - c;
     }
-    // Quad i of the lane (kRows i rows below its first) and column offset co are inside
-    // (N is a multiple of 8, so the 4 columns are inside together).
-    __device__ __forceinline__ bool in(int i, int co) const { return Q::kRows * i < rows && co < cols; }
-    __device__ __forceinline__ long long at(long long ld, int i, int co) const {
-        return off + Q::kRows * i * ld + co;
+    static __device__ __forceinline__ int row(int j) {
+        return j / R::kAcc / R::kColGroups * R::kRows + j % R::kAcc * R::kAccRows;
+    }
+    static __device__ __forceinline__ int col(int j) { return j / R::kAcc % R::kColGroups * R::kCols; }
+    // Access j is inside the matrix (N is a multiple of 8, so its 4 columns are inside
+    // together).
+    __device__ __forceinline__ bool in(int j) const { return row(j) < rows && col(j) < cols; }
+    __device__ __forceinline__ long long at(long long ld, int j) const {
+        return off + row(j) * ld + col(j);
     }
     // That element of a matrix m, or m itself outside the matrix: always readable, so that
     // a batch of loads has no branches between them.
     template <typename TT>
-    __device__ __forceinline__ const TT* src(const TT* m, long long ld, int i, int co) const {
-        return in(i, co) ? m + at(ld, i, co) : m;
+    __device__ __forceinline__ const TT* src(const TT* m, long long ld, int j) const {
+        return in(j) ? m + at(ld, j) : m;
     }
 };
 
@@ -553,17 +557,19 @@ struct QuadPos {
 // nothing that waits between its loads: loads issued one by one between the uses of the
 // batch before shared the warp's few scoreboards with it, and each use waited for the
 // newest load (the update of T 512, d 2048, d_ff 8264, 4 layers: 278 us, 230 of them with
-// the loads alone, 115 without; 200 us with batches.  Two batches in flight gave nothing
-// more, nor did 16 warps, L2 prefetches of the next tile or streaming cache hints).
-
+// the loads alone, 115 without; 195 us with batches, and 176 with 256 bytes of two rows per
+// access (kRows 16) instead of 128 bytes of four (kRows 32).  512 bytes of one row (kRows 8)
+// gave 162 but cost 2% of a T 200 step, as every lane reads the accumulator once per row
+// group.  Two batches in flight gave nothing more, nor did 16 warps, L2 prefetches of the
+// next tile or streaming cache hints).
 // Slots of per-warp partial sums per (256-row block, 256-column tile): 8 blocks of 32 rows
 // times the two column halves.
 constexpr int kColSlots = 16;
 
-__device__ __forceinline__ long long quad_slot(int g, int m256, int n_blocks, int nb, int row0,
+__device__ __forceinline__ long long slot_of(int g, int m256, int n_blocks, int nb, int row0,
                                                int n0) {
     return ((static_cast<long long>(g) * m256 + row0 / 256) * n_blocks + nb) * kColSlots +
-           ((n0 % 256) / QuadChunk::kTileCols) * 8 + (row0 % 256) / 32;
+           ((n0 % 256) / RowChunk::kTileCols) * 8 + (row0 % 256) / 32;
 }
 
 __device__ __forceinline__ float warp_sum_f32(float x) {
@@ -586,18 +592,18 @@ struct EpiUpdate {
         int M, N;
         float neg_lr;
     };
-    using Q = QuadChunk;
-    QuadPos pos;
+    using R = RowChunk;
+    RowPos pos;
     float* wm;
     __nv_bfloat16* wo;
     __nv_bfloat16* go;
-    float4 w[Q::kQuads];  // master values of the next chunk
+    float4 w[R::kAcc];  // master values of the next chunk
 
-    __device__ __forceinline__ void load(const Params& p, int co) {
+    __device__ __forceinline__ void load(const Params& p, int c) {
         if (!wm) return;
 #pragma unroll
-        for (int i = 0; i < Q::kQuads; ++i)
-            w[i] = *reinterpret_cast<const float4*>(pos.src(wm, p.ld, i, co));
+        for (int i = 0; i < R::kAcc; ++i)
+            w[i] = *reinterpret_cast<const float4*>(pos.src(wm, p.ld, R::kAcc * c + i));
     }
 
     __device__ __forceinline__ EpiUpdate(const Params& p, int g, int row0, int n0, int lane)
@@ -608,12 +614,12 @@ struct EpiUpdate {
         load(p, 0);
     }
 
-    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co) {
+    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int c) {
 #pragma unroll
-        for (int i = 0; i < Q::kQuads; ++i) {
-            const float4 v = Q::read(buf, lane, i);
-            const long long o = pos.at(p.ld, i, co);
-            const bool in = pos.in(i, co);
+        for (int i = 0; i < R::kAcc; ++i) {
+            const float4 v = R::read(buf, lane, i);
+            const long long o = pos.at(p.ld, R::kAcc * c + i);
+            const bool in = pos.in(R::kAcc * c + i);
             if (wm) {
                 float4 a = w[i];
                 a.x = fmaf(p.neg_lr, v.x, a.x);
@@ -631,7 +637,7 @@ struct EpiUpdate {
                 *reinterpret_cast<uint2*>(go + o) =
                     make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
         }
-        if (co + Q::kCols < Q::kTileCols) load(p, co + Q::kCols);
+        if (c + 1 < R::kChunks) load(p, c + 1);
     }
 
     __device__ __forceinline__ void finish(const Params&, int, int) {}
@@ -641,7 +647,7 @@ struct EpiUpdate {
 // Pseudogradients with the layer-viability diagnostic's cosine (Sec. 2.2 Eq. (cosine),
 // Eq. (w3update)): for group (layer) g, G_out[g] = bf16(G), and the three sums of the
 // cosine of that stored G against Y[g] (<G, Y>, ||G||^2, ||Y||^2) over the warp's 32 rows
-// x 128 columns (fp32 per lane, then a fixed butterfly), one triple per quad_slot, so the
+// x 128 columns (fp32 per lane, then a fixed butterfly), one triple per slot_of, so the
 // cosine needs no second pass over G.
 struct EpiGradCos {
     static constexpr int kWarps = 8;
@@ -653,16 +659,16 @@ struct EpiGradCos {
         int M, N;
         int m256, n_blocks;
     };
-    using Q = QuadChunk;
-    QuadPos pos;
+    using R = RowChunk;
+    RowPos pos;
     int g, row0, n0;
     float2 s_gy, s_gg, s_yy;
-    uint2 y[Q::kQuads];  // Y of the next chunk
+    uint2 y[R::kAcc];  // Y of the next chunk
 
-    __device__ __forceinline__ void load(const Params& p, int co) {
+    __device__ __forceinline__ void load(const Params& p, int c) {
 #pragma unroll
-        for (int i = 0; i < Q::kQuads; ++i)
-            y[i] = __ldg(reinterpret_cast<const uint2*>(pos.src(p.Y[g], p.ld, i, co)));
+        for (int i = 0; i < R::kAcc; ++i)
+            y[i] = __ldg(reinterpret_cast<const uint2*>(pos.src(p.Y[g], p.ld, R::kAcc * c + i)));
     }
 
     __device__ __forceinline__ EpiGradCos(const Params& p, int g_, int row0_, int n0_, int lane)
@@ -671,15 +677,15 @@ struct EpiGradCos {
         load(p, 0);
     }
 
-    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co) {
+    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int c) {
 #pragma unroll
-        for (int i = 0; i < Q::kQuads; ++i) {
-            const float4 v = Q::read(buf, lane, i);
+        for (int i = 0; i < R::kAcc; ++i) {
+            const float4 v = R::read(buf, lane, i);
             const uint32_t pk[2] = {pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w)};
-            if (!pos.in(i, co)) continue;
+            if (!pos.in(R::kAcc * c + i)) continue;
             const uint2 yv = y[i];
             const uint32_t yk[2] = {yv.x, yv.y};
-            *reinterpret_cast<uint2*>(p.G_out[g] + pos.at(p.ld, i, co)) =
+            *reinterpret_cast<uint2*>(p.G_out[g] + pos.at(p.ld, R::kAcc * c + i)) =
                 make_uint2(pk[0], pk[1]);
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
@@ -692,14 +698,14 @@ struct EpiGradCos {
                 s_yy = __ffma2_rn(yr, yr, s_yy);
             }
         }
-        if (co + Q::kCols < Q::kTileCols) load(p, co + Q::kCols);
+        if (c + 1 < R::kChunks) load(p, c + 1);
     }
 
     __device__ __forceinline__ void finish(const Params& p, int nb, int lane) {
         const float gy = warp_sum_f32(s_gy.x + s_gy.y), gg = warp_sum_f32(s_gg.x + s_gg.y),
                     yy = warp_sum_f32(s_yy.x + s_yy.y);
         if (lane == 0) {
-            float* o = p.part + quad_slot(g, p.m256, p.n_blocks, nb, row0, n0) * 3;
+            float* o = p.part + slot_of(g, p.m256, p.n_blocks, nb, row0, n0) * 3;
             o[0] = gy;
             o[1] = gg;
             o[2] = yy;
@@ -711,7 +717,7 @@ struct EpiGradCos {
 // Pseudogradient only, fp32, one output per group (layer): G[g] = g~^T A_l, for
 // the optimizers that need the whole G before they step.  With W_master set (the relative
 // clip on the gradient) also ||W||^2 and ||G||^2 of the warp's 32 rows x 128 columns, one
-// pair per quad_slot, so that the clip factor needs no pass over W and G of its own
+// pair per slot_of, so that the clip factor needs no pass over W and G of its own
 // (448 us of 1823 for 3 layers of 3072 x 23040).
 struct EpiStoreGroupF32 {
     static constexpr int kWarps = 8;
@@ -723,19 +729,19 @@ struct EpiStoreGroupF32 {
         int M, N;
         int m256, n_blocks;
     };
-    using Q = QuadChunk;
-    QuadPos pos;
+    using R = RowChunk;
+    RowPos pos;
     int g, row0, n0;
     float* G;
     const float* wm;
     float s_ww, s_gg;
-    float4 w[Q::kQuads];  // master values of the next chunk
+    float4 w[R::kAcc];  // master values of the next chunk
 
-    __device__ __forceinline__ void load(const Params& p, int co) {
+    __device__ __forceinline__ void load(const Params& p, int c) {
         if (!wm) return;
 #pragma unroll
-        for (int i = 0; i < Q::kQuads; ++i)
-            w[i] = *reinterpret_cast<const float4*>(pos.src(wm, p.ld, i, co));
+        for (int i = 0; i < R::kAcc; ++i)
+            w[i] = *reinterpret_cast<const float4*>(pos.src(wm, p.ld, R::kAcc * c + i));
     }
 
     __device__ __forceinline__ EpiStoreGroupF32(const Params& p, int g_, int row0_, int n0_,
@@ -745,26 +751,26 @@ struct EpiStoreGroupF32 {
         load(p, 0);
     }
 
-    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co) {
+    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int c) {
 #pragma unroll
-        for (int i = 0; i < Q::kQuads; ++i) {
-            const float4 v = Q::read(buf, lane, i);
-            if (!pos.in(i, co)) continue;
-            *reinterpret_cast<float4*>(G + pos.at(p.ld, i, co)) = v;
+        for (int i = 0; i < R::kAcc; ++i) {
+            const float4 v = R::read(buf, lane, i);
+            if (!pos.in(R::kAcc * c + i)) continue;
+            *reinterpret_cast<float4*>(G + pos.at(p.ld, R::kAcc * c + i)) = v;
             if (wm) {
                 s_gg = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, s_gg))));
                 s_ww = fmaf(w[i].x, w[i].x,
                             fmaf(w[i].y, w[i].y, fmaf(w[i].z, w[i].z, fmaf(w[i].w, w[i].w, s_ww))));
             }
         }
-        if (co + Q::kCols < Q::kTileCols) load(p, co + Q::kCols);
+        if (c + 1 < R::kChunks) load(p, c + 1);
     }
 
     __device__ __forceinline__ void finish(const Params& p, int nb, int lane) {
         if (!wm) return;
         const float ww = warp_sum_f32(s_ww), gg = warp_sum_f32(s_gg);
         if (lane == 0) {
-            float* o = p.part + quad_slot(g, p.m256, p.n_blocks, nb, row0, n0) * 2;
+            float* o = p.part + slot_of(g, p.m256, p.n_blocks, nb, row0, n0) * 2;
             o[0] = ww;
             o[1] = gg;
         }
@@ -777,14 +783,15 @@ struct EpiStoreGroupF32 {
 // ||dW|| <= clip_frac ||W||).  With G from the accumulator, each element's optimizer state
 // advances and its unclipped step d = opt_step(G, W, s1, s2) is stored (fp32, D[g], null
 // for momentum, whose step -lr s1 the state holds; the state sees the unclipped gradient), and ||W||^2, ||d||^2 of the warp's 32 rows x 128
-// columns are written as one pair per quad_slot; a kernel then scales each layer's steps
+// columns are written as one pair per slot_of; a kernel then scales each layer's steps
 // by min(1, clip_frac ||W|| / ||d||) and applies them (W is not written here, so its norm
 // is the pre-step one).  Without a clip the stand-alone passes are used: taking the whole
 // step here made the update faster but the power-capped step slower (its epilogue then
 // held the tensor pipe back at full draw).
-// The operands of the next 4 quads are loaded as each quad is done: its arithmetic hides
-// the wait that the batches of the other epilogues avoid (2362 us; batches of a whole or
-// half a chunk 3006 and 2500, 2 quads ahead 2561, 8 ahead 2840, 16 warps 2990).
+// The operands of the access 4 ahead are loaded as each one is done: its arithmetic hides the
+// wait that the batches of the other epilogues avoid (T 4096, d 4096, d_ff 11008, 8 layers,
+// AdamW, with 4 rows x 128 bytes per access: 2362 us; batches of a whole or half a chunk
+// 3006 and 2500, 2 ahead 2561, 8 ahead 2840, 16 warps 2990).
 struct EpiOptStep {
     static constexpr int kWarps = 8;
     struct Params {
@@ -798,21 +805,21 @@ struct EpiOptStep {
         int M, N;
         int m256, n_blocks;
     };
-    using Q = QuadChunk;
+    using R = RowChunk;
     static constexpr int kAhead = 4;
-    QuadPos pos;
+    RowPos pos;
     int g, row0, n0;
     const float* wm;
     float* p1;
     float* p2;
     float* D;
     float s_ww, s_dd;
-    float4 w[kAhead], a[kAhead], b[kAhead];  // of the next kAhead quads
+    float4 w[kAhead], a[kAhead], b[kAhead];  // of the next kAhead accesses
 
-    __device__ __forceinline__ void load(const Params& p, int k, int i, int co) {
+    __device__ __forceinline__ void load(const Params& p, int k, int j) {
         w[k] = a[k] = b[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (!pos.in(i, co)) return;
-        const long long o = pos.at(p.ld, i, co);
+        if (!pos.in(j)) return;
+        const long long o = pos.at(p.ld, j);
         w[k] = *reinterpret_cast<const float4*>(wm + o);
         if (p1) a[k] = *reinterpret_cast<const float4*>(p1 + o);
         if (p2) b[k] = *reinterpret_cast<const float4*>(p2 + o);
@@ -825,22 +832,22 @@ struct EpiOptStep {
         p2 = p.s2[g_];
         D = p.D[g_];
 #pragma unroll
-        for (int k = 0; k < kAhead; ++k) load(p, k, k, 0);
+        for (int k = 0; k < kAhead; ++k) load(p, k, k);
     }
 
-    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co) {
+    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int c) {
 #pragma unroll 1
-        for (int h = 0; h < Q::kQuads; h += kAhead) {
+        for (int h = 0; h < R::kAcc; h += kAhead) {
 #pragma unroll
             for (int k = 0; k < kAhead; ++k) {
                 const int i = h + k;
-                const float4 v4 = Q::read(buf, lane, i);
+                const float4 v4 = R::read(buf, lane, i);
                 const float v[4] = {v4.x, v4.y, v4.z, v4.w};
                 const float wv[4] = {w[k].x, w[k].y, w[k].z, w[k].w};
                 float av[4] = {a[k].x, a[k].y, a[k].z, a[k].w};
                 float bv[4] = {b[k].x, b[k].y, b[k].z, b[k].w};
                 float out[4];
-                const bool in = pos.in(i, co);
+                const bool in = pos.in(R::kAcc * c + i);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     out[e] = opt_step(p.op, v[e], wv[e], av[e], bv[e]);
@@ -850,17 +857,14 @@ struct EpiOptStep {
                     }
                 }
                 if (in) {
-                    const long long o = pos.at(p.ld, i, co);
+                    const long long o = pos.at(p.ld, R::kAcc * c + i);
                     if (D)
                         *reinterpret_cast<float4*>(D + o) =
                             make_float4(out[0], out[1], out[2], out[3]);
                     if (p1) *reinterpret_cast<float4*>(p1 + o) = make_float4(av[0], av[1], av[2], av[3]);
                     if (p2) *reinterpret_cast<float4*>(p2 + o) = make_float4(bv[0], bv[1], bv[2], bv[3]);
                 }
-                if (i + kAhead < Q::kQuads)
-                    load(p, k, i + kAhead, co);
-                else if (co + Q::kCols < Q::kTileCols)
-                    load(p, k, i + kAhead - Q::kQuads, co + Q::kCols);
+                if (R::kAcc * c + i + kAhead < R::kAcc * R::kChunks) load(p, k, R::kAcc * c + i + kAhead);
             }
         }
     }
@@ -868,7 +872,7 @@ struct EpiOptStep {
     __device__ __forceinline__ void finish(const Params& p, int nb, int lane) {
         const float ww = warp_sum_f32(s_ww), dd = warp_sum_f32(s_dd);
         if (lane == 0) {
-            float* o = p.part + quad_slot(g, p.m256, p.n_blocks, nb, row0, n0) * 2;
+            float* o = p.part + slot_of(g, p.m256, p.n_blocks, nb, row0, n0) * 2;
             o[0] = ww;
             o[1] = dd;
         }
@@ -889,15 +893,15 @@ struct EpiSwiglu {
         long long ld;
         int M, N;
     };
-    using Q = QuadChunk;
-    QuadPos pos;
-    uint2 ua[Q::kQuads], ub[Q::kQuads];  // a and b of the next chunk
+    using R = RowChunk;
+    RowPos pos;
+    uint2 ua[R::kAcc], ub[R::kAcc];  // a and b of the next chunk
 
-    __device__ __forceinline__ void load(const Params& p, int co) {
+    __device__ __forceinline__ void load(const Params& p, int c) {
 #pragma unroll
-        for (int i = 0; i < Q::kQuads; ++i) {
-            ua[i] = *reinterpret_cast<const uint2*>(pos.src(p.a, p.ld, i, co));
-            ub[i] = *reinterpret_cast<const uint2*>(pos.src(p.b, p.ld, i, co));
+        for (int i = 0; i < R::kAcc; ++i) {
+            ua[i] = *reinterpret_cast<const uint2*>(pos.src(p.a, p.ld, R::kAcc * c + i));
+            ub[i] = *reinterpret_cast<const uint2*>(pos.src(p.b, p.ld, R::kAcc * c + i));
         }
     }
 
@@ -906,10 +910,10 @@ struct EpiSwiglu {
         load(p, 0);
     }
 
-    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int co) {
+    __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int c) {
 #pragma unroll
-        for (int i = 0; i < Q::kQuads; ++i) {
-            const float4 v4 = Q::read(buf, lane, i);
+        for (int i = 0; i < R::kAcc; ++i) {
+            const float4 v4 = R::read(buf, lane, i);
             const float v[4] = {v4.x, v4.y, v4.z, v4.w};
             const uint2 a2 = ua[i], b2 = ub[i];
             const float xa[4] = {__uint_as_float(a2.x << 16), __uint_as_float(a2.x & 0xffff0000u),
@@ -927,15 +931,15 @@ struct EpiSwiglu {
                 da[k] = v[k] * xb[k] * sg * fmaf(x, 1.f - sg, 1.f);
                 db[k] = v[k] * x * sg;
             }
-            if (pos.in(i, co)) {
-                const long long o = pos.at(p.ld, i, co);
+            if (pos.in(R::kAcc * c + i)) {
+                const long long o = pos.at(p.ld, R::kAcc * c + i);
                 *reinterpret_cast<uint2*>(p.dA + o) =
                     make_uint2(pack_bf16x2(da[0], da[1]), pack_bf16x2(da[2], da[3]));
                 *reinterpret_cast<uint2*>(p.dB + o) =
                     make_uint2(pack_bf16x2(db[0], db[1]), pack_bf16x2(db[2], db[3]));
             }
         }
-        if (co + Q::kCols < Q::kTileCols) load(p, co + Q::kCols);
+        if (c + 1 < R::kChunks) load(p, c + 1);
     }
 
     __device__ __forceinline__ void finish(const Params&, int, int) {}

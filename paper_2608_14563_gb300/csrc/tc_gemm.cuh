@@ -149,21 +149,41 @@ __device__ __forceinline__ void out_stage_row(uint32_t buf, int r, const uint32_
                      w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
 }
 
-// Chunks of the 8-warp epilogues: 32 rows x 32 fp32 columns, staged in the warp's 4 KB of
-// output staging with one row per lane and read back with 8 lanes to a row, 4 columns each,
-// so that a warp's global accesses cover whole row segments.  16-byte pieces are swizzled
-// (out_stage_row), so neither side has bank conflicts.
-struct QuadChunk {
-    static constexpr int kCols = 32;
-    static constexpr int kLanes = 8;        // lanes sharing a row
-    static constexpr int kRows = 4;         // rows of one access of the warp
-    static constexpr int kQuads = 8;        // accesses per chunk
-    static constexpr int kTileCols = 128;   // of a 256-column tile, per warp
+// Chunks of the 8-warp epilogues: kRows of the warp's 32 rows x kCols of its 128 fp32
+// columns, staged in the warp's 4 KB of output staging by the lanes that hold the rows and
+// read back with kLanes lanes to a row, 4 columns each, so that every global access of a
+// warp covers kCols consecutive columns of kAccRows rows.  16-byte pieces are swizzled by
+// row, so neither side has bank conflicts.
+struct RowChunk {
+    static constexpr int kRows = 16;
+    static constexpr int kCols = 1024 / kRows;
+    static constexpr int kLanes = kCols / 4;
+    static constexpr int kAccRows = 32 / kLanes;           // rows of one access
+    static constexpr int kAcc = kRows / kAccRows;          // accesses per chunk (8)
+    static constexpr int kTileCols = 128;                  // of a 256-column tile, per warp
+    static constexpr int kColGroups = kTileCols / kCols;
+    static constexpr int kChunks = 32 / kRows * kColGroups;
 
-    // Columns 4 (lane mod kLanes) .. of row kRows i + lane / kLanes, i in [0, kQuads).
+    static __device__ __forceinline__ uint32_t piece(uint32_t buf, uint32_t r, uint32_t c) {
+        return buf + r * (kCols * 4u) + ((c ^ (r & 7u)) << 4);
+    }
+    // Columns [32 h, 32 h + 32) of the chunk's, one row per lane; the rows of row group rg
+    // go to the staging buffer.
+    static __device__ __forceinline__ void stage(uint32_t buf, int lane, int rg, int h,
+                                                 const float (&v)[32]) {
+        if (lane / kRows != rg) return;
+        const uint32_t r = static_cast<uint32_t>(lane % kRows);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            st_shared_v4(piece(buf, r, static_cast<uint32_t>(8 * h + k)),
+                         __float_as_uint(v[4 * k]), __float_as_uint(v[4 * k + 1]),
+                         __float_as_uint(v[4 * k + 2]), __float_as_uint(v[4 * k + 3]));
+    }
+    // Access i of the staged chunk: row kAccRows i + lane / kLanes, columns
+    // 4 (lane mod kLanes) .. of it.
     static __device__ __forceinline__ float4 read(uint32_t buf, int lane, int i) {
-        const uint32_t r = static_cast<uint32_t>(kRows * i + lane / kLanes);
-        return ld_shared_f4(buf + r * 128u + ((static_cast<uint32_t>(lane % kLanes) ^ (r & 7u)) << 4));
+        return ld_shared_f4(piece(buf, static_cast<uint32_t>(kAccRows * i + lane / kLanes),
+                                  static_cast<uint32_t>(lane % kLanes)));
     }
 };
 
@@ -171,8 +191,8 @@ struct QuadChunk {
 // walks all BN columns, one row per thread (Epi(params, group, row, n0); chunk(params,
 // v[32], column, offset in the tile, io); finish(params, n_block)).  With 8, two warps
 // share the rows and take half of the columns each, and every chunk goes through the warp's
-// staging buffer (QuadChunk; Epi(params, group, first row, first column, lane);
-// chunk(params, staged chunk, lane, offset); finish(params, n_block, lane)).  The functor
+// staging buffer (RowChunk; Epi(params, group, first row, first column, lane);
+// chunk(params, staged chunk, lane, chunk index); finish(params, n_block, lane)).  The functor
 // is made before the accumulator is awaited, so that what its constructor loads arrives
 // during the mainloop.  `ready` waits for the accumulator (false: give up), `release`
 // gives it back once its last columns are in registers.
@@ -194,23 +214,23 @@ __device__ __forceinline__ bool epilogue_tile(const typename Epi::Params& ep, in
         }
         epi.finish(ep, nb);
     } else {
-        using Q = QuadChunk;
+        using R = RowChunk;
         static_assert(BN == 256, "the 8-warp epilogues split 256 columns");
-        const int c0 = warp_half * Q::kTileCols;
+        const int c0 = warp_half * R::kTileCols;
         Epi epi(ep, g, row0, nb * BN + c0, io.lane);
         if (!ready()) return false;
-        constexpr int kChunks = Q::kTileCols / Q::kCols;
 #pragma unroll 1
-        for (int c = 0; c < kChunks; ++c) {
-            float v[32];
-            tmem_ld_32x32b_x32(t_row + c0 + c * Q::kCols, v);
-            if (c == kChunks - 1) release();
-            uint32_t w[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) w[j] = __float_as_uint(v[j]);
-            out_stage_row(io.out, io.lane, w);
-            __syncwarp();
-            epi.chunk(ep, io.out, io.lane, c * Q::kCols);
+        for (int c = 0; c < R::kChunks; ++c) {
+            // every lane reads its row's columns again for each row group
+#pragma unroll 1
+            for (int h = 0; h < R::kCols / 32; ++h) {
+                float v[32];
+                tmem_ld_32x32b_x32(t_row + c0 + (c % R::kColGroups) * R::kCols + 32 * h, v);
+                if (c == R::kChunks - 1 && h == R::kCols / 32 - 1) release();
+                R::stage(io.out, io.lane, c / R::kColGroups, h, v);
+                __syncwarp();
+            }
+            epi.chunk(ep, io.out, io.lane, c);
             __syncwarp();
         }
         epi.finish(ep, nb, io.lane);
