@@ -324,7 +324,6 @@ int32_t fpo_error_signal(const fpo_error_signal_desc* desc, const void* h, const
                                            part, L.n_tiles, zy, nullptr, L.ldv, st));
         FPO_TRY(per_chunk ? ev(2) : mark(2));
         FPO_TRY(launch_lse_combine(part, L.n_tiles, T, zy, lse, ce, st));
-        if (loss_out) FPO_TRY(launch_mean(ce, T, loss_out, st));
         FPO_TRY(per_chunk ? ev(3) : mark(3));
         // 3./4. per token chunk: recompute the logits -> E, then g = E W_U
         for (int64_t c0 = 0, ci = 0; c0 < T; c0 += L.Tc, ++ci) {
@@ -352,11 +351,10 @@ int32_t fpo_error_signal(const fpo_error_signal_desc* desc, const void* h, const
             FPO_TRY(cmark(ci, 5));
         }
     } else {
-        // 2.-4. per token chunk: logits pass storing z -> lse -> E from z -> g = E W_U
+        // 2.-4. per token chunk: logits pass storing z -> lse and E from z -> g = E W_U
         float* z = reinterpret_cast<float*>(ws + L.z);
         for (int64_t c0 = 0, ci = 0; c0 < T; c0 += L.Tc, ++ci) {
             const int tc = static_cast<int>(L.Tc < T - c0 ? L.Tc : T - c0);
-            const bool last = c0 + tc >= T;
             const void* yh = static_cast<const uint8_t*>(yhat) + static_cast<size_t>(c0) * d * esz;
             float2* pc = part + static_cast<size_t>(c0) * L.n_tiles;
             float* zyc = zy ? zy + c0 : nullptr;
@@ -369,11 +367,9 @@ int32_t fpo_error_signal(const fpo_error_signal_desc* desc, const void* h, const
                                                static_cast<const float*>(W_U), targets + c0, tc, T,
                                                d, V, pc, L.n_tiles, zyc, z, L.ldv, st));
             FPO_TRY(cmark(ci, 2));
-            FPO_TRY(launch_lse_combine(pc, L.n_tiles, tc, zyc, lse + c0, cec, st));
-            if (last && loss_out) FPO_TRY(launch_mean(ce, T, loss_out, st));
-            FPO_TRY(cmark(ci, 3));
-            FPO_TRY(launch_error_from_logits(desc->dtype, z, lse + c0, targets + c0, tc, V,
-                                             L.ldv, desc->loss_scale, E, st));
+            FPO_TRY(cmark(ci, 3));  // the combine is part of the next kernel
+            FPO_TRY(launch_error_from_logits(desc->dtype, z, pc, L.n_tiles, zyc, targets + c0, tc, V,
+                                             L.ldv, desc->loss_scale, lse + c0, cec, E, st));
             FPO_TRY(cmark(ci, 4));
             if (bf16)
                 FPO_TRY(launch_proj_bf16(E, W_U, tc, T, d, V, g + c0 * d, sk, status, st));
@@ -384,11 +380,11 @@ int32_t fpo_error_signal(const fpo_error_signal_desc* desc, const void* h, const
             FPO_TRY(cmark(ci, 5));
         }
     }
-    // 5. final-norm VJP with the min-RMS clamp -> g~ (already in the direct algorithm's
-    //    projection epilogue; the stage is then empty)
+    // 5. final-norm VJP with the min-RMS clamp -> g~, and the mean loss (both done by the
+    //    direct algorithm above; the stage is then empty)
     if (!direct)
-        FPO_TRY(launch_rmsnorm_vjp(desc->dtype, g, h, norm_w, rho, T, d, desc->min_rms, g_out,
-                                   st));
+        FPO_TRY(launch_rmsnorm_vjp(desc->dtype, g, h, norm_w, rho, T, d, desc->min_rms, g_out, ce,
+                                   loss_out, st));
     FPO_TRY(per_chunk ? ev(2 + 4 * n_chunks) : mark(6));
     return FPO_OK;
 }

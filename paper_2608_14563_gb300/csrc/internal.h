@@ -237,17 +237,19 @@ cudaError_t launch_direct_fixup_factors(const float* sx, const float* qz, const 
 cudaError_t launch_lse_combine(const float2* part, int n_tiles, int T, const float* zy,
                                float* lse, float* ce, cudaStream_t st);
 cudaError_t launch_mean(const float* x, int n, float* out, cudaStream_t st);
-// Stored-logits algorithm: E[M, ld] = s (exp(z - lse) - onehot(y)) from z[M, ld] fp32, in
+// Stored-logits algorithm: lse (and with ce the cross-entropies lse - zy) of M rows from the
+// logits pass's partials, and E[M, ld] = s (exp(z - lse) - onehot(y)) from z[M, ld] fp32, in
 // dtype (bf16 through the same formula as the recompute epilogue, or fp32); ld, a multiple
 // of 8, is the row stride of both, and columns V and above are left unspecified.
-cudaError_t launch_error_from_logits(int dtype, const float* z, const float* lse, const int32_t* y,
-                                     int M, int V, long long ld, float s, void* E,
-                                     cudaStream_t st);
+cudaError_t launch_error_from_logits(int dtype, const float* z, const float2* part, int n_tiles,
+                                     const float* zy, const int32_t* y, int M, int V, long long ld,
+                                     float s, float* lse, float* ce, void* E, cudaStream_t st);
 // dst[n] = src[n] rounded to dtype (a plain copy for fp32).
 cudaError_t launch_cast_f32(int dtype, const float* src, size_t n, void* dst, cudaStream_t st);
+// With loss also the mean of the batch's cross-entropies ce[0, T).
 cudaError_t launch_rmsnorm_vjp(int dtype, const float* g, const void* h, const void* w,
                                const float* rho, int T, int d, float min_rms, void* out,
-                               cudaStream_t st);
+                               const float* ce, float* loss, cudaStream_t st);
 // Layer-specific signals: out[l] = pre-MLP VJP at x[l] of (post-FFN VJP at m[l] of g), either
 // stage skipped when its array is null (not both); one launch for all layers.
 cudaError_t launch_layer_signals(int dtype, int n_layers, const void* g, const void* const* m,

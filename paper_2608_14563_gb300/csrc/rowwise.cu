@@ -262,13 +262,60 @@ __global__ void __launch_bounds__(kBlkThreads)
     }
 }
 
+// Mean of x[0, n) by one block, in a fixed order: thread i adds x[i], x[i + THREADS], ...,
+// its loads issued kBatch at a time (the loop waits once per batch), then a fixed butterfly
+// per warp and the warps' sums in warp order.
+template <int THREADS>
+__device__ __forceinline__ void block_mean(const float* __restrict__ x, int n,
+                                           float* __restrict__ out) {
+    __shared__ double buf[THREADS / 32];
+    constexpr int kBatch = 16;
+    double acc = 0.0;
+    long long i = threadIdx.x;
+    for (; i + (kBatch - 1) * static_cast<long long>(THREADS) < n; i += kBatch * THREADS) {
+        float v[kBatch];
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) v[k] = x[i + k * THREADS];
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) acc += static_cast<double>(v[k]);
+    }
+    for (; i < n; i += THREADS) acc += static_cast<double>(x[i]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+#pragma unroll
+        for (int k = 0; k < THREADS / 32; ++k) t += buf[k];
+        out[0] = static_cast<float>(t / static_cast<double>(n));
+    }
+}
+
+// log-sum-exp of one row from its (max, sum exp) partials, by one warp; every lane gets it.
+__device__ __forceinline__ float row_lse(const float2* __restrict__ pr, int n_tiles, int lane) {
+    float m = -INFINITY;
+    for (int i = lane; i < n_tiles; i += 32) m = fmaxf(m, pr[i].x);
+    m = warp_max(m);
+    float s = 0.f;
+    for (int i = lane; i < n_tiles; i += 32) {
+        const float2 p = pr[i];
+        if (p.y > 0.f) s += p.y * expf(p.x - m);
+    }
+    s = warp_sum(s);
+    return m + logf(s);
+}
+
 template <int EPT>
 __global__ void __launch_bounds__(kBlkThreads)
     rmsnorm_vjp_row_kernel(const float* __restrict__ g, const __nv_bfloat16* __restrict__ h,
                            const __nv_bfloat16* __restrict__ w, const float* __restrict__ rho,
-                           int T, int d, float min_rms, __nv_bfloat16* __restrict__ out) {
+                           int T, int d, float min_rms, __nv_bfloat16* __restrict__ out,
+                       const float* __restrict__ ce, float* __restrict__ loss) {
     grid_dependency_trigger();
     grid_dependency_wait();
+    // the batch's mean cross-entropy beside the rows (every token's is final by now)
+    if (loss && blockIdx.x == 0) block_mean<kBlkThreads>(ce, T, loss);
     constexpr int NV = EPT / 8;
     for (int row = blockIdx.x; row < T; row += gridDim.x) {
         const float r = rho[row];
@@ -331,9 +378,12 @@ template <typename TT, int VEC>
 __global__ void __launch_bounds__(kRowThreads)
     rmsnorm_vjp_kernel(const float* __restrict__ g, const TT* __restrict__ h,
                        const TT* __restrict__ w, const float* __restrict__ rho, int T, int d,
-                       float min_rms, TT* __restrict__ out) {
+                       float min_rms, TT* __restrict__ out,
+                       const float* __restrict__ ce, float* __restrict__ loss) {
     grid_dependency_trigger();
     grid_dependency_wait();
+    // the batch's mean cross-entropy beside the rows (every token's is final by now)
+    if (loss && blockIdx.x == 0) block_mean<kRowThreads>(ce, T, loss);
     const int lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
     for (int row = blockIdx.x * wpb + (threadIdx.x >> 5); row < T; row += gridDim.x * wpb) {
@@ -374,17 +424,7 @@ __global__ void __launch_bounds__(kRowThreads)
     const int lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
     for (int row = blockIdx.x * wpb + (threadIdx.x >> 5); row < T; row += gridDim.x * wpb) {
-        const float2* pr = part + static_cast<size_t>(row) * n_tiles;
-        float m = -INFINITY;
-        for (int i = lane; i < n_tiles; i += 32) m = fmaxf(m, pr[i].x);
-        m = warp_max(m);
-        float s = 0.f;
-        for (int i = lane; i < n_tiles; i += 32) {
-            const float2 p = pr[i];
-            if (p.y > 0.f) s += p.y * expf(p.x - m);
-        }
-        s = warp_sum(s);
-        const float l = m + logf(s);
+        const float l = row_lse(part + static_cast<size_t>(row) * n_tiles, n_tiles, lane);
         if (lane == 0) {
             lse[row] = l;
             if (ce) ce[row] = l - zy[row];
@@ -488,18 +528,8 @@ __global__ void __launch_bounds__(kRowThreads)
     const int n = *fix_count;
     for (int i = blockIdx.x * wpb + (threadIdx.x >> 5); i < n; i += gridDim.x * wpb) {
         const int row = fix[i];
-        const float2* pr = part + static_cast<size_t>(row) * n_tiles;
-        float m = -INFINITY;
-        for (int k = lane; k < n_tiles; k += 32) m = fmaxf(m, pr[k].x);
-        m = warp_max(m);
-        float e = 0.f;
-        for (int k = lane; k < n_tiles; k += 32) {
-            const float2 p = pr[k];
-            if (p.y > 0.f) e += p.y * expf(p.x - m);
-        }
-        e = warp_sum(e);
+        const float l = row_lse(part + static_cast<size_t>(row) * n_tiles, n_tiles, lane);
         if (lane == 0) {
-            const float l = m + logf(e);
             lse[row] = l;
             if (ce) ce[row] = l - anchor[row];
         }
@@ -538,37 +568,13 @@ __global__ void __launch_bounds__(kRowThreads)
     }
 }
 
-// Mean of x[0, n) by one block, in a fixed order: thread i adds x[i], x[i + kMeanThreads],
-// ..., its loads issued kBatch at a time (the loop waits once per batch), then a fixed
-// butterfly per warp and the warps' sums in warp order.
 constexpr int kMeanThreads = 512;
 
 __global__ void __launch_bounds__(kMeanThreads) mean_kernel(const float* __restrict__ x, int n,
                                                             float* __restrict__ out) {
     grid_dependency_trigger();
     grid_dependency_wait();
-    __shared__ double buf[kMeanThreads / 32];
-    constexpr int kBatch = 16;
-    double acc = 0.0;
-    long long i = threadIdx.x;
-    for (; i + (kBatch - 1) * static_cast<long long>(kMeanThreads) < n; i += kBatch * kMeanThreads) {
-        float v[kBatch];
-#pragma unroll
-        for (int k = 0; k < kBatch; ++k) v[k] = x[i + k * kMeanThreads];
-#pragma unroll
-        for (int k = 0; k < kBatch; ++k) acc += static_cast<double>(v[k]);
-    }
-    for (; i < n; i += kMeanThreads) acc += static_cast<double>(x[i]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-#pragma unroll
-        for (int k = 0; k < kMeanThreads / 32; ++k) t += buf[k];
-        out[0] = static_cast<float>(t / static_cast<double>(n));
-    }
+    block_mean<kMeanThreads>(x, n, out);
 }
 
 __global__ void cast_f32_kernel(const float* __restrict__ src, size_t n, __nv_bfloat16* __restrict__ dst) {
@@ -577,19 +583,28 @@ __global__ void cast_f32_kernel(const float* __restrict__ src, size_t n, __nv_bf
         dst[i] = __float2bfloat16_rn(src[i]);
 }
 
-// One block per row (grid-stride over rows): 8 logits per thread per step,
-// two 16-byte loads of z and one 16-byte (bf16) or two (fp32) stores of E.
+// One block per row (grid-stride over rows): the row's lse from the logits pass's partials
+// (every warp forms it for itself; thread 0 stores it and the token's cross-entropy), then
+// E: 8 logits per thread per step, two 16-byte loads of z and one 16-byte (bf16) or two
+// (fp32) stores of E.
 constexpr int kErrThreads = 256;
 
 template <bool kBf16>
 __global__ void __launch_bounds__(kErrThreads)
-    error_from_logits_kernel(const float* __restrict__ z, const float* __restrict__ lse,
+    error_from_logits_kernel(const float* __restrict__ z, const float2* __restrict__ part,
+                             int n_tiles, const float* __restrict__ zy,
                              const int32_t* __restrict__ y, int M, int V, long long ld, float s,
+                             float* __restrict__ lse, float* __restrict__ ce,
                              void* __restrict__ E) {
     grid_dependency_trigger();
     grid_dependency_wait();
     for (int row = blockIdx.x; row < M; row += gridDim.x) {
-        const float l = lse[row];
+        const float l =
+            row_lse(part + static_cast<size_t>(row) * n_tiles, n_tiles, threadIdx.x & 31);
+        if (threadIdx.x == 0) {
+            lse[row] = l;
+            if (ce) ce[row] = l - zy[row];
+        }
         const float l2 = l * kLog2e;
         const int yt = y[row];
         const float* zr = z + row * ld;  // V <= ld, a multiple of 8
@@ -1102,7 +1117,7 @@ cudaError_t launch_direct_fixup_factors(const float* sx, const float* qz, const 
 
 cudaError_t launch_rmsnorm_vjp(int dtype, const float* g, const void* h, const void* w,
                                const float* rho, int T, int d, float min_rms, void* out,
-                               cudaStream_t st) {
+                               const float* ce, float* loss, cudaStream_t st) {
     if (T <= 0) return cudaSuccess;
     const int grid = row_grid(T);
     const int ept = dtype == 1 ? row_ept(d) : 0;
@@ -1112,26 +1127,26 @@ cudaError_t launch_rmsnorm_vjp(int dtype, const float* g, const void* h, const v
         auto* oo = static_cast<__nv_bfloat16*>(out);
         if (ept == 8)
             return launch_chained(rmsnorm_vjp_row_kernel<8>, dim3(blk_grid(T)), kBlkThreads, 0, st,
-                                  g, hh, ww, rho, T, d, min_rms, oo);
+                                  g, hh, ww, rho, T, d, min_rms, oo, ce, loss);
         else if (ept == 16)
             return launch_chained(rmsnorm_vjp_row_kernel<16>, dim3(blk_grid(T)), kBlkThreads, 0,
-                                  st, g, hh, ww, rho, T, d, min_rms, oo);
+                                  st, g, hh, ww, rho, T, d, min_rms, oo, ce, loss);
         else
             return launch_chained(rmsnorm_vjp_row_kernel<32>, dim3(blk_grid(T)), kBlkThreads, 0,
-                                  st, g, hh, ww, rho, T, d, min_rms, oo);
+                                  st, g, hh, ww, rho, T, d, min_rms, oo, ce, loss);
     } else if (dtype == 1) {
         return launch_chained(rmsnorm_vjp_kernel<__nv_bfloat16, 8>, dim3(grid), kRowThreads, 0, st,
                               g, static_cast<const __nv_bfloat16*>(h),
                               static_cast<const __nv_bfloat16*>(w), rho, T, d, min_rms,
-                              static_cast<__nv_bfloat16*>(out));
+                              static_cast<__nv_bfloat16*>(out), ce, loss);
     } else if (d % 4 == 0) {
         return launch_chained(rmsnorm_vjp_kernel<float, 4>, dim3(grid), kRowThreads, 0, st, g,
                               static_cast<const float*>(h), static_cast<const float*>(w), rho, T,
-                              d, min_rms, static_cast<float*>(out));
+                              d, min_rms, static_cast<float*>(out), ce, loss);
     } else {
         return launch_chained(rmsnorm_vjp_kernel<float, 1>, dim3(grid), kRowThreads, 0, st, g,
                               static_cast<const float*>(h), static_cast<const float*>(w), rho, T,
-                              d, min_rms, static_cast<float*>(out));
+                              d, min_rms, static_cast<float*>(out), ce, loss);
     }
 }
 
@@ -1143,19 +1158,18 @@ cudaError_t launch_cast_f32(int dtype, const float* src, size_t n, void* dst, cu
     return cudaGetLastError();
 }
 
-cudaError_t launch_error_from_logits(int dtype, const float* z, const float* lse, const int32_t* y,
-                                     int M, int V, long long ld, float s, void* E,
-                                     cudaStream_t st) {
+cudaError_t launch_error_from_logits(int dtype, const float* z, const float2* part, int n_tiles,
+                                     const float* zy, const int32_t* y, int M, int V, long long ld,
+                                     float s, float* lse, float* ce, void* E, cudaStream_t st) {
     if (M <= 0) return cudaSuccess;
     DevInfo di;
     const int sms = current_device_info(&di) ? di.sm_count : 148;
     const int grid = M < sms * 8 ? M : sms * 8;
     if (dtype == 1)
-        return launch_chained(error_from_logits_kernel<true>, dim3(grid), kErrThreads, 0, st, z,
-                              lse, y, M, V, ld, s, E);
-    else
-        return launch_chained(error_from_logits_kernel<false>, dim3(grid), kErrThreads, 0, st, z,
-                              lse, y, M, V, ld, s, E);
+        return launch_chained(error_from_logits_kernel<true>, dim3(grid), kErrThreads, 0, st, z, part,
+                              n_tiles, zy, y, M, V, ld, s, lse, ce, E);
+    return launch_chained(error_from_logits_kernel<false>, dim3(grid), kErrThreads, 0, st, z, part,
+                          n_tiles, zy, y, M, V, ld, s, lse, ce, E);
 }
 
 cudaError_t launch_wait_timeout(unsigned* status, uint64_t limit_ns, cudaStream_t st) {
