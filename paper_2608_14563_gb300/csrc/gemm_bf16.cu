@@ -405,11 +405,14 @@ int proj_clusters() {
 // last wave.  Below that the clusters without a tile would idle through a K loop over the
 // whole vocabulary, so such a batch runs on 256 x 256 tiles, each in the number of ranges
 // that costs least.  Measured, in ns: a 64-deep k-block 344 (at the clock the tensor cores
-// hold under load), with a split the fixup's launch 4000 and its read of the fp32 parts
-// 4.3 bytes a ns.  Ranges have at least 32 k-blocks, and the units fit the scratch.  T is
-// the whole batch where that is small, so that its sums do not depend on the chunking, and
-// otherwise the chunk (the last one of T 9000 has 808 tokens).  Projection with its fixup, T x d x V: 333 x 4096 x 100352 (16 tiles of 512 columns on 76
-// clusters) 887 us whole, 246 us in 7 ranges; 2048 x 2048 x 50304 (32 tiles) 434 and 276.
+// hold under load), with a split 2500 per wave of units for the epilogue that stores their
+// fp32 parts, the fixup's launch 4000 and its read of the parts 4.3 bytes a ns.  Ranges
+// have at least 32 k-blocks, and the units fit the scratch.  T is the whole batch where
+// that is small, so that its sums do not depend on the chunking, and otherwise the chunk
+// (the last one of T 9000 has 808 tokens).  Projection with its fixup, T x d x V:
+// 333 x 4096 x 100352 (16 tiles of 512 columns on 76 clusters) 887 us whole, 246 us in 7
+// ranges; 2048 x 2048 x 50304 (32 such tiles) 434 us, 276 in 7 ranges of 256 columns and
+// about the same in whole 256-column tiles, which draw less power (step 818 and 777 us).
 int proj_split(int T, int d, int V) {
     const long long clusters = proj_clusters();
     const long long m_blocks = (T + kPairBM - 1) / kPairBM;
@@ -421,9 +424,9 @@ int proj_split(int T, int d, int V) {
     int best = 1;
     for (int S = 1; S <= 64; ++S) {
         if (S > 1 && (kb / S < 32 || tiles * S > cap)) break;
-        double cost = static_cast<double>((tiles * S + clusters - 1) / clusters) *
-                          ((kb + S - 1) / S) * 344.0;
-        if (S > 1) cost += 4000.0 + tiles * S * (kProjBN * 1024.0) / 4300.0;
+        const double waves = static_cast<double>((tiles * S + clusters - 1) / clusters);
+        double cost = waves * ((kb + S - 1) / S) * 344.0;
+        if (S > 1) cost += waves * 2500.0 + 4000.0 + tiles * S * (kProjBN * 1024.0) / 4300.0;
         if (S == 1 || cost < best_cost) {
             best_cost = cost;
             best = S;

@@ -12,10 +12,10 @@
 // and outputs whose rows are 16-byte aligned take 16-byte accesses.
 //
 // Bound: the FMA pipe.  128-tiles keep it 69% busy over a long launch (logits pass of
-// T 777, d 768, V 32001: 1510 us with 64 x 64 tiles and one slice in flight, 837 us now);
-// 8 x 16 outputs per thread or scalar FMAs were slower (930 and 877 us), as was unrolling
-// the slice fully (900 us, spills).  The split along K is for outputs too small to fill
-// the SMs: the projection of those sizes 3154 -> 981 us, at T 128, d 64, V 512 27 -> 10 us.
+// T 777, d 768, V 32001: 1510 us with 64 x 64 tiles and one slice in flight, 850 us now);
+// 8 x 16 outputs per thread, scalar FMAs or 32-deep slices were slower (930, 877 and 991
+// us).  The split along K is for outputs too small to fill the SMs: the projection of those
+// sizes 3154 -> 980 us, at T 128, d 64, V 512 27 -> 10 us.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -197,7 +197,9 @@ __global__ void __launch_bounds__(kThreads, 2)
             la.load(A, ops.lda, m0, ops.M, (s + 1) * kKs, ops.K, ops.vec_a);
             lb.load(B, ops.ldb, n0, ops.N, (s + 1) * kKs, ops.K, ops.vec_b);
         }
-#pragma unroll 2
+        // (128-tiles unrolled by 2: the logits pass 905 us instead of 852; 4 and 16 slower)
+        constexpr int kUnroll = BT == 128 ? 1 : 2;
+#pragma unroll kUnroll
         for (int kk = 0; kk < kKs; ++kk) {
             float a[kR];
             float2 b[2 * kH];
