@@ -521,11 +521,13 @@ struct EpiProjVjp {
     __device__ __forceinline__ void finish(const Params&, int) {}
 };
 
-// A lane's place in a warp's 32 rows x 128 columns of an 8-warp epilogue: the 4 columns of
-// access i of chunk c (numbered j = kAcc c + i over the whole block), as element offsets
-// into matrices of row stride ld.
+// A lane's place in a warp's 32 rows x 64 kCG columns (kCG = 2 or 1 groups of chunk columns,
+// of tiles of 256 or 128) of an 8-warp epilogue: the 4 columns of access i of chunk c (numbered
+// j = kAcc c + i over the whole block), as element offsets into matrices of row stride ld.
+template <int kCG>
 struct RowPos {
     using R = RowChunk;
+    static constexpr int kChunks = 32 / R::kRows * kCG;
     long long off;    // of the lane's columns in its first row
     int rows, cols;   // rows from the lane's first, columns from its first, inside
 
@@ -536,9 +538,9 @@ struct RowPos {
         cols = N - c;
     }
     static __device__ __forceinline__ int row(int j) {
-        return j / R::kAcc / R::kColGroups * R::kRows + j % R::kAcc * R::kAccRows;
+        return j / R::kAcc / kCG * R::kRows + j % R::kAcc * R::kAccRows;
     }
-    static __device__ __forceinline__ int col(int j) { return j / R::kAcc % R::kColGroups * R::kCols; }
+    static __device__ __forceinline__ int col(int j) { return j / R::kAcc % kCG * R::kCols; }
     // Access j is inside the matrix (N is a multiple of 8, so its 4 columns are inside
     // together).
     __device__ __forceinline__ bool in(int j) const { return row(j) < rows && col(j) < cols; }
@@ -562,15 +564,37 @@ struct RowPos {
 // gave 162 but cost 2% of a T 200 step, as every lane reads the accumulator once per row
 // group.  Two batches in flight gave nothing more, nor did 16 warps, L2 prefetches of the
 // next tile or streaming cache hints).
-// Slots of per-warp partial sums per (256-row block, 256-column tile): 8 blocks of 32 rows
-// times the two column halves.
-constexpr int kColSlots = 16;
+// Slots of per-warp partial sums per (256-row block, 256 columns): 8 blocks of 32 rows times
+// 4 column quarters.  A warp with two column groups keeps their sums apart, so that tiles of
+// 128 columns leave the same slots.
+constexpr int kColSlots = 32;
 
-__device__ __forceinline__ long long slot_of(int g, int m256, int n_blocks, int nb, int row0,
-                                               int n0) {
-    return ((static_cast<long long>(g) * m256 + row0 / 256) * n_blocks + nb) * kColSlots +
-           ((n0 % 256) / RowChunk::kTileCols) * 8 + (row0 % 256) / 32;
+template <int N>
+__device__ __forceinline__ float* slot_of(float* part, int g, int m256, int n256, int row0, int n0) {
+    return part + (((static_cast<long long>(g) * m256 + row0 / 256) * n256 + n0 / 256) * kColSlots +
+                   (n0 % 256) / 64 * 8 + (row0 % 256) / 32) * N;
 }
+
+// N sums per column group, added chunk by chunk.
+template <int N, int kCG>
+struct GroupSums {
+    float v[kCG][N];
+    __device__ __forceinline__ GroupSums() {
+#pragma unroll
+        for (int k = 0; k < N; ++k) v[0][k] = v[kCG - 1][k] = 0.f;
+    }
+    __device__ __forceinline__ void add(int chunk, const float (&x)[N]) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            if (chunk % kCG == 0)
+                v[0][k] += x[k];
+            else
+                v[kCG - 1][k] += x[k];
+        }
+    }
+    // The warp's totals (a fixed butterfly) to the slots of its one or two groups.
+    __device__ __forceinline__ void store(float* slot, int lane) const;
+};
 
 __device__ __forceinline__ float warp_sum_f32(float x) {
 #pragma unroll
@@ -578,12 +602,23 @@ __device__ __forceinline__ float warp_sum_f32(float x) {
     return x;
 }
 
+template <int N, int kCG>
+__device__ __forceinline__ void GroupSums<N, kCG>::store(float* slot, int lane) const {
+#pragma unroll
+    for (int c = 0; c < kCG; ++c) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const float t = warp_sum_f32(v[c][k]);
+            if (lane == 0) slot[8 * c * N + k] = t;
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Pseudogradient update (Eq. w3update, App. A): for group (layer) g,
 //   W_master[g] -= lr * G ;  W_out[g] = bf16(W_master[g]) ;  G_out[g] = bf16(G)
 // Any of the three pointers may be null for a layer.
-struct EpiUpdate {
-    static constexpr int kWarps = 8;
+struct EpiUpdateBase {
     struct Params {
         float* W_master[kMaxGroups];
         __nv_bfloat16* W_out[kMaxGroups];
@@ -592,8 +627,13 @@ struct EpiUpdate {
         int M, N;
         float neg_lr;
     };
+};
+
+template <int kCG>
+struct EpiUpdate : EpiUpdateBase {
+    static constexpr int kWarps = 8, kColGroups = kCG;
     using R = RowChunk;
-    RowPos pos;
+    RowPos<kCG> pos;
     float* wm;
     __nv_bfloat16* wo;
     __nv_bfloat16* go;
@@ -637,20 +677,19 @@ struct EpiUpdate {
                 *reinterpret_cast<uint2*>(go + o) =
                     make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
         }
-        if (c + 1 < R::kChunks) load(p, c + 1);
+        if (c + 1 < pos.kChunks) load(p, c + 1);
     }
 
-    __device__ __forceinline__ void finish(const Params&, int, int) {}
+    __device__ __forceinline__ void finish(const Params&, int) {}
 };
 
 // ---------------------------------------------------------------------------
 // Pseudogradients with the layer-viability diagnostic's cosine (Sec. 2.2 Eq. (cosine),
 // Eq. (w3update)): for group (layer) g, G_out[g] = bf16(G), and the three sums of the
-// cosine of that stored G against Y[g] (<G, Y>, ||G||^2, ||Y||^2) over the warp's 32 rows
-// x 128 columns (fp32 per lane, then a fixed butterfly), one triple per slot_of, so the
+// cosine of that stored G against Y[g] (<G, Y>, ||G||^2, ||Y||^2) over the warp's
+// block (fp32 per lane, then a fixed butterfly), one triple per slot (slot_of), so the
 // cosine needs no second pass over G.
-struct EpiGradCos {
-    static constexpr int kWarps = 8;
+struct EpiGradCosBase {
     struct Params {
         __nv_bfloat16* G_out[kMaxGroups];
         const __nv_bfloat16* Y[kMaxGroups];
@@ -659,10 +698,15 @@ struct EpiGradCos {
         int M, N;
         int m256, n_blocks;
     };
+};
+
+template <int kCG>
+struct EpiGradCos : EpiGradCosBase {
+    static constexpr int kWarps = 8, kColGroups = kCG;
     using R = RowChunk;
-    RowPos pos;
+    RowPos<kCG> pos;
     int g, row0, n0;
-    float2 s_gy, s_gg, s_yy;
+    GroupSums<3, kCG> sums;  // <G, Y>, ||G||^2, ||Y||^2
     uint2 y[R::kAcc];  // Y of the next chunk
 
     __device__ __forceinline__ void load(const Params& p, int c) {
@@ -673,11 +717,11 @@ struct EpiGradCos {
 
     __device__ __forceinline__ EpiGradCos(const Params& p, int g_, int row0_, int n0_, int lane)
         : pos(p.M, p.N, p.ld, row0_, n0_, lane), g(g_), row0(row0_), n0(n0_) {
-        s_gy = s_gg = s_yy = make_float2(0.f, 0.f);
         load(p, 0);
     }
 
     __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int c) {
+        float2 s_gy = make_float2(0.f, 0.f), s_gg = s_gy, s_yy = s_gy;
 #pragma unroll
         for (int i = 0; i < R::kAcc; ++i) {
             const float4 v = R::read(buf, lane, i);
@@ -698,29 +742,22 @@ struct EpiGradCos {
                 s_yy = __ffma2_rn(yr, yr, s_yy);
             }
         }
-        if (c + 1 < R::kChunks) load(p, c + 1);
+        if (c + 1 < pos.kChunks) load(p, c + 1);
+        sums.add(c, {s_gy.x + s_gy.y, s_gg.x + s_gg.y, s_yy.x + s_yy.y});
     }
 
-    __device__ __forceinline__ void finish(const Params& p, int nb, int lane) {
-        const float gy = warp_sum_f32(s_gy.x + s_gy.y), gg = warp_sum_f32(s_gg.x + s_gg.y),
-                    yy = warp_sum_f32(s_yy.x + s_yy.y);
-        if (lane == 0) {
-            float* o = p.part + slot_of(g, p.m256, p.n_blocks, nb, row0, n0) * 3;
-            o[0] = gy;
-            o[1] = gg;
-            o[2] = yy;
-        }
+    __device__ __forceinline__ void finish(const Params& p, int lane) {
+        sums.store(slot_of<3>(p.part, g, p.m256, p.n_blocks, row0, n0), lane);
     }
 };
 
 // ---------------------------------------------------------------------------
 // Pseudogradient only, fp32, one output per group (layer): G[g] = g~^T A_l, for
 // the optimizers that need the whole G before they step.  With W_master set (the relative
-// clip on the gradient) also ||W||^2 and ||G||^2 of the warp's 32 rows x 128 columns, one
+// clip on the gradient) also ||W||^2 and ||G||^2 of the warp's block, one
 // pair per slot_of, so that the clip factor needs no pass over W and G of its own
 // (448 us of 1823 for 3 layers of 3072 x 23040).
-struct EpiStoreGroupF32 {
-    static constexpr int kWarps = 8;
+struct EpiStoreGroupF32Base {
     struct Params {
         float* G[kMaxGroups];
         const float* W_master[kMaxGroups];  // or null: no norms
@@ -729,12 +766,17 @@ struct EpiStoreGroupF32 {
         int M, N;
         int m256, n_blocks;
     };
+};
+
+template <int kCG>
+struct EpiStoreGroupF32 : EpiStoreGroupF32Base {
+    static constexpr int kWarps = 8, kColGroups = kCG;
     using R = RowChunk;
-    RowPos pos;
+    RowPos<kCG> pos;
     int g, row0, n0;
     float* G;
     const float* wm;
-    float s_ww, s_gg;
+    GroupSums<2, kCG> sums;  // ||W||^2, ||G||^2
     float4 w[R::kAcc];  // master values of the next chunk
 
     __device__ __forceinline__ void load(const Params& p, int c) {
@@ -747,11 +789,12 @@ struct EpiStoreGroupF32 {
     __device__ __forceinline__ EpiStoreGroupF32(const Params& p, int g_, int row0_, int n0_,
                                                 int lane)
         : pos(p.M, p.N, p.ld, row0_, n0_, lane), g(g_), row0(row0_), n0(n0_), G(p.G[g_]),
-          wm(p.W_master[g_]), s_ww(0.f), s_gg(0.f) {
+          wm(p.W_master[g_]) {
         load(p, 0);
     }
 
     __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int c) {
+        float s_ww = 0.f, s_gg = 0.f;
 #pragma unroll
         for (int i = 0; i < R::kAcc; ++i) {
             const float4 v = R::read(buf, lane, i);
@@ -763,17 +806,12 @@ struct EpiStoreGroupF32 {
                             fmaf(w[i].y, w[i].y, fmaf(w[i].z, w[i].z, fmaf(w[i].w, w[i].w, s_ww))));
             }
         }
-        if (c + 1 < R::kChunks) load(p, c + 1);
+        if (c + 1 < pos.kChunks) load(p, c + 1);
+        sums.add(c, {s_ww, s_gg});
     }
 
-    __device__ __forceinline__ void finish(const Params& p, int nb, int lane) {
-        if (!wm) return;
-        const float ww = warp_sum_f32(s_ww), gg = warp_sum_f32(s_gg);
-        if (lane == 0) {
-            float* o = p.part + slot_of(g, p.m256, p.n_blocks, nb, row0, n0) * 2;
-            o[0] = ww;
-            o[1] = gg;
-        }
+    __device__ __forceinline__ void finish(const Params& p, int lane) {
+        if (wm) sums.store(slot_of<2>(p.part, g, p.m256, p.n_blocks, row0, n0), lane);
     }
 };
 
@@ -783,7 +821,7 @@ struct EpiStoreGroupF32 {
 // ||dW|| <= clip_frac ||W||).  With G from the accumulator, each element's optimizer state
 // advances and its unclipped step d = opt_step(G, W, s1, s2) is stored (fp32, D[g], null
 // for momentum, whose step -lr s1 the state holds; the state sees the unclipped gradient), and ||W||^2, ||d||^2 of the warp's 32 rows x 128
-// columns are written as one pair per slot_of; a kernel then scales each layer's steps
+// columns are written as one pair per slot; a kernel then scales each layer's steps
 // by min(1, clip_frac ||W|| / ||d||) and applies them (W is not written here, so its norm
 // is the pre-step one).  Without a clip the stand-alone passes are used: taking the whole
 // step here made the update faster but the power-capped step slower (its epilogue then
@@ -792,8 +830,7 @@ struct EpiStoreGroupF32 {
 // wait that the batches of the other epilogues avoid (T 4096, d 4096, d_ff 11008, 8 layers,
 // AdamW, with 4 rows x 128 bytes per access: 2362 us; batches of a whole or half a chunk
 // 3006 and 2500, 2 ahead 2561, 8 ahead 2840, 16 warps 2990).
-struct EpiOptStep {
-    static constexpr int kWarps = 8;
+struct EpiOptStepBase {
     struct Params {
         const float* W_master[kMaxGroups];
         float* s1[kMaxGroups];             // momentum / AdamW first moment (or null)
@@ -805,15 +842,20 @@ struct EpiOptStep {
         int M, N;
         int m256, n_blocks;
     };
+};
+
+template <int kCG>
+struct EpiOptStep : EpiOptStepBase {
+    static constexpr int kWarps = 8, kColGroups = kCG;
     using R = RowChunk;
     static constexpr int kAhead = 4;
-    RowPos pos;
+    RowPos<kCG> pos;
     int g, row0, n0;
     const float* wm;
     float* p1;
     float* p2;
     float* D;
-    float s_ww, s_dd;
+    GroupSums<2, kCG> sums;  // ||W||^2, ||d||^2
     float4 w[kAhead], a[kAhead], b[kAhead];  // of the next kAhead accesses
 
     __device__ __forceinline__ void load(const Params& p, int k, int j) {
@@ -826,7 +868,7 @@ struct EpiOptStep {
     }
 
     __device__ __forceinline__ EpiOptStep(const Params& p, int g_, int row0_, int n0_, int lane)
-        : pos(p.M, p.N, p.ld, row0_, n0_, lane), g(g_), row0(row0_), n0(n0_), s_ww(0.f), s_dd(0.f) {
+        : pos(p.M, p.N, p.ld, row0_, n0_, lane), g(g_), row0(row0_), n0(n0_) {
         wm = p.W_master[g_];
         p1 = p.s1[g_];
         p2 = p.s2[g_];
@@ -836,6 +878,7 @@ struct EpiOptStep {
     }
 
     __device__ __forceinline__ void chunk(const Params& p, uint32_t buf, int lane, int c) {
+        float s_ww = 0.f, s_dd = 0.f;
 #pragma unroll 1
         for (int h = 0; h < R::kAcc; h += kAhead) {
 #pragma unroll
@@ -864,18 +907,14 @@ struct EpiOptStep {
                     if (p1) *reinterpret_cast<float4*>(p1 + o) = make_float4(av[0], av[1], av[2], av[3]);
                     if (p2) *reinterpret_cast<float4*>(p2 + o) = make_float4(bv[0], bv[1], bv[2], bv[3]);
                 }
-                if (R::kAcc * c + i + kAhead < R::kAcc * R::kChunks) load(p, k, R::kAcc * c + i + kAhead);
+                if (R::kAcc * c + i + kAhead < R::kAcc * pos.kChunks) load(p, k, R::kAcc * c + i + kAhead);
             }
         }
+        sums.add(c, {s_ww, s_dd});
     }
 
-    __device__ __forceinline__ void finish(const Params& p, int nb, int lane) {
-        const float ww = warp_sum_f32(s_ww), dd = warp_sum_f32(s_dd);
-        if (lane == 0) {
-            float* o = p.part + slot_of(g, p.m256, p.n_blocks, nb, row0, n0) * 2;
-            o[0] = ww;
-            o[1] = dd;
-        }
+    __device__ __forceinline__ void finish(const Params& p, int lane) {
+        sums.store(slot_of<2>(p.part, g, p.m256, p.n_blocks, row0, n0), lane);
     }
 };
 
@@ -883,8 +922,7 @@ struct EpiOptStep {
 // Gate / up signals of a SwiGLU MLP (Sec. 3.1 step 5, Eq. errh): the GEMM gives
 // error_h = g W3_init; with the cached pre-activations a (gate) and b (up),
 //   dA = error_h (.) b (.) silu'(a),  dB = error_h (.) silu(a)   (bf16 out)
-struct EpiSwiglu {
-    static constexpr int kWarps = 8;
+struct EpiSwigluBase {
     struct Params {
         __nv_bfloat16* dA;       // [M, N]
         __nv_bfloat16* dB;
@@ -893,8 +931,13 @@ struct EpiSwiglu {
         long long ld;
         int M, N;
     };
+};
+
+template <int kCG>
+struct EpiSwiglu : EpiSwigluBase {
+    static constexpr int kWarps = 8, kColGroups = kCG;
     using R = RowChunk;
-    RowPos pos;
+    RowPos<kCG> pos;
     uint2 ua[R::kAcc], ub[R::kAcc];  // a and b of the next chunk
 
     __device__ __forceinline__ void load(const Params& p, int c) {
@@ -939,10 +982,10 @@ struct EpiSwiglu {
                     make_uint2(pack_bf16x2(db[0], db[1]), pack_bf16x2(db[2], db[3]));
             }
         }
-        if (c + 1 < R::kChunks) load(p, c + 1);
+        if (c + 1 < pos.kChunks) load(p, c + 1);
     }
 
-    __device__ __forceinline__ void finish(const Params&, int, int) {}
+    __device__ __forceinline__ void finish(const Params&, int) {}
 };
 
 }  // namespace fpo

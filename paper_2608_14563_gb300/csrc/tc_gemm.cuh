@@ -149,8 +149,8 @@ __device__ __forceinline__ void out_stage_row(uint32_t buf, int r, const uint32_
                      w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
 }
 
-// Chunks of the 8-warp epilogues: kRows of the warp's 32 rows x kCols of its 128 fp32
-// columns, staged in the warp's 4 KB of output staging by the lanes that hold the rows and
+// Chunks of the 8-warp epilogues: kRows of the warp's 32 rows x kCols of its fp32 columns
+// (half of the tile's: 128 or 64), staged in the warp's 4 KB of output staging by the lanes that hold the rows and
 // read back with kLanes lanes to a row, 4 columns each, so that every global access of a
 // warp covers kCols consecutive columns of kAccRows rows.  16-byte pieces are swizzled by
 // row, so neither side has bank conflicts.
@@ -160,10 +160,6 @@ struct RowChunk {
     static constexpr int kLanes = kCols / 4;
     static constexpr int kAccRows = 32 / kLanes;           // rows of one access
     static constexpr int kAcc = kRows / kAccRows;          // accesses per chunk (8)
-    static constexpr int kTileCols = 128;                  // of a 256-column tile, per warp
-    static constexpr int kColGroups = kTileCols / kCols;
-    static constexpr int kChunks = 32 / kRows * kColGroups;
-
     static __device__ __forceinline__ uint32_t piece(uint32_t buf, uint32_t r, uint32_t c) {
         return buf + r * (kCols * 4u) + ((c ^ (r & 7u)) << 4);
     }
@@ -192,7 +188,7 @@ struct RowChunk {
 // v[32], column, offset in the tile, io); finish(params, n_block)).  With 8, two warps
 // share the rows and take half of the columns each, and every chunk goes through the warp's
 // staging buffer (RowChunk; Epi(params, group, first row, first column, lane);
-// chunk(params, staged chunk, lane, chunk index); finish(params, n_block, lane)).  The functor
+// chunk(params, staged chunk, lane, chunk index); finish(params, lane)).  The functor
 // is made before the accumulator is awaited, so that what its constructor loads arrives
 // during the mainloop.  `ready` waits for the accumulator (false: give up), `release`
 // gives it back once its last columns are in registers.
@@ -215,25 +211,27 @@ __device__ __forceinline__ bool epilogue_tile(const typename Epi::Params& ep, in
         epi.finish(ep, nb);
     } else {
         using R = RowChunk;
-        static_assert(BN == 256, "the 8-warp epilogues split 256 columns");
-        const int c0 = warp_half * R::kTileCols;
+        constexpr int kWarpCols = BN / 2, kColGroups = Epi::kColGroups;
+        static_assert(kWarpCols == kColGroups * R::kCols, "the epilogue's share of the columns");
+        constexpr int kChunks = 32 / R::kRows * kColGroups;
+        const int c0 = warp_half * kWarpCols;
         Epi epi(ep, g, row0, nb * BN + c0, io.lane);
         if (!ready()) return false;
 #pragma unroll 1
-        for (int c = 0; c < R::kChunks; ++c) {
+        for (int c = 0; c < kChunks; ++c) {
             // every lane reads its row's columns again for each row group
 #pragma unroll 1
             for (int h = 0; h < R::kCols / 32; ++h) {
                 float v[32];
-                tmem_ld_32x32b_x32(t_row + c0 + (c % R::kColGroups) * R::kCols + 32 * h, v);
-                if (c == R::kChunks - 1 && h == R::kCols / 32 - 1) release();
-                R::stage(io.out, io.lane, c / R::kColGroups, h, v);
+                tmem_ld_32x32b_x32(t_row + c0 + (c % kColGroups) * R::kCols + 32 * h, v);
+                if (c == kChunks - 1 && h == R::kCols / 32 - 1) release();
+                R::stage(io.out, io.lane, c / kColGroups, h, v);
                 __syncwarp();
             }
             epi.chunk(ep, io.out, io.lane, c);
             __syncwarp();
         }
-        epi.finish(ep, nb, io.lane);
+        epi.finish(ep, io.lane);
     }
     return true;
 }

@@ -31,7 +31,8 @@
 // TMEM (512 columns) is allocated collectively by warp 1 of both CTAs.
 //
 // BN is 256 (two accumulator buffers of 256 columns: the epilogue of one tile
-// overlaps the mainloop of the next) or 512 (two N=256 MMAs per K slice into
+// overlaps the mainloop of the next), 128 (the same, for problems of few tiles: twice as
+// many SMs share the epilogue) or 512 (two N=256 MMAs per K slice into
 // one 512-column accumulator: a quarter less operand traffic per FLOP, but the
 // next tile waits for the epilogue; for GEMMs with a long K loop).
 // All waits are bounded as in the single-CTA kernel.  Teardown: the pair meets at
@@ -50,7 +51,7 @@ constexpr int kPairBM = 256;  // output rows of one pair tile
 // 64-deep k-blocks per pipeline stage of a BN-column pair tile.
 template <int BN, bool A_MN, bool B_MN>
 constexpr int pair_ksub() {
-    return BN == 256 ? 2 : 1;
+    return BN <= 256 ? 2 : 1;
 }
 
 template <int BN, int STAGES, int KSUB>
@@ -222,15 +223,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<Epi>(),
     tc_gemm_pair_kernel(const __grid_constant__ GemmMaps<MAXG> maps,
                         const __grid_constant__ typename Epi::Params ep, const GemmShape sh_in,
                         unsigned int* status, unsigned long long wait_limit_ns) {
-    static_assert(BN == 256 || BN == 512, "pair tiles are 256 or 512 columns wide");
+    static_assert(BN == 128 || BN == 256 || BN == 512, "widths of pair tiles");
     using L = GemmPairSmem<BN, STAGES, pair_ksub<BN, A_MN, B_MN>()>;
     constexpr int kSub = L::kSub;                  // 64-deep k-blocks per stage
-    constexpr int kNSub = BN / 256;                // N = 256 MMAs per K slice
+    constexpr int kMmaN = BN < 256 ? BN : 256;     // columns of one MMA
+    constexpr int kNSub = BN / kMmaN;              // MMAs per K slice
     constexpr int kAccBufs = kNSub == 1 ? 2 : 1;   // accumulator buffers in TMEM
-    constexpr int kBSub = 128;                     // B columns per CTA per N = 256 MMA
+    constexpr int kBSub = kMmaN / 2;               // B columns per CTA per MMA
     constexpr uint32_t kBSubBytes = kBSub * kBK * 2;
-    constexpr uint32_t kIdesc = idesc_bf16_f32(kPairBM, 256, A_MN, B_MN);
-    constexpr int kTmemCols = kAccBufs * BN;       // 512 either way
+    constexpr uint32_t kIdesc = idesc_bf16_f32(kPairBM, kMmaN, A_MN, B_MN);
+    constexpr int kTmemCols = kAccBufs * BN;       // 512, or 256 for 128-column tiles
     constexpr uint16_t kBoth = 0x3;                // both CTAs of the pair
 
     GemmShape sh = sh_in;
@@ -333,7 +335,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<Epi>(),
 #pragma unroll
                         for (int h = 0; h < kNSub; ++h)
                             load_operand_pair<B_MN, kBSub>(
-                                bmap, sb + j * L::kBBytes + h * kBSubBytes, fb, b_row + 256 * h, k0);
+                                bmap, sb + j * L::kBBytes + h * kBSubBytes, fb, b_row + kMmaN * h, k0);
                     }
                     ++issued;
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -370,7 +372,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<Epi>(),
 #pragma unroll
                             for (int h = 0; h < kNSub; ++h)
                                 tc_mma_bf16_pair(
-                                    d_tmem + 256u * h, operand_desc<A_MN>(sa + j * L::kABytes, kk),
+                                    d_tmem + kMmaN * h, operand_desc<A_MN>(sa + j * L::kABytes, kk),
                                     operand_desc<B_MN>(sb + j * L::kBBytes + h * kBSubBytes, kk),
                                     kIdesc, (kb != kb0 || j != 0 || kk != 0) ? 1u : 0u);
                         issued_any = true;

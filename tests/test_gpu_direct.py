@@ -329,3 +329,37 @@ def test_logits_kernel_by_row_blocks(fpo, T):
     for o in outs[1:]:
         for k in ("g", "lse", "loss"):
             assert torch.equal(outs[0][k], o[k]), k
+
+
+@pytest.mark.parametrize("layers", [19, 20])
+@pytest.mark.parametrize("d_ff", [264, 392, 512])
+def test_grouped_gemms_on_half_tiles(fpo, layers, d_ff):
+    """38 tiles of 256 x 256 (19 layers of two) still leave a pair cluster for each half and
+    run as tiles of 128 columns on a 152-SM device, 40 do not; 264 and 392 columns leave a
+    half outside, or a quarter inside, the last tile.  Update and cosines agree with the
+    single-CTA kernel bit for bit either way (same sums per element and per slot)."""
+    T, d = 72, 136
+    gen = torch.Generator(device="cuda").manual_seed(layers + d_ff)
+    rn = lambda *s: torch.randn(*s, device="cuda", generator=gen)  # noqa: E731
+    g = (rn(T, d) * 1e-2).to(torch.bfloat16)
+    A = [rn(T, d_ff).to(torch.bfloat16) for _ in range(layers)]
+    Y = [rn(d, d_ff).to(torch.bfloat16) for _ in range(layers)]
+    W0 = [0.02 * rn(d, d_ff) for _ in range(layers)]
+    prev = fpo.set_gemm_variant(0)
+    outs = []
+    try:
+        for v in (0, 2):
+            fpo.set_gemm_variant(v)
+            Wm = [w.clone() for w in W0]
+            Wo = [torch.empty(d, d_ff, dtype=torch.bfloat16, device="cuda") for _ in A]
+            Go = [torch.empty_like(w) for w in Wo]
+            ws = fpo.layer_update_grouped(g, A, 1e-3, W_masters=Wm, W_outs=Wo, G_outs=Go)
+            assert fpo.get_device_status(ws) == fpo.OK
+            Gc = [torch.empty_like(w) for w in Wo]
+            outs.append(Wm + Wo + Go + Gc + [fpo.layer_grad_cosine_grouped(g, A, Y, Gc)])
+    finally:
+        fpo.set_gemm_variant(prev)
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)
+    ref = f64(g).T @ f64(A[-1])
+    assert rel_frob(f64(outs[1][3 * layers - 1]), ref) < 4e-3  # bf16 rounding of G
