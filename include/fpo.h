@@ -457,8 +457,8 @@ size_t fpo_layer_grad_cosine_workspace(int32_t n_layers, int64_t d, int64_t d_ff
  *   out[4 l + {0,1,2,3}] = <G_l, Y_l>, ||G_l||^2, ||Y_l||^2, cos_l   of the stored G_l
  *                                                        (cos = 0 if a norm is 0)
  * with Y_l [d, d_ff] (dtype) the gradient G_l is compared with.  bf16: the GEMM's
- * epilogue adds up the three sums as it writes G_l (per tile and warp, in fp32 over a
- * warp's 32 x 256 block, then in fp64 in a fixed order), so G_l is not read back; fp32:
+ * epilogue adds up the three sums as it writes G_l (in fp32 over each 32 x 64 block of a
+ * tile, then in fp64 in a fixed order), so G_l is not read back; fp32:
  * the update writes G_l and fpo_cosine_grouped reduces it.
  * g [T, d], A_l [T, d_ff] (dtype); 1 <= n_layers <= FPO_MAX_GROUPED_LAYERS; pointers
  * 16-byte aligned, out (device, 4 x n_layers fp64) 8-byte aligned; bf16 needs d and d_ff

@@ -379,7 +379,7 @@ int band_for(bool) {
 // Whether a GEMM of `tiles` 256 x 256 pair tiles runs on tiles of 128 columns instead: when
 // twice as many tiles still have a cluster each.  What bounds so small a GEMM is the
 // epilogue's traffic through one SM (32 bytes a clock to L2), which twice as many SMs share.
-// T 200, d 256, d_ff 384, V 1024, 2 layers: update 13.1 -> 9.9 us, projection 15.1 -> 12.6.
+// T 200, d 256, d_ff 384, V 1024, 2 layers: update 13.1 -> 9.5 us, projection 15.1 -> 12.1.
 bool half_tiles(long long tiles) {
     DevInfo di;
     return current_device_info(&di) && 2 * tiles <= di.sm_count / 2;
