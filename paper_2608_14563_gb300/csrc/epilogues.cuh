@@ -394,6 +394,16 @@ struct EpiStoreF32 {
 };
 
 // ---------------------------------------------------------------------------
+// Every tile split over K: the pair kernel stores the parts itself and no tile is whole.
+struct EpiParts {
+    static constexpr int kWarps = 4;
+    struct Params {};
+    __device__ __forceinline__ EpiParts(const Params&, int, int, int) {}
+    __device__ __forceinline__ void chunk(const Params&, const float (&)[32], int, int, EpiIO&) {}
+    __device__ __forceinline__ void finish(const Params&, int) {}
+};
+
+// ---------------------------------------------------------------------------
 // Projection of the direct algorithm with the final-norm VJP (App. E,
 // Eq. rmsnorm-vjp) fused in.  With acc = P W_U (target column of P zero), the
 // unnormalised error signal of token t is

@@ -279,6 +279,29 @@ struct VjpArgs {
     float min_rms, inv_d;
 };
 
+// N summed columns from n of a row of P W_U to those of g~.
+template <int N>
+__device__ __forceinline__ void vjp_row(const VjpArgs& va, int row, int n, int d,
+                                        const float (&acc)[N], float (&o)[N]) {
+    const float a = va.alpha[row], bb = va.beta[row];
+    const float rr = va.rho[row];
+    const float kd = va.cv[row] * va.inv_d;
+    const float pref = 1.0f / fmaxf(rr, va.min_rms);
+    // the same association as EpiProjVjp: w (a pref sum + b pref W_U[y]) - h (kd pref / rho)
+    const float ap = a * pref, bp = bb * pref, nk = -(kd * (1.0f / rr)) * pref;
+    const __nv_bfloat16* wy =
+        (a != 0.f && bb != 0.f) ? va.W_U + static_cast<long long>(va.y[row]) * d : nullptr;
+    const __nv_bfloat16* hr = va.h + static_cast<long long>(row) * d;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        const float yv = wy ? __bfloat162float(wy[n + j]) : 0.f;
+        const float t = fmaf(bp, yv, ap * acc[j]);
+        o[j] = a == 0.f ? 0.f
+                        : fmaf(__bfloat162float(va.w[n + j]), t,
+                               nk * __bfloat162float(hr[n + j]));
+    }
+}
+
 template <int BN>
 __global__ void __launch_bounds__(kFixupThreads)
     sk_fixup_vjp_kernel(const GemmShape sh, const float* __restrict__ scratch,
@@ -288,24 +311,8 @@ __global__ void __launch_bounds__(kFixupThreads)
     int row, n;
     float s4[4];
     if (!sk_tail_sum<BN>(sh, scratch, row, n, s4)) return;
-    const float a = va.alpha[row], bb = va.beta[row];
-    const float rr = va.rho[row];
-    const float kd = va.cv[row] * va.inv_d;
-    const float pref = 1.0f / fmaxf(rr, va.min_rms);
-    // the same association as EpiProjVjp: w (a pref sum + b pref W_U[y]) - h (kd pref / rho)
-    const float ap = a * pref, bp = bb * pref, nk = -(kd * (1.0f / rr)) * pref;
-    const __nv_bfloat16* wy =
-        (a != 0.f && bb != 0.f) ? va.W_U + static_cast<long long>(va.y[row]) * sh.N : nullptr;
-    const __nv_bfloat16* hr = va.h + static_cast<long long>(row) * sh.N;
     float o[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const float yv = wy ? __bfloat162float(wy[n + j]) : 0.f;
-        const float t = fmaf(bp, yv, ap * s4[j]);
-        o[j] = a == 0.f ? 0.f
-                        : fmaf(__bfloat162float(va.w[n + j]), t,
-                               nk * __bfloat162float(hr[n + j]));
-    }
+    vjp_row<4>(va, row, n, sh.N, s4, o);
     *reinterpret_cast<uint2*>(out + static_cast<size_t>(row) * sh.N + n) =
         make_uint2(pack_bf16x2(o[0], o[1]), pack_bf16x2(o[2], o[3]));
 }
@@ -337,6 +344,69 @@ cudaError_t launch_sk_fixup_vjp(const SkPlan& plan, const GemmShape& sh, const f
     if (plan.tail_tiles <= 0) return cudaSuccess;
     return launch_chained(sk_fixup_vjp_kernel<BN>, sk_fixup_grid<BN>(plan), kFixupThreads, 0, st,
                           sk_fixup_shape(plan, sh), scratch, static_cast<__nv_bfloat16*>(out), va);
+}
+
+// Fixup of the projection computed with its tokens along N (run_proj_tokens_n): the parts are
+// [d, tokens] tiles of 256 x BN.  A block sums 64 d x 32 tokens in range order, turns them
+// around in shared memory and writes 8 columns of a token per thread.  kVjp: out is bf16
+// g~ as above; else fp32 g.
+constexpr int kTurnD = 64, kTurnT = 32;
+
+template <int BN, bool kVjp>
+__global__ void __launch_bounds__(kFixupThreads)
+    sk_fixup_turn_kernel(const GemmShape sh, const float* __restrict__ scratch,
+                         void* __restrict__ out, const VjpArgs va) {
+    static_assert(kTurnD * kTurnT == 8 * kFixupThreads && BN % kTurnT == 0, "8 elements per thread");
+    __shared__ float tile[kTurnT][kTurnD + 1];
+    grid_dependency_trigger();
+    grid_dependency_wait();
+    const long long R = sh.tail_tiles;
+    int g, mb, nb;
+    tile_coords(blockIdx.x, sh, g, mb, nb);
+    const int d0 = blockIdx.y * kTurnD, t0 = blockIdx.z * kTurnT;  // in the tile
+    if (mb * kPairBM + d0 >= sh.M || nb * BN + t0 >= sh.N) return;
+    const int r = threadIdx.x / 8, c = threadIdx.x % 8;
+    float4 s[2] = {};
+    const float* p = scratch + (static_cast<size_t>(blockIdx.x) * kPairBM + d0 + r) * BN + t0 + 4 * c;
+    const size_t step = static_cast<size_t>(R) * kPairBM * BN;  // one range to the next
+#pragma unroll 4
+    for (int q = 0; q < sh.tail_split; ++q) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const float4 u = *reinterpret_cast<const float4*>(p + q * step + 32 * i * BN);
+            s[i].x += u.x;
+            s[i].y += u.y;
+            s[i].z += u.z;
+            s[i].w += u.w;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        tile[4 * c][r + 32 * i] = s[i].x;
+        tile[4 * c + 1][r + 32 * i] = s[i].y;
+        tile[4 * c + 2][r + 32 * i] = s[i].z;
+        tile[4 * c + 3][r + 32 * i] = s[i].w;
+    }
+    __syncthreads();
+    const int row = nb * BN + t0 + r;           // token
+    const int n = mb * kPairBM + d0 + 8 * c;    // column of g; d is a multiple of 8
+    if (row >= sh.N || n >= sh.M) return;
+    float acc[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[j] = tile[r][8 * c + j];
+    if constexpr (!kVjp) {
+        float4* o = reinterpret_cast<float4*>(static_cast<float*>(out) +
+                                              static_cast<size_t>(row) * sh.M + n);
+        o[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        o[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+    } else {
+        float o[8];
+        vjp_row<8>(va, row, n, sh.M, acc, o);
+        *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(out) +
+                                  static_cast<size_t>(row) * sh.M + n) =
+            make_uint4(pack_bf16x2(o[0], o[1]), pack_bf16x2(o[2], o[3]), pack_bf16x2(o[4], o[5]),
+                       pack_bf16x2(o[6], o[7]));
+    }
 }
 
 constexpr int kProjBN = 256;     // projection tiles where 512 columns are too wide
@@ -442,26 +512,69 @@ int proj_clusters() {
 // 333 x 4096 x 100352 (16 tiles of 512 columns on 76 clusters) 887 us whole, 246 us in 7
 // ranges; 2048 x 2048 x 50304 (32 such tiles) 434 us, 276 in 7 ranges of 256 columns and
 // about the same in whole 256-column tiles, which draw less power (step 818 and 777 us).
-int proj_split(int T, int d, int V) {
+//
+// The split projection can also run the other way around, g^T = W_U^T P^T with the tokens
+// along N, in 256 x 384 tiles: a 64-deep k-block takes 560 ns, but 40 KB of operands per SM
+// serve up to 384 tokens where two 256 x 256 tiles take 64 KB.  The costs choose it where
+// about a third of the other form's rows would be empty.  Error signal, T x d x V: 333 x
+// 4096 x 100352 497 -> 464 us, 333 x 2048 x 50304 182 -> 172, 1100 x 4096 x 100352 1234 ->
+// 1120; 512 x 4096 x 100352 would take 629 instead of 535, 768 x 4096 x 100352 the same.
+struct ProjPlan {
+    int split = 0;          // K ranges per tile; 0: whole 512-column tiles
+    bool tokens_n = false;
+};
+
+constexpr int kTurnBN = 384;     // tokens of a tile with the tokens along N
+constexpr int kTurnStages = 4;   // 40 KB stages
+
+ProjPlan proj_plan(int T, int d, int V) {
     const long long clusters = proj_clusters();
     const long long m_blocks = (T + kPairBM - 1) / kPairBM;
-    if (m_blocks * ((d + kWideBN - 1) / kWideBN) >= clusters) return 0;
+    ProjPlan best;
+    if (m_blocks * ((d + kWideBN - 1) / kWideBN) >= clusters) return best;
     const int kb = (V + kBK - 1) / kBK;
-    const long long tiles = m_blocks * ((d + kProjBN - 1) / kProjBN);
-    const long long cap = kTailWaves * clusters * (kWideBN / kProjBN);  // units of scratch
     double best_cost = 0.0;
-    int best = 1;
-    for (int S = 1; S <= 64; ++S) {
-        if (S > 1 && (kb / S < 32 || tiles * S > cap)) break;
-        const double waves = static_cast<double>((tiles * S + clusters - 1) / clusters);
-        double cost = waves * ((kb + S - 1) / S) * 344.0;
-        if (S > 1) cost += waves * 2500.0 + 4000.0 + tiles * S * (kProjBN * 1024.0) / 4300.0;
-        if (S == 1 || cost < best_cost) {
-            best_cost = cost;
-            best = S;
+    auto consider = [&](bool tokens_n, long long tiles, int width, double k_block_ns) {
+        const long long cap = kTailWaves * clusters * kWideBN / width;  // units of scratch
+        for (int S = tokens_n ? 2 : 1; S <= 64; ++S) {
+            if (S > 1 && (kb / S < 32 || tiles * S > cap)) break;
+            const double waves = static_cast<double>((tiles * S + clusters - 1) / clusters);
+            double cost = waves * ((kb + S - 1) / S) * k_block_ns;
+            if (S > 1) cost += waves * 2500.0 + 4000.0 + tiles * S * (width * 1024.0) / 4300.0;
+            if (best.split == 0 || cost < best_cost) {
+                best_cost = cost;
+                best.split = S;
+                best.tokens_n = tokens_n;
+            }
         }
-    }
+    };
+    consider(false, m_blocks * ((d + kProjBN - 1) / kProjBN), kProjBN, 344.0);
+    consider(true, ((d + kPairBM - 1) / kPairBM) * static_cast<long long>((T + kTurnBN - 1) / kTurnBN),
+             kTurnBN, 560.0);
     return best;
+}
+
+ProjPlan proj_plan(int T_all, int Tc, int d, int V) {
+    const ProjPlan p = proj_plan(T_all, d, V);
+    return p.split ? p : proj_plan(Tc, d, V);  // a short chunk of a large batch
+}
+
+// The split projection with the tokens along N, and its fixup.
+template <bool kVjp>
+cudaError_t run_proj_tokens_n(const void* E, const void* W_U, int Tc, int d, int V, int split,
+                              float* sk_scratch, void* out, const VjpArgs& va, unsigned* status,
+                              cudaStream_t st) {
+    GemmMaps<1> maps;
+    if (!map_mnmajor(&maps.a[0], W_U, V, d) || !map_kmajor(&maps.b[0], E, Tc, V, kTurnBN / 4))
+        return cudaErrorInvalidValue;
+    const GemmShape sh = make_shape(d, Tc, V, kTurnBN, 1, band_for(true), kPairBM);
+    SkPlan plan;
+    const cudaError_t e = run_gemm_pair<kTurnBN, true, false, kTurnStages, 1, EpiParts>(
+        maps, EpiParts::Params{}, sh, status, st, sk_scratch, &plan, split);
+    if (e != cudaSuccess || plan.tail_tiles <= 0) return e;
+    const dim3 grid(static_cast<unsigned>(plan.tail_tiles), kPairBM / kTurnD, kTurnBN / kTurnT);
+    return launch_chained(sk_fixup_turn_kernel<kTurnBN, kVjp>, grid, kFixupThreads, 0, st,
+                          sk_fixup_shape(plan, sh), static_cast<const float*>(sk_scratch), out, va);
 }
 
 }  // namespace
@@ -627,9 +740,11 @@ cudaError_t launch_proj_vjp_bf16(const void* P, const void* W_U, const int32_t* 
     ep.N = d;
     if (wide_proj()) {
         SkPlan plan;
-        int split = proj_split(T_all, d, V);
-        if (split == 0) split = proj_split(Tc, d, V);  // a short chunk of a large batch
-        if (split == 0) {
+        const ProjPlan pp = proj_plan(T_all, Tc, d, V);
+        if (pp.tokens_n)
+            return run_proj_tokens_n<true>(P, W_U, Tc, d, V, pp.split, sk_scratch, g_tilde, va,
+                                           status, st);
+        if (pp.split == 0) {
             ep.tile_n = kWideBN;
             const GemmShape sh = make_shape(Tc, d, V, kWideBN, 1, band_for(true), kPairBM);
             const cudaError_t e = run_gemm_pair<kWideBN, false, true, kWideStages, 1, EpiProjVjp>(
@@ -638,14 +753,14 @@ cudaError_t launch_proj_vjp_bf16(const void* P, const void* W_U, const int32_t* 
             return launch_sk_fixup_vjp<kWideBN>(plan, sh, sk_scratch, g_tilde, va, st);
         }
         const GemmShape sh = make_shape(Tc, d, V, kProjBN, 1, band_for(true), kPairBM);
-        if (split == 1 && half_tiles(sh.tiles)) {
+        if (pp.split == 1 && half_tiles(sh.tiles)) {
             ep.tile_n = kHalfBN;
             return run_gemm_pair<kHalfBN, false, true, kHalfStages, 1, EpiProjVjp>(
                 maps, ep, make_shape(Tc, d, V, kHalfBN, 1, band_for(true), kPairBM), status, st);
         }
         ep.tile_n = kProjBN;
         const cudaError_t e = run_gemm_pair<kProjBN, false, true, kPairStages, 1, EpiProjVjp>(
-            maps, ep, sh, status, st, split > 1 ? sk_scratch : nullptr, &plan, split);
+            maps, ep, sh, status, st, pp.split > 1 ? sk_scratch : nullptr, &plan, pp.split);
         if (e != cudaSuccess) return e;
         return launch_sk_fixup_vjp<kProjBN>(plan, sh, sk_scratch, g_tilde, va, st);
     }
@@ -668,9 +783,11 @@ cudaError_t launch_proj_bf16(const void* E, const void* W_U, int Tc, int T_all, 
     ep.N = d;
     if (wide_proj()) {
         SkPlan plan;
-        int split = proj_split(T_all, d, V);
-        if (split == 0) split = proj_split(Tc, d, V);  // a short chunk of a large batch
-        if (split == 0) {
+        const ProjPlan pp = proj_plan(T_all, Tc, d, V);
+        if (pp.tokens_n)
+            return run_proj_tokens_n<false>(E, W_U, Tc, d, V, pp.split, sk_scratch, g, VjpArgs{},
+                                            status, st);
+        if (pp.split == 0) {
             const GemmShape sh = make_shape(Tc, d, V, kWideBN, 1, band_for(true), kPairBM);
             const cudaError_t e = run_gemm_pair<kWideBN, false, true, kWideStages, 1, EpiStoreF32>(
                 maps, ep, sh, status, st, sk_scratch, &plan);
@@ -679,7 +796,7 @@ cudaError_t launch_proj_bf16(const void* E, const void* W_U, int Tc, int T_all, 
         }
         const GemmShape sh = make_shape(Tc, d, V, kProjBN, 1, band_for(true), kPairBM);
         const cudaError_t e = run_gemm_pair<kProjBN, false, true, kPairStages, 1, EpiStoreF32>(
-            maps, ep, sh, status, st, split > 1 ? sk_scratch : nullptr, &plan, split);
+            maps, ep, sh, status, st, pp.split > 1 ? sk_scratch : nullptr, &plan, pp.split);
         if (e != cudaSuccess) return e;
         return launch_sk_fixup<kProjBN>(plan, sh, sk_scratch, g, st);
     }

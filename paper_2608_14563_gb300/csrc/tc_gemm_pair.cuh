@@ -32,8 +32,8 @@
 //
 // BN is 256 (two accumulator buffers of 256 columns: the epilogue of one tile
 // overlaps the mainloop of the next), 128 (the same, for problems of few tiles: twice as
-// many SMs share the epilogue) or 512 (two N=256 MMAs per K slice into
-// one 512-column accumulator: a quarter less operand traffic per FLOP, but the
+// many SMs share the epilogue) or 384 or 512 (two MMAs per K slice into
+// one accumulator: less operand traffic per FLOP, but the
 // next tile waits for the epilogue; for GEMMs with a long K loop).
 // All waits are bounded as in the single-CTA kernel.  Teardown: the pair meets at
 // a cluster barrier, the leader waits (with a separate, fixed limit) for every
@@ -223,16 +223,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<Epi>(),
     tc_gemm_pair_kernel(const __grid_constant__ GemmMaps<MAXG> maps,
                         const __grid_constant__ typename Epi::Params ep, const GemmShape sh_in,
                         unsigned int* status, unsigned long long wait_limit_ns) {
-    static_assert(BN == 128 || BN == 256 || BN == 512, "widths of pair tiles");
+    static_assert(BN == 128 || BN == 256 || BN == 384 || BN == 512, "widths of pair tiles");
     using L = GemmPairSmem<BN, STAGES, pair_ksub<BN, A_MN, B_MN>()>;
     constexpr int kSub = L::kSub;                  // 64-deep k-blocks per stage
-    constexpr int kMmaN = BN < 256 ? BN : 256;     // columns of one MMA
+    constexpr int kMmaN = BN <= 256 ? BN : BN / 2;  // columns of one MMA
     constexpr int kNSub = BN / kMmaN;              // MMAs per K slice
     constexpr int kAccBufs = kNSub == 1 ? 2 : 1;   // accumulator buffers in TMEM
     constexpr int kBSub = kMmaN / 2;               // B columns per CTA per MMA
     constexpr uint32_t kBSubBytes = kBSub * kBK * 2;
     constexpr uint32_t kIdesc = idesc_bf16_f32(kPairBM, kMmaN, A_MN, B_MN);
-    constexpr int kTmemCols = kAccBufs * BN;       // 512, or 256 for 128-column tiles
+    constexpr int kTmemCols = BN == 128 ? 256 : 512;  // a power of two
     constexpr uint16_t kBoth = 0x3;                // both CTAs of the pair
 
     GemmShape sh = sh_in;
