@@ -519,9 +519,13 @@ int proj_clusters() {
 // about a third of the other form's rows would be empty.  Error signal, T x d x V: 333 x
 // 4096 x 100352 497 -> 464 us, 333 x 2048 x 50304 182 -> 172, 1100 x 4096 x 100352 1234 ->
 // 1120; 512 x 4096 x 100352 would take 629 instead of 535, 768 x 4096 x 100352 the same.
+//
+// Ranges of 256 x 512 tiles (670 ns a k-block, and 5000 for the store, which the next unit
+// of their single accumulator waits for) leave half as many parts to add: 200 x 4096 x
+// 100352 350 -> 338 us, 200 x 5120 x 152064 600 -> 570, 600 x 4096 x 100352 715 -> 695.
 struct ProjPlan {
-    int split = 0;          // K ranges per tile; 0: whole 512-column tiles
-    bool tokens_n = false;
+    int split = 0;        // K ranges per tile; 0: whole 512-column tiles
+    int width = kWideBN;  // columns of a tile: of g, or kTurnBN tokens
 };
 
 constexpr int kTurnBN = 384;     // tokens of a tile with the tokens along N
@@ -534,23 +538,24 @@ ProjPlan proj_plan(int T, int d, int V) {
     if (m_blocks * ((d + kWideBN - 1) / kWideBN) >= clusters) return best;
     const int kb = (V + kBK - 1) / kBK;
     double best_cost = 0.0;
-    auto consider = [&](bool tokens_n, long long tiles, int width, double k_block_ns) {
+    auto consider = [&](int width, long long tiles, double k_block_ns, double store_ns) {
         const long long cap = kTailWaves * clusters * kWideBN / width;  // units of scratch
-        for (int S = tokens_n ? 2 : 1; S <= 64; ++S) {
+        for (int S = width == kProjBN ? 1 : 2; S <= 64; ++S) {
             if (S > 1 && (kb / S < 32 || tiles * S > cap)) break;
             const double waves = static_cast<double>((tiles * S + clusters - 1) / clusters);
             double cost = waves * ((kb + S - 1) / S) * k_block_ns;
-            if (S > 1) cost += waves * 2500.0 + 4000.0 + tiles * S * (width * 1024.0) / 4300.0;
+            if (S > 1) cost += waves * store_ns + 4000.0 + tiles * S * (width * 1024.0) / 4300.0;
             if (best.split == 0 || cost < best_cost) {
                 best_cost = cost;
                 best.split = S;
-                best.tokens_n = tokens_n;
+                best.width = width;
             }
         }
     };
-    consider(false, m_blocks * ((d + kProjBN - 1) / kProjBN), kProjBN, 344.0);
-    consider(true, ((d + kPairBM - 1) / kPairBM) * static_cast<long long>((T + kTurnBN - 1) / kTurnBN),
-             kTurnBN, 560.0);
+    consider(kProjBN, m_blocks * ((d + kProjBN - 1) / kProjBN), 344.0, 2500.0);
+    consider(kWideBN, m_blocks * ((d + kWideBN - 1) / kWideBN), 670.0, 5000.0);
+    consider(kTurnBN, ((d + kPairBM - 1) / kPairBM) * static_cast<long long>((T + kTurnBN - 1) / kTurnBN),
+             560.0, 2500.0);
     return best;
 }
 
@@ -741,14 +746,14 @@ cudaError_t launch_proj_vjp_bf16(const void* P, const void* W_U, const int32_t* 
     if (wide_proj()) {
         SkPlan plan;
         const ProjPlan pp = proj_plan(T_all, Tc, d, V);
-        if (pp.tokens_n)
+        if (pp.width == kTurnBN)
             return run_proj_tokens_n<true>(P, W_U, Tc, d, V, pp.split, sk_scratch, g_tilde, va,
                                            status, st);
-        if (pp.split == 0) {
+        if (pp.width == kWideBN) {
             ep.tile_n = kWideBN;
             const GemmShape sh = make_shape(Tc, d, V, kWideBN, 1, band_for(true), kPairBM);
             const cudaError_t e = run_gemm_pair<kWideBN, false, true, kWideStages, 1, EpiProjVjp>(
-                maps, ep, sh, status, st, sk_scratch, &plan);
+                maps, ep, sh, status, st, sk_scratch, &plan, pp.split);
             if (e != cudaSuccess) return e;
             return launch_sk_fixup_vjp<kWideBN>(plan, sh, sk_scratch, g_tilde, va, st);
         }
@@ -784,13 +789,13 @@ cudaError_t launch_proj_bf16(const void* E, const void* W_U, int Tc, int T_all, 
     if (wide_proj()) {
         SkPlan plan;
         const ProjPlan pp = proj_plan(T_all, Tc, d, V);
-        if (pp.tokens_n)
+        if (pp.width == kTurnBN)
             return run_proj_tokens_n<false>(E, W_U, Tc, d, V, pp.split, sk_scratch, g, VjpArgs{},
                                             status, st);
-        if (pp.split == 0) {
+        if (pp.width == kWideBN) {
             const GemmShape sh = make_shape(Tc, d, V, kWideBN, 1, band_for(true), kPairBM);
             const cudaError_t e = run_gemm_pair<kWideBN, false, true, kWideStages, 1, EpiStoreF32>(
-                maps, ep, sh, status, st, sk_scratch, &plan);
+                maps, ep, sh, status, st, sk_scratch, &plan, pp.split);
             if (e != cudaSuccess) return e;
             return launch_sk_fixup<kWideBN>(plan, sh, sk_scratch, g, st);
         }

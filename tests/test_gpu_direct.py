@@ -281,11 +281,12 @@ def test_update_is_bitwise_identical_across_gemm_kernels(fpo, shape):
 
 @pytest.mark.parametrize("algo", [2, 3])  # stored logits, direct
 @pytest.mark.parametrize("shape", [(300, 520, 8200), (33, 264, 4104), (257, 256, 20000),
-                                   (300, 2056, 20000), (337, 4104, 8200)])
+                                   (300, 2056, 20000), (337, 4104, 8200), (40, 3848, 42008)])
 def test_projection_of_a_small_batch_split_over_k(fpo, algo, shape):
     """Batches of fewer 256 x 512 projection tiles than pair clusters split every tile's K
     loop into ranges of at least 32 k-blocks (2048 vocabulary entries) and sum them in the
-    fixup kernel; the last two shapes run with the tokens along N in 384-wide tiles.  Against whole tiles (the 256 x 256 kernel), the oracle, and across
+    fixup kernel; the fourth and fifth shape run with the tokens along N in 384-wide
+    tiles, the last in ranges of 512-wide ones.  Against whole tiles (the 256 x 256 kernel), the oracle, and across
     chunkings (the split depends on the batch only); every third token is clamped."""
     T, d, V = shape
     wl = Workload("skb", T=T, d=d, d_ff=8, V=V, layers=1, targets="zipf")
