@@ -48,6 +48,14 @@ namespace fpo {
 
 constexpr int kPairBM = 256;  // output rows of one pair tile
 
+// Registers per thread of the pair kernels: what leaves room on the SM for a block of the
+// host-input copy (csrc/host_copy.cu), which runs beside them.  A quarter of the SM has 16384
+// registers for its 2 (4 epilogue warps) or 3 (8) warps of the GEMM and the copy's.
+template <class Epi>
+constexpr int pair_regs() {
+    return Epi::kWarps == 4 ? 224 : 160;
+}
+
 // 64-deep k-blocks per pipeline stage of a BN-column pair tile.
 template <int BN, bool A_MN, bool B_MN>
 constexpr int pair_ksub() {
@@ -219,7 +227,7 @@ __device__ __forceinline__ void pair_drain_copies(uint32_t bar0, long long n_sel
 }
 
 template <int BN, bool A_MN, bool B_MN, int STAGES, int MAXG, class Epi>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<Epi>(), 1)
+__global__ void __cluster_dims__(2, 1, 1) __maxnreg__(pair_regs<Epi>())
     tc_gemm_pair_kernel(const __grid_constant__ GemmMaps<MAXG> maps,
                         const __grid_constant__ typename Epi::Params ep, const GemmShape sh_in,
                         unsigned int* status, unsigned long long wait_limit_ns) {
