@@ -504,7 +504,7 @@ int32_t fpo_norm_ratio(int32_t n_layers, int64_t n, int32_t g_dtype, const void*
  * targets, the cached activations A_l) arrive in host memory.  The paper has no
  * counterpart.  One kernel launch copies every buffer; its threads read the host
  * memory through its device mapping, so the copy does not use the copy engines
- * and runs beside kernels on other streams (one 256-thread block per SM, no
+ * and runs beside kernels on other streams (one 128-thread block per SM, no
  * shared memory).
  *
  * src[i]    host, 16-byte aligned, inside page-locked memory that is mapped into
