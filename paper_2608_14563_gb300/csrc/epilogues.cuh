@@ -141,7 +141,7 @@ struct EpiAnchorProb {
         : row(row_), pair_out(false) {
         valid = row_ < p.M;
         yoff = valid ? __ldg(p.y + row_) - n0 : -1;
-        const float nc = valid ? -__ldg(p.anchor + row_) * kLog2e : 0.f;
+        const float nc = valid ? -p.anchor[row_] * kLog2e : 0.f;
         nc2 = make_float2(nc, nc);
         u0 = u1 = s0 = s1 = q0 = q1 = make_float2(0.f, 0.f);
     }
@@ -340,7 +340,7 @@ struct EpiError {
     __device__ __forceinline__ EpiError(const Params& p, int, int row_, int) : row(row_) {
         const bool valid = row_ < p.M;
         yt = valid ? __ldg(p.y + row_) : -1;
-        lse2 = valid ? __ldg(p.lse + row_) * kLog2e : 0.f;
+        lse2 = valid ? p.lse[row_] * kLog2e : 0.f;
         pair_out = false;
     }
 
@@ -461,10 +461,10 @@ struct EpiProjVjp {
     __device__ __forceinline__ EpiProjVjp(const Params& p, int, int row, int n0)
         : pair_out(false) {
         valid = row < p.M;
-        a = valid ? __ldg(p.alpha + row) : 0.f;
-        const float b = valid ? __ldg(p.beta + row) : 0.f;
-        const float r = valid ? __ldg(p.rho + row) : 1.f;
-        const float kd = valid ? __ldg(p.cv + row) * p.inv_d : 0.f;
+        a = valid ? p.alpha[row] : 0.f;
+        const float b = valid ? p.beta[row] : 0.f;
+        const float r = valid ? p.rho[row] : 1.f;
+        const float kd = valid ? p.cv[row] * p.inv_d : 0.f;
         const float pref = 1.0f / fmaxf(r, p.min_rms);
         // g~_j = w_j (a pref acc_j + b pref W_U[y]_j) - h_j (kd pref / rho)
         a2 = make_float2(a * pref, a * pref);

@@ -224,7 +224,7 @@ constexpr int kFixupThreads = 256;
 
 // The summed partials of this thread's 4 columns; false outside the matrix.
 template <int BN>
-__device__ __forceinline__ bool sk_tail_sum(const GemmShape& sh, const float* __restrict__ scratch,
+__device__ __forceinline__ bool sk_tail_sum(const GemmShape& sh, const float* scratch,
                                             int& row, int& n, float (&s4)[4]) {
     constexpr int kThreadsPerRow = BN / 4;
     constexpr int kRowsPerBlock = kFixupThreads / kThreadsPerRow;
@@ -254,7 +254,7 @@ __device__ __forceinline__ bool sk_tail_sum(const GemmShape& sh, const float* __
 // Plain fp32 sums, as EpiStoreF32 writes whole tiles (the projection g = E W_U).
 template <int BN>
 __global__ void __launch_bounds__(kFixupThreads)
-    sk_fixup_kernel(const GemmShape sh, const float* __restrict__ scratch, float* __restrict__ C) {
+    sk_fixup_kernel(const GemmShape sh, const float* scratch, float* __restrict__ C) {
     grid_dependency_trigger();
     grid_dependency_wait();
     int row, n;
@@ -304,7 +304,7 @@ __device__ __forceinline__ void vjp_row(const VjpArgs& va, int row, int n, int d
 
 template <int BN>
 __global__ void __launch_bounds__(kFixupThreads)
-    sk_fixup_vjp_kernel(const GemmShape sh, const float* __restrict__ scratch,
+    sk_fixup_vjp_kernel(const GemmShape sh, const float* scratch,
                         __nv_bfloat16* __restrict__ out, const VjpArgs va) {
     grid_dependency_trigger();
     grid_dependency_wait();
@@ -354,7 +354,7 @@ constexpr int kTurnD = 64, kTurnT = 32;
 
 template <int BN, bool kVjp>
 __global__ void __launch_bounds__(kFixupThreads)
-    sk_fixup_turn_kernel(const GemmShape sh, const float* __restrict__ scratch,
+    sk_fixup_turn_kernel(const GemmShape sh, const float* scratch,
                          void* __restrict__ out, const VjpArgs va) {
     static_assert(kTurnD * kTurnT == 8 * kFixupThreads && BN % kTurnT == 0, "8 elements per thread");
     __shared__ float tile[kTurnT][kTurnD + 1];
@@ -934,7 +934,7 @@ size_t opt_step_partial_bytes(int n_layers, int d, int d_ff) {
 // Second pass of the fused cosine: a cluster per layer adds the layer's slot triples in a
 // fixed order and writes <G, Y>, ||G||^2, ||Y||^2 and the cosine.
 __global__ void __cluster_dims__(kSlotBlocks, 1, 1) __launch_bounds__(kSlotThreads)
-    grad_cosine_final_kernel(const float* __restrict__ part, int slots, double* __restrict__ out) {
+    grad_cosine_final_kernel(const float* part, int slots, double* __restrict__ out) {
     grid_dependency_trigger();
     grid_dependency_wait();
     const int layer = blockIdx.x / kSlotBlocks;

@@ -179,7 +179,7 @@ __device__ __forceinline__ double warp_sum_f64(double x) {
     return x;
 }
 
-__global__ void grouped_final_kernel(const double* __restrict__ partial, int blocks,
+__global__ void grouped_final_kernel(const double* partial, int blocks,
                                      int n_layers, int mode, double rel,
                                      double* __restrict__ out) {
     grid_dependency_wait();

@@ -52,7 +52,12 @@ uint64_t launches();
 // is still running (programmatic dependent launch).  Every such kernel calls
 // grid_dependency_wait() in every thread before it touches memory that another kernel reads
 // or writes, and before any block of it exits: the wait ends when the kernel before has
-// completed and its writes are visible.  It calls grid_dependency_trigger() where the next
+// completed and its writes are visible.  Whatever another kernel of the chain wrote is read
+// by ordinary loads after that: no __ldg, and no const __restrict__ on the pointer, either of
+// which declares the memory unchanging for the kernel's whole life (it overlaps the writer's)
+// and so lets the compiler move the load above the wait.  Both are for the caller's inputs
+// (h, w, W_U, y, A, Y): a memset at the start of every call keeps its first kernel from
+// overlapping the caller's own.  A chained kernel calls grid_dependency_trigger() where the next
 // kernel may start taking its place: at once in short kernels, near the end in the GEMMs,
 // whose SMs would otherwise be shared with waiting blocks for milliseconds.
 template <class... P, class... A>

@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kOptThreads)
 // (||W||^2, ||d||^2) slot pairs in a fixed order and writes the layer's scale
 // min(1, clip_frac ||W|| / ||d||).
 __global__ void __cluster_dims__(kSlotBlocks, 1, 1) __launch_bounds__(kSlotThreads)
-    opt_scale_kernel(const float* __restrict__ part, int slots, const OptimParams op,
+    opt_scale_kernel(const float* part, int slots, const OptimParams op,
                      float* __restrict__ scales) {
     grid_dependency_wait();
     const int layer = blockIdx.x / kSlotBlocks;

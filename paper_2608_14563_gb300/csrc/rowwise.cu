@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(kBlkThreads)
 // its loads issued kBatch at a time (the loop waits once per batch), then a fixed butterfly
 // per warp and the warps' sums in warp order.
 template <int THREADS>
-__device__ __forceinline__ void block_mean(const float* __restrict__ x, int n,
+__device__ __forceinline__ void block_mean(const float* x, int n,
                                            float* __restrict__ out) {
     __shared__ double buf[THREADS / 32];
     constexpr int kBatch = 16;
@@ -293,7 +293,7 @@ __device__ __forceinline__ void block_mean(const float* __restrict__ x, int n,
 }
 
 // log-sum-exp of one row from its (max, sum exp) partials, by one warp; every lane gets it.
-__device__ __forceinline__ float row_lse(const float2* __restrict__ pr, int n_tiles, int lane) {
+__device__ __forceinline__ float row_lse(const float2* pr, int n_tiles, int lane) {
     float m = -INFINITY;
     for (int i = lane; i < n_tiles; i += 32) m = fmaxf(m, pr[i].x);
     m = warp_max(m);
@@ -308,10 +308,10 @@ __device__ __forceinline__ float row_lse(const float2* __restrict__ pr, int n_ti
 
 template <int EPT>
 __global__ void __launch_bounds__(kBlkThreads)
-    rmsnorm_vjp_row_kernel(const float* __restrict__ g, const __nv_bfloat16* __restrict__ h,
-                           const __nv_bfloat16* __restrict__ w, const float* __restrict__ rho,
-                           int T, int d, float min_rms, __nv_bfloat16* __restrict__ out,
-                       const float* __restrict__ ce, float* __restrict__ loss) {
+    rmsnorm_vjp_row_kernel(const float* g, const __nv_bfloat16* __restrict__ h,
+                           const __nv_bfloat16* __restrict__ w, const float* rho, int T, int d,
+                           float min_rms, __nv_bfloat16* __restrict__ out, const float* ce,
+                           float* __restrict__ loss) {
     grid_dependency_trigger();
     grid_dependency_wait();
     // the batch's mean cross-entropy beside the rows (every token's is final by now)
@@ -376,10 +376,9 @@ int blk_grid(int T) {
 
 template <typename TT, int VEC>
 __global__ void __launch_bounds__(kRowThreads)
-    rmsnorm_vjp_kernel(const float* __restrict__ g, const TT* __restrict__ h,
-                       const TT* __restrict__ w, const float* __restrict__ rho, int T, int d,
-                       float min_rms, TT* __restrict__ out,
-                       const float* __restrict__ ce, float* __restrict__ loss) {
+    rmsnorm_vjp_kernel(const float* g, const TT* __restrict__ h, const TT* __restrict__ w,
+                       const float* rho, int T, int d, float min_rms, TT* __restrict__ out,
+                       const float* ce, float* __restrict__ loss) {
     grid_dependency_trigger();
     grid_dependency_wait();
     // the batch's mean cross-entropy beside the rows (every token's is final by now)
@@ -417,8 +416,8 @@ __global__ void __launch_bounds__(kRowThreads)
 }
 
 __global__ void __launch_bounds__(kRowThreads)
-    lse_combine_kernel(const float2* __restrict__ part, int n_tiles, int T,
-                       const float* __restrict__ zy, float* __restrict__ lse, float* __restrict__ ce) {
+    lse_combine_kernel(const float2* part, int n_tiles, int T, const float* zy,
+                       float* __restrict__ lse, float* __restrict__ ce) {
     grid_dependency_trigger();
     grid_dependency_wait();
     const int lane = threadIdx.x & 31;
@@ -449,13 +448,12 @@ constexpr double kWindowHi = 1.2089258196146292e24;   // 2^80
 constexpr double kWindowLo = 8.271806125530277e-25;  // 2^-80
 
 __global__ void __launch_bounds__(kRowThreads)
-    direct_combine_kernel(const float* __restrict__ su, const float* __restrict__ sx,
-                          const float* __restrict__ qz, int n_tiles, int T, int V,
-                          const int32_t* __restrict__ y,
-                          const float* __restrict__ anchor, float s, float* __restrict__ lse,
-                          float* __restrict__ ce, float* __restrict__ alpha,
-                          float* __restrict__ beta, float* __restrict__ cv,
-                          int* __restrict__ fix, int* __restrict__ fix_count) {
+    direct_combine_kernel(const float* su, const float* sx, const float* qz, int n_tiles, int T,
+                          int V, const int32_t* __restrict__ y, const float* anchor, float s,
+                          float* __restrict__ lse, float* __restrict__ ce,
+                          float* __restrict__ alpha, float* __restrict__ beta,
+                          float* __restrict__ cv, int* __restrict__ fix,
+                          int* __restrict__ fix_count) {
     grid_dependency_trigger();
     grid_dependency_wait();
     const int lane = threadIdx.x & 31;
@@ -502,8 +500,8 @@ __global__ void __launch_bounds__(kRowThreads)
 // matrix for the tensor-core recomputation (16-byte vectors; the row count is read on
 // the device, so with no such row the launch returns at once).
 __global__ void __launch_bounds__(kRowThreads)
-    gather_rows_kernel(const uint4* __restrict__ src, const int* __restrict__ fix,
-                       const int* __restrict__ count, int v8, uint4* __restrict__ dst) {
+    gather_rows_kernel(const uint4* src, const int* fix, const int* count, int v8,
+                       uint4* __restrict__ dst) {
     grid_dependency_trigger();
     grid_dependency_wait();
     const long long n = static_cast<long long>(*count) * v8;
@@ -517,10 +515,8 @@ __global__ void __launch_bounds__(kRowThreads)
 // lse and ce of the rows outside the anchor window, from the (max, sum exp) partials of
 // the first fixup pass: lse = m + log sum_tiles s_i exp(m_i - m), ce = lse - c.
 __global__ void __launch_bounds__(kRowThreads)
-    direct_fixup_lse_kernel(const float2* __restrict__ part, const int* __restrict__ fix,
-                            const int* __restrict__ fix_count, int n_tiles,
-                            const float* __restrict__ anchor, float* __restrict__ lse,
-                            float* __restrict__ ce) {
+    direct_fixup_lse_kernel(const float2* part, const int* fix, const int* fix_count, int n_tiles,
+                            const float* anchor, float* __restrict__ lse, float* __restrict__ ce) {
     grid_dependency_trigger();
     grid_dependency_wait();
     const int lane = threadIdx.x & 31;
@@ -539,9 +535,8 @@ __global__ void __launch_bounds__(kRowThreads)
 // Row factors of the fixed rows (anchored at lse: alpha = s, beta = -s S', and the
 // VJP's row term cv = s (Qz - c S')).
 __global__ void __launch_bounds__(kRowThreads)
-    direct_fixup_factors_kernel(const float* __restrict__ sx, const float* __restrict__ qz,
-                                const int* __restrict__ fix, const int* __restrict__ fix_count,
-                                int n_tiles, const float* __restrict__ anchor, float s,
+    direct_fixup_factors_kernel(const float* sx, const float* qz, const int* fix,
+                                const int* fix_count, int n_tiles, const float* anchor, float s,
                                 float* __restrict__ alpha, float* __restrict__ beta,
                                 float* __restrict__ cv) {
     grid_dependency_trigger();
@@ -570,7 +565,7 @@ __global__ void __launch_bounds__(kRowThreads)
 
 constexpr int kMeanThreads = 512;
 
-__global__ void __launch_bounds__(kMeanThreads) mean_kernel(const float* __restrict__ x, int n,
+__global__ void __launch_bounds__(kMeanThreads) mean_kernel(const float* x, int n,
                                                             float* __restrict__ out) {
     grid_dependency_trigger();
     grid_dependency_wait();
@@ -591,8 +586,7 @@ constexpr int kErrThreads = 256;
 
 template <bool kBf16>
 __global__ void __launch_bounds__(kErrThreads)
-    error_from_logits_kernel(const float* __restrict__ z, const float2* __restrict__ part,
-                             int n_tiles, const float* __restrict__ zy,
+    error_from_logits_kernel(const float* z, const float2* part, int n_tiles, const float* zy,
                              const int32_t* __restrict__ y, int M, int V, long long ld, float s,
                              float* __restrict__ lse, float* __restrict__ ce,
                              void* __restrict__ E) {

@@ -118,7 +118,7 @@ struct SliceLoader {
     static constexpr int kLd = BT + 4;
     float4 r[kV];
 
-    __device__ __forceinline__ void load(const float* __restrict__ p, long long ld, int row0,
+    __device__ __forceinline__ void load(const float* p, long long ld, int row0,
                                          int rows, int k0, int K, bool vec) {
 #pragma unroll
         for (int q = 0; q < kV; ++q) {

@@ -24,7 +24,7 @@ __device__ __forceinline__ double ld_shared_cluster_f64(uint32_t cluster_addr) {
 // per warp, the warps' sums in order, the blocks' sums in rank order.  Every thread of the
 // cluster calls it; true in the one thread that holds the totals.
 template <int N>
-__device__ __forceinline__ bool slot_sum(const float* __restrict__ p, int slots, double (&tot)[N]) {
+__device__ __forceinline__ bool slot_sum(const float* p, int slots, double (&tot)[N]) {
     __shared__ double warp_part[kSlotThreads / 32][N];
     __shared__ double block_part[N];
     const int rank = static_cast<int>(cluster_ctarank());

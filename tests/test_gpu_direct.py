@@ -165,6 +165,43 @@ def test_rows_outside_the_anchor_window_are_fixed(fpo):
     assert abs(outs[0]["loss"].item() - oracle.mean_ce(ref["lse"], ref["zy"])) < 1e-4 * np.mean(ce)
 
 
+@pytest.mark.parametrize("t_chunk", [0, 128])
+@pytest.mark.parametrize("algo", [1, 2, 3])  # recompute, stored logits, direct
+def test_back_to_back_calls_on_one_workspace(fpo, algo, t_chunk):
+    """Each kernel is resident while the one before it still writes; a value read too early
+    (a fixup row count, a row factor, an lse) is the previous call's.  Inputs with 100, 30
+    and no rows to fix take turns on one workspace with nothing waited for in between, and
+    give the bits of calls that had the GPU and the workspace to themselves."""
+    h0, w, W_U, y0 = _window_input()
+    perm = torch.randperm(h0.shape[0], generator=torch.Generator().manual_seed(1))
+    few = [h0.clone(), y0.clone()]
+    few[0][0:70] = h0[180:250]
+    few[1][0:70] = y0[180:250]
+    none = [h0.clone(), y0.clone()]
+    none[0][0:100] = h0[150:250]
+    none[1][0:100] = y0[150:250]
+    sets = [(h0[perm], y0[perm]), tuple(few), tuple(none)]
+    alone = [run(fpo, h, w, W_U, y, eps=0.0, algo=algo, t_chunk=t_chunk) for h, y in sets]
+    if algo == 3 and t_chunk == 0:
+        assert [a["fixed"] for a in alone] == [100, 30, 0]
+    w, W_U = w.cuda(), W_U.cuda()
+    sets = [(h.cuda(), y.cuda()) for h, y in sets]
+    desc = fpo.error_signal_desc(*h0.shape, W_U.shape[0], fpo.BF16, algo=algo, t_chunk=t_chunk)
+    ws = torch.empty(fpo.error_signal_workspace(desc), dtype=torch.uint8, device="cuda")
+    turns = [k % 3 for k in range(24)] + [0, 2, 1] * 8
+    outs = [(torch.empty_like(sets[0][0]), torch.empty(h0.shape[0], device="cuda"),
+             torch.empty(1, device="cuda")) for _ in turns]
+    torch.cuda.synchronize()
+    for k, (g, lse, loss) in zip(turns, outs):
+        h, y = sets[k]
+        fpo.error_signal(h, w, W_U, y, g, eps=0.0, min_rms=0.5, t_chunk=t_chunk, lse_out=lse,
+                         loss_out=loss, algo=algo, workspace=ws)
+    assert fpo.get_device_status(ws) == fpo.OK
+    for k, (g, lse, loss) in zip(turns, outs):
+        for a, b in ((alone[k]["g"], g), (alone[k]["lse"], lse), (alone[k]["loss"], loss)):
+            assert torch.equal(a, b), k
+
+
 @pytest.mark.parametrize("variant", [0, 1, 2])
 @pytest.mark.parametrize("algo", [1, 2, 3])  # recompute, stored logits, direct
 def test_results_do_not_depend_on_workspace_contents(fpo, ragged, variant, algo):
