@@ -123,9 +123,10 @@ typedef enum fpo_status {
  * RECOMPUTE and STORED_LOGITS compute every value with the same arithmetic:
  * their outputs are bit-identical.  DIRECT agrees with them to the bf16
  * rounding of the probabilities.  Results are deterministic; across t_chunk
- * values they are bit-identical while the projection has whole tiles (fewer
- * than one wave), and otherwise agree to rounding (its last partial wave is
- * split into k ranges).
+ * values they are bit-identical while the projection of a chunk has fewer tiles
+ * (256 x 512) than one wave: it sums the whole of K, or, where the whole batch
+ * has less than a wave, the k ranges chosen from the batch.  Otherwise they agree
+ * to rounding (the last partial wave of a chunk is split into k ranges).
  */
 
 /* Tokens per error-matrix chunk when fpo_error_signal_desc.t_chunk is 0. */

@@ -506,9 +506,8 @@ int proj_clusters() {
 // that costs least.  Measured, in ns: a 64-deep k-block 344 (at the clock the tensor cores
 // hold under load), with a split 2500 per wave of units for the epilogue that stores their
 // fp32 parts, the fixup's launch 4000 and its read of the parts 4.3 bytes a ns.  Ranges
-// have at least 32 k-blocks, and the units fit the scratch.  T is the whole batch where
-// that is small, so that its sums do not depend on the chunking, and otherwise the chunk
-// (the last one of T 9000 has 808 tokens).  Projection with its fixup, T x d x V:
+// have at least 32 k-blocks, and the units fit the scratch.  T is the whole batch, so that
+// its sums do not depend on the chunking.  Projection with its fixup, T x d x V:
 // 333 x 4096 x 100352 (16 tiles of 512 columns on 76 clusters) 887 us whole, 246 us in 7
 // ranges; 2048 x 2048 x 50304 (32 such tiles) 434 us, 276 in 7 ranges of 256 columns and
 // about the same in whole 256-column tiles, which draw less power (step 818 and 777 us).
@@ -559,9 +558,22 @@ ProjPlan proj_plan(int T, int d, int V) {
     return best;
 }
 
+// A chunk of Tc of the batch's T_all tokens.  A large batch's sums run over the whole of K in
+// every chunk of less than a wave (the last one of T 9000 has 808 tokens), whichever the
+// chunking; its tiles are 256 columns wide where all of them then have a cluster at once
+// (344 against 670 ns a k-block, the same sums).  Error signal, T x d x V, in
+// 512-column tiles and so: 9000 x 4096 x 50304 4490 and 4328 us, 9000 x 2048 x 100352 4840 and
+// 4560, 9984 x 1024 x 8192 in chunks of 1024 1425 and 710.  (K ranges chosen from the chunk
+// are 0.1-1.9% faster still, 14% in the last, but make the sums depend on the chunking.)
 ProjPlan proj_plan(int T_all, int Tc, int d, int V) {
-    const ProjPlan p = proj_plan(T_all, d, V);
-    return p.split ? p : proj_plan(Tc, d, V);  // a short chunk of a large batch
+    ProjPlan p = proj_plan(T_all, d, V);
+    const long long narrow = static_cast<long long>((Tc + kPairBM - 1) / kPairBM) *
+                             ((d + kProjBN - 1) / kProjBN);
+    if (p.split == 0 && narrow <= proj_clusters()) {
+        p.split = 1;
+        p.width = kProjBN;
+    }
+    return p;
 }
 
 // The split projection with the tokens along N, and its fixup.

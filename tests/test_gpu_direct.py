@@ -349,6 +349,25 @@ def test_projection_of_a_small_batch_split_over_k(fpo, algo, shape):
     assert rel_frob(g, ref["g_tilde"]) < TOL and cos(g, ref["g_tilde"]) >= COS_MIN
 
 
+@pytest.mark.parametrize("algo", [2, 3])  # stored logits, direct
+def test_chunks_of_a_large_batch_sum_the_whole_of_k(fpo, algo):
+    """A batch of at least one wave of 256 x 512 projection tiles (78 on 76 pair clusters) in
+    chunks of less than one: the documented promise of the same bits for every such chunking,
+    also where the last chunk is short, and those of whole 256 x 256 tiles."""
+    wl = Workload("chunks", T=9984, d=1024, d_ff=8, V=8192, layers=1, targets="zipf")
+    inp = synth.make_all(wl)
+    prev = fpo.set_gemm_variant(2)
+    try:
+        runs = [run(fpo, inp["h"], inp["w"], inp["W_U"], inp["y"], eps=wl.eps, algo=algo, t_chunk=c)
+                for c in (744, 1024, 2048, 4096)]
+        fpo.set_gemm_variant(1)
+        runs.append(run(fpo, inp["h"], inp["w"], inp["W_U"], inp["y"], eps=wl.eps, algo=algo))
+    finally:
+        fpo.set_gemm_variant(prev)
+    for r in runs[1:]:
+        assert torch.equal(runs[0]["g"], r["g"])
+
+
 @pytest.mark.parametrize("T", [1, 127, 128, 129, 257, 384, 385, 513, 640, 641])
 def test_logits_kernel_by_row_blocks(fpo, T):
     """Batches of an odd number (at most 5) of 128-row blocks run the logits pass on single
