@@ -203,3 +203,19 @@ def test_block_per_row_widths(fpo, d, min_rms):
             row = np.linalg.norm(f64(outs[l]) - ref, axis=1) / np.linalg.norm(ref, axis=1)
             # bf16 results of fp32 arithmetic: half an ulp (2^-9) per element
             assert np.max(row) < 2.0 ** -8, (mode, l, int(np.argmax(row)))
+
+
+@pytest.mark.parametrize("d", [520, 4096, 8192, 12288])
+def test_rows_of_tiny_rms_without_clamp_or_eps(fpo, d):
+    """eps = 0 and min_rms = 0 with g, m and x rows of RMS 2^-70, 2^-66 and 2^-62: the two
+    prefactors are finite, and so is the result (2^58), but their product is not.  The sums'
+    terms are subnormal, exact to 2^-13 of themselves, far below the bf16 tolerance."""
+    wl = Workload("tiny-rms", T=5, d=d, d_ff=8, V=8, layers=1)
+    g, m, gp, x, gq = _case(wl, 1)
+    scaled = lambda t, e: (t.double() / t.double().pow(2).mean(1, keepdim=True).sqrt()
+                           * 2.0 ** e).to(t.dtype)  # noqa: E731
+    g, m, x = scaled(g, -70), [scaled(m[0], -66)], [scaled(x[0], -62)]
+    out = f64(_run(fpo, g, m, gp, x, gq, True, True, eps=0.0, min_rms=0.0)[0])
+    ref = _ref(g, m, gp, x, gq, True, True, 0, eps=0.0, min_rms=0.0)
+    assert np.all(np.isfinite(ref)) and np.all(np.isfinite(out))
+    assert rel_frob(out, ref) < 2e-2
