@@ -189,12 +189,18 @@ def _ptr(t):
     return t.data_ptr()
 
 
+# torch's private call for a stream's handle, where this torch has it
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream):
     if stream is not None:
         return stream.cuda_stream
     # the current stream's handle without building a torch Stream object (3 us a call, a
     # tenth of the host time of a small step)
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _nbytes(t: torch.Tensor) -> int:

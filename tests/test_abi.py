@@ -41,6 +41,23 @@ def test_library_exports_every_declared_symbol():
         assert hasattr(lib, n)
 
 
+def test_current_stream_without_the_private_call(monkeypatch):
+    """The binding takes the current stream's handle from a private call of torch; without
+    it, from the public one."""
+    import types
+    import torch
+    import paper_2608_14563_gb300 as fpo
+    public = types.SimpleNamespace(cuda_stream=0x55)
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(fpo, "_raw_stream", None, raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: public)
+    assert fpo._stream(None) == 0x55
+    assert fpo._stream(types.SimpleNamespace(cuda_stream=0x77)) == 0x77
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(fpo, "_raw_stream", lambda device: 0x100 + device)
+    assert fpo._stream(None) == 0x103
+
+
 def test_binding_loads_and_reports_version():
     import paper_2608_14563_gb300 as fpo
     assert fpo.abi_version() == 2
