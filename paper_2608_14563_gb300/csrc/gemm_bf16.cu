@@ -188,7 +188,8 @@ cudaError_t run_gemm_pair(const GemmMaps<MAXG>& maps, const typename Epi::Params
     if (plan) *plan = SkPlan{};
     if (sh_in.tiles <= 0 || sh_in.k_blocks <= 0) return cudaSuccess;
     using L = GemmPairSmem<BN, STAGES, pair_ksub<BN, A_MN, B_MN>()>;
-    static_assert(L::kBytes <= 227 * 1024, "stages exceed the shared memory of a CTA");
+    static_assert(L::kBytes + 2 * kSmemReserve <= kSmemPerSm,
+                  "the stages leave the shared memory that a block of the host-input copy takes");
     constexpr auto kern = tc_gemm_pair_kernel<BN, A_MN, B_MN, STAGES, MAXG, Epi>;
     const cudaError_t attr_err = set_smem_limit<kern>(L::kBytes);
     if (attr_err != cudaSuccess) return attr_err;

@@ -4,8 +4,8 @@
 // The copy is done by SM loads of page-locked host memory through its device
 // mapping, not by the copy engines: one launch walks a list of buffers, each
 // thread keeping four 16-byte loads in flight.  A block needs no shared memory
-// beyond the per-block reserve and 128 threads of 32 registers, so one block fits on every SM
-// beside a persistent GEMM block that uses the rest of the SM's shared memory,
+// beyond the per-block reserve and 128 threads of 32 registers, so one block fits on every
+// SM beside a persistent GEMM block that uses the rest of the SM's shared memory,
 // and the copy runs concurrently with the step on another stream.  The kernel
 // prefers the largest shared-memory carve-out, so an SM that it occupies first
 // stays configured for the GEMM blocks that follow.
@@ -18,12 +18,10 @@
 namespace fpo {
 namespace {
 
-constexpr int kCopyThreads = 128;  // one warp per quarter of the SM, with what the GEMM leaves of
-                                   // its registers (pair_regs in tc_gemm_pair.cuh)
-// 16-byte vectors in flight per thread.  Host loads take microseconds, and every one
-// in flight holds a memory request slot of its SM: with 16 KB per SM the step's kernels
-// beside the copy ran ~9% slower; 8 KB per SM still keep the at its 210 GB/s and leave them within ~1%.
-constexpr int kCopyUnroll = 4;
+// Host loads take microseconds, and every one in flight holds a memory request slot of its
+// SM: with 16 KB per SM the step's kernels beside the copy ran ~9% slower; 8 KB per SM still
+// keep the host link at its 210 GB/s and leave the kernels within ~1%.
+static_assert(kCopyThreads * kCopyUnroll * 16 == 8192, "bytes in flight per SM");
 
 struct CopySeg {
     const uint4* src;          // device mapping of the host buffer
@@ -37,7 +35,7 @@ struct CopyList {
     int n;
 };
 
-__global__ void __launch_bounds__(kCopyThreads, 16)
+__global__ void __launch_bounds__(kCopyThreads, 4 * kQuarterRegs / (kCopyThreads * kCopyRegs))
     h2d_copy_kernel(const __grid_constant__ CopyList list) {
     const unsigned long long tid =
         static_cast<unsigned long long>(blockIdx.x) * kCopyThreads + threadIdx.x;

@@ -48,6 +48,16 @@ uint64_t wait_limit_ns();
 void note_launch();
 uint64_t launches();
 
+// The host-input copy (csrc/host_copy.cu) runs beside the pair GEMMs: one of its blocks on
+// every SM, in what they leave of its registers (pair_regs, csrc/tc_gemm_pair.cuh, which
+// checks the sum) and shared memory.
+constexpr int kCopyThreads = 128;         // one warp per quarter of the SM
+constexpr int kCopyUnroll = 4;            // 16-byte loads in flight per thread
+constexpr int kCopyRegs = 32;             // registers per thread
+constexpr int kQuarterRegs = 16384;       // of a quarter of an SM
+constexpr int kSmemPerSm = 228 * 1024;    // shared memory of an SM
+constexpr int kSmemReserve = 1024;        // of every block, for the system
+
 // Launches a kernel so that it may become resident while the kernel before it in the stream
 // is still running (programmatic dependent launch).  Every such kernel calls
 // grid_dependency_wait() in every thread before it touches memory that another kernel reads

@@ -28,7 +28,7 @@
 //                       accumulator-ready barriers of BOTH CTAs (multicast)
 //   both CTAs, warps 2-   epilogue on the CTA's 128 rows (Epi::kWarps warps); arrive
 //                       on the leader's accumulator-empty barrier
-// TMEM (512 columns) is allocated collectively by warp 1 of both CTAs.
+// TMEM (512 columns; 256 for BN 128) is allocated collectively by warp 1 of both CTAs.
 //
 // BN is 256 (two accumulator buffers of 256 columns: the epilogue of one tile
 // overlaps the mainloop of the next), 128 (the same, for problems of few tiles: twice as
@@ -50,10 +50,18 @@ constexpr int kPairBM = 256;  // output rows of one pair tile
 
 // Registers per thread of the pair kernels: what leaves room on the SM for a block of the
 // host-input copy (csrc/host_copy.cu), which runs beside them.  A quarter of the SM has 16384
-// registers for its 2 (4 epilogue warps) or 3 (8) warps of the GEMM and the copy's.
+// registers for its 2 (4 epilogue warps) or 3 (8) warps of the GEMM and the copy's.  Without
+// the limit the projection took 226 and the update 168, and the copies of a step's inputs ran
+// after the projection instead of beside it (27.05 instead of 23.97 ms a step).  At 160
+// two epilogues spill a little: EpiUpdate<2> 24 bytes, EpiStoreGroupF32<2> 20.
 template <class Epi>
 constexpr int pair_regs() {
-    return Epi::kWarps == 4 ? 224 : 160;
+    constexpr int kRegs = Epi::kWarps == 4 ? 224 : 160;
+    constexpr int kGemmWarps = (2 + Epi::kWarps + 3) / 4;  // of a quarter of the SM
+    constexpr int kCopyWarps = (kCopyThreads / 32 + 3) / 4;
+    static_assert(32 * (kGemmWarps * kRegs + kCopyWarps * kCopyRegs) <= kQuarterRegs,
+                  "a block of the host-input copy fits beside a pair GEMM's");
+    return kRegs;
 }
 
 // 64-deep k-blocks per pipeline stage of a BN-column pair tile.

@@ -127,6 +127,55 @@ def test_copy_beside_a_gemm():
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("kernel", ["logits", "projection", "update"])
+def test_copy_ends_while_a_gemm_runs(kernel):
+    """A block of the copy fits beside a pair GEMM's on every SM (4 epilogue warps in the
+    logits pass and the projection, 8 in the update): a copy of 10 us that starts 0.3 to 0.6 ms
+    into a kernel of 3 ms or more ends in its first half.  Without the room it would wait for
+    the kernel's blocks to leave."""
+    src = pinned_bytes(1 << 20, 3)
+    _, dst = guarded_dst(src.numel())
+    sa, sb = torch.cuda.Stream(), torch.cuda.Stream()
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(fpo.STAGE_EVENTS)]
+    rn = lambda *s: torch.randn(*s, dtype=torch.bfloat16, device="cuda")  # noqa: E731
+    if kernel == "update":
+        g, As = rn(16384, 4096), [rn(16384, 8192) for _ in range(5)]
+        Wm = [torch.zeros(4096, 8192, device="cuda") for _ in As]
+        ws = torch.empty(4096, dtype=torch.uint8, device="cuda")
+        first, last = ev[0], ev[1]
+
+        def gemm():
+            with torch.cuda.stream(sa):
+                first.record()
+                fpo.layer_update_grouped(g, As, 1e-3, W_masters=Wm, workspace=ws)
+                last.record()
+    else:
+        T, d, V = 8192, 4096, 100352
+        h, w, W_U, g = rn(T, d), rn(d), rn(V, d), rn(T, d)
+        y = torch.zeros(T, dtype=torch.int32, device="cuda")
+        ws = torch.empty(fpo.error_signal_workspace(fpo.error_signal_desc(T, d, V)),
+                         dtype=torch.uint8, device="cuda")
+        for e in ev:
+            e.record()  # their handles exist from here on
+        first, last = (ev[1], ev[2]) if kernel == "logits" else (ev[4], ev[5])
+
+        def gemm():
+            fpo.error_signal(h, w, W_U, y, g, workspace=ws, stream=sa, stage_events=ev)
+    torch.cuda.synchronize()
+    done = torch.cuda.Event(enable_timing=True)
+    for turn in range(2):  # the first maps the host pages and loads the kernels
+        gemm()
+        sb.wait_event(first)
+        with torch.cuda.stream(sb):
+            torch.cuda._sleep(600_000)  # one thread; 0.3 to 0.6 ms at 1 to 2 GHz
+            fpo.h2d_copy([dst], [src])
+            done.record()
+        torch.cuda.synchronize()
+    assert torch.equal(dst.cpu(), src)
+    length, at = first.elapsed_time(last), first.elapsed_time(done)
+    assert length > 2.5 and at < 0.5 * length, (length, at)
+
+
 def test_host_errors():
     dst = torch.empty(4096, dtype=torch.uint8, device="cuda")
     pageable = torch.zeros(4096, dtype=torch.uint8)
