@@ -34,8 +34,9 @@ int32_t fpo_testing_gemm_bf16(int64_t M, int64_t N, int64_t K, int32_t a_mn, int
  * 0 = one CTA per 128 x 256 output tile, 1 = a CTA pair (tcgen05 cta_group::2)
  * per 256 x 256 tile, 2 = as 1 but 256 x 512 pair tiles for the projection
  * g = E W_U (one accumulator, a quarter less operand traffic; the default).
- * Any other value selects 0.  Returns the previous setting.  All compute the same sums in the same order per
- * output element.
+ * Any other value selects 0.  Returns the previous setting.  All compute the same sums in
+ * the same order per output element, except where 2 splits the projection's K (batches of
+ * less than a wave of its tiles, and the tiles of a last partial wave).
  */
 int32_t fpo_testing_set_gemm_variant(int32_t variant);
 
@@ -45,6 +46,13 @@ int32_t fpo_testing_set_gemm_variant(int32_t variant);
  * Tuning hook; results do not depend on it.
  */
 void fpo_testing_set_band(int32_t band);
+
+/*
+ * Width and height of the fp32 GEMMs' output tiles: 128 or 64, or 0 (the default) for
+ * whichever is estimated faster.  Any other value selects 0.  Returns the previous setting.
+ * Tuning hook; results do not depend on it.
+ */
+int32_t fpo_testing_set_simt_tile(int32_t tile);
 
 /*
  * Rows of the last token chunk of the most recent fpo_error_signal call on

@@ -165,6 +165,12 @@ def set_gemm_variant(variant: int) -> int:
     return _lib.fpo_testing_set_gemm_variant(int(variant))
 
 
+def set_simt_tile(tile: int) -> int:
+    """fpo_testing_set_simt_tile: fp32 GEMM tiles of 128 or 64, 0 for the estimated faster
+    (the default).  Returns the setting in force before the call."""
+    return _lib.fpo_testing_set_simt_tile(int(tile))
+
+
 def _check(code: int, where: str) -> None:
     if code != OK:
         raise FpoError(code, where)

@@ -845,6 +845,12 @@ int32_t fpo_testing_set_gemm_variant(int32_t variant) {
     return prev;
 }
 
+int32_t fpo_testing_set_simt_tile(int32_t tile) {
+    const int32_t prev = simt_tile();
+    set_simt_tile(tile);
+    return prev;
+}
+
 void fpo_testing_set_band(int32_t band) { set_band_override(band); }
 
 uint64_t fpo_testing_kernel_launches(void) { return fpo::launches(); }

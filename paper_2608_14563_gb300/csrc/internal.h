@@ -296,6 +296,9 @@ cudaError_t launch_cosine(int dtype, int64_t n, const void* X, const void* Y, do
 
 // ------------------------------------------------------------ fp32 SIMT path
 constexpr int kSimtTile = 64;  // columns of one (max, sum exp) partial
+// Output tiles of 128 or 64 for every later call, 0: by estimated time (tests).
+void set_simt_tile(int tile);
+int simt_tile();
 // T: the rows of this call (a token chunk), T_all: the rows of the whole batch, from which
 // the split of the k range is chosen (so that it does not depend on the chunking).
 // ldz, ldE: row strides of the logits and the error matrix, multiples of 4.

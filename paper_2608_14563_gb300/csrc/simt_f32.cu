@@ -19,6 +19,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include "error_math.cuh"
@@ -351,6 +352,8 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
 }
 
+std::atomic<int> g_simt_tile{0};  // > 0: tile width (tests)
+
 int sm_count() {
     DevInfo di;
     return current_device_info(&di) ? di.sm_count : 148;
@@ -422,6 +425,7 @@ cudaError_t run_tile(SimtOps ops, const Epi& ep, int groups, cudaStream_t st) {
     return e;
 }
 
+
 // Tiles of 128 or 64, whichever simt_cost estimates faster (the same sums either way).
 template <bool kAKC, bool kBKC, class Epi>
 cudaError_t run(const SimtOps& ops, const Epi& ep, int groups, cudaStream_t st) {
@@ -429,7 +433,8 @@ cudaError_t run(const SimtOps& ops, const Epi& ep, int groups, cudaStream_t st) 
     const int sms = sm_count(), slices = (ops.K + kKs - 1) / kKs;
     const double c128 = simt_cost(128, groups * simt_tiles(ops.M, ops.N, 128), slices, ops.splits, sms);
     const double c64 = simt_cost(64, groups * simt_tiles(ops.M, ops.N, 64), slices, ops.splits, sms);
-    if (c128 <= c64) return run_tile<128, kAKC, kBKC>(ops, ep, groups, st);
+    const int tile = g_simt_tile.load(std::memory_order_relaxed);
+    if (tile ? tile == 128 : c128 <= c64) return run_tile<128, kAKC, kBKC>(ops, ep, groups, st);
     return run_tile<64, kAKC, kBKC>(ops, ep, groups, st);
 }
 
@@ -451,6 +456,11 @@ SimtOps ops_of(const float* A, long long lda, const float* B, long long ldb, int
 }
 
 }  // namespace
+
+int simt_tile() { return g_simt_tile.load(std::memory_order_relaxed); }
+void set_simt_tile(int tile) {
+    g_simt_tile.store(tile == 64 || tile == 128 ? tile : 0, std::memory_order_relaxed);
+}
 
 cudaError_t launch_lse_partial_f32(const float* yhat, const float* W_U, const int32_t* y, int T,
                                    int T_all, int d, int V, float2* part, int part_ld, float* zy,

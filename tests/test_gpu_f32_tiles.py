@@ -24,8 +24,16 @@ SHAPES = [
 ]
 
 
+@pytest.fixture(params=[64, 128])
+def tile(fpo, request):
+    """Either tile width, whichever the sizes would choose (64: they are small)."""
+    fpo.set_simt_tile(request.param)
+    yield request.param
+    fpo.set_simt_tile(0)
+
+
 @pytest.mark.parametrize("shape", SHAPES, ids=["T%dd%df%dV%d" % s for s in SHAPES])
-def test_fp32_step_at_tile_edges(fpo, shape):
+def test_fp32_step_at_tile_edges(fpo, shape, tile):
     T, d, d_ff, V = shape
     wl = Workload("tiles32", T=T, d=d, d_ff=d_ff, V=V, layers=2, dtype="f32", targets="zipf",
                   lr=1e-2)
@@ -33,11 +41,16 @@ def test_fp32_step_at_tile_edges(fpo, shape):
     ref = oracle_step(wl, inp)
     runs = [gpu_step(fpo, wl, inp, algo=a, t_chunk=c) for a, c in ((2, 0), (1, 0), (2, 40))]
     check(runs[0], ref, inp, wl.lr, F32_TOL)
-    for r in runs[1:]:  # the split of K does not depend on the algorithm or the chunking
-        assert torch.equal(runs[0]["g"], r["g"]) and torch.equal(runs[0]["lse"], r["lse"])
+    fpo.set_simt_tile(192 - tile)
+    runs.append(gpu_step(fpo, wl, inp, algo=2))
+    # the order of a sum depends neither on the algorithm or the chunking nor on the tiles
+    for r in runs[1:]:
+        for a, b in zip([runs[0]["g"], runs[0]["lse"]] + runs[0]["G"] + runs[0]["W"],
+                        [r["g"], r["lse"]] + r["G"] + r["W"]):
+            assert torch.equal(a, b)
 
 
-def test_fp32_gate_up_at_tile_edges(fpo):
+def test_fp32_gate_up_at_tile_edges(fpo, tile):
     T, d, d_ff = 130, 1030, 67
     gen = torch.Generator(device="cuda").manual_seed(5)
     r = lambda *s: torch.randn(*s, device="cuda", generator=gen)  # noqa: E731
@@ -48,3 +61,19 @@ def test_fp32_gate_up_at_tile_edges(fpo):
     sg = torch.sigmoid(a.double())
     assert rel_frob(f64(dA), f64(e * b * sg * (1 + a * (1 - sg)))) < F32_TOL
     assert rel_frob(f64(dB), f64(e * a * sg)) < F32_TOL
+    fpo.set_simt_tile(192 - tile)
+    oA, oB = torch.empty_like(a), torch.empty_like(b)
+    fpo.gate_up_signals(g, W3, a, b, oA, oB)
+    assert torch.equal(dA, oA) and torch.equal(dB, oB)
+
+
+def test_fp32_sizes_that_choose_128_tiles(fpo):
+    """Without an override: a logits pass and a grouped update of more tiles of 64 than the
+    SMs hold at once, odd everywhere, whose chunks of 40 tokens choose the tiles of 64."""
+    wl = Workload("tiles32", T=777, d=131, d_ff=1027, V=5003, layers=6, dtype="f32",
+                  targets="zipf", lr=1e-2)
+    inp = synth.make_all(wl)
+    runs = [gpu_step(fpo, wl, inp, t_chunk=0), gpu_step(fpo, wl, inp, t_chunk=40, grouped=False)]
+    check(runs[0], oracle_step(wl, inp), inp, wl.lr, F32_TOL)
+    assert torch.equal(runs[0]["g"], runs[1]["g"]) and torch.equal(runs[0]["lse"], runs[1]["lse"])
+    assert all(torch.equal(a, b) for a, b in zip(runs[0]["W"], runs[1]["W"]))
