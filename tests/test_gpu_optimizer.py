@@ -163,7 +163,7 @@ def test_adamw_step_clip_full_size(fpo):
 def test_optimizer_pass_edges(fpo, kind, clip, size):
     """fp32 layers of a multiple of 4 elements (16-byte passes; the odd ones above take 4-byte
     ones) and bf16 layers whose last column half, or 32-row block, is partly or wholly outside
-    the matrix (norm slots that only part of a warp, or none, adds to)."""
+    the matrix (their norm slots: test_clip_norms_of_ragged_edges)."""
     dtype, T, d, d_ff = size
     wl = Workload("opt-edges", T=T, d=d, d_ff=d_ff, V=8, layers=3, dtype=dtype, seed=5)
     g = synth.normal((T, d), std=1e-2, seed=5, tensor="h").to(wl.torch_dtype)
@@ -192,3 +192,56 @@ def test_optimizer_pass_edges(fpo, kind, clip, size):
         if kind != "sgd":
             assert rel_frob(f64(S1[l]), ref["s1"]) < tol
         assert rel_frob(f64(Wo[l]), ref["W"]) < max(tol, 4e-3 if dtype == "bf16" else 0)
+
+
+@pytest.mark.parametrize("slot", ["column", "row", "corner"])
+@pytest.mark.parametrize("larger", ["W", "x"])
+@pytest.mark.parametrize("kind,clip", [("sgd", "step"), ("sgd", "grad"), ("sgdm", "step"),
+                                       ("adamw", "step")])
+@pytest.mark.parametrize("layers", [3, 8])
+def test_clip_norms_of_ragged_edges(fpo, kind, clip, larger, slot, layers):
+    """The clip factor is a ratio of two norms whose squares the GEMM's epilogue leaves in
+    slots of 32 rows x 64 columns; in a homogeneous matrix a slot that is lost or added twice
+    changes both alike.  Here one slot at the ragged edge (32 rows x the last 8 columns, the
+    last 8 rows x 64 columns, the last 8 x 8) holds most of one of the norms and little of the
+    other: without it, or with it twice, the factor is off by a fifth or more.  The workspace
+    starts as NaN, so that an unwritten slot shows.  3 layers run on tiles of 128 columns, 8 on
+    256.  The factor is compared on the other elements: G and the steps are fp32 (sums of 33
+    terms), and W' resolves a step to some 1e-3 of itself, 1e-5 over 200,000 elements."""
+    T, d, d_ff = 33, 392, 520
+    wl = Workload("opt-norms", T=T, d=d, d_ff=d_ff, V=8, layers=layers, seed=9)
+    g = synth.normal((T, d), std=100.0, seed=9, tensor="h")
+    A = [synth.make_A(wl, l) for l in range(layers)]
+    W = [synth.make_W_master(wl, l) for l in range(layers)]
+    rows = {"column": slice(0, 32), "row": slice(384, 392), "corner": slice(384, 392)}[slot]
+    cols = {"column": slice(512, 520), "row": slice(0, 64), "corner": slice(512, 520)}[slot]
+    if larger == "x" and kind == "sgd":
+        g[:, rows] *= 16
+        for a in A:
+            a[:, cols] *= 16
+    g = g.to(wl.torch_dtype)
+    e = synth.to_numpy_exact
+    Gs = [oracle.pseudograd(e(g), e(a)) for a in A]
+    s1, s2 = _states(wl, Gs, kind, 3)
+    for m in (W if larger == "W" else s1 if kind != "sgd" else []):
+        m[rows, cols] *= 200
+    lr = {"sgd": 50.0, "sgdm": 50.0, "adamw": 2.0}[kind]  # every step is clipped
+    opt = fpo.optimizer_desc(KINDS[kind], lr=lr, clip=CLIPS[clip], step=3)
+    Wm = [w.cuda() for w in W]
+    S1 = [torch.from_numpy(x).cuda() for x in s1] if kind != "sgd" else None
+    S2 = [torch.from_numpy(x).cuda() for x in s2] if kind == "adamw" else None
+    ws = torch.full((fpo.layer_optimize_workspace(layers, d, d_ff),), 0xFF, dtype=torch.uint8,
+                    device="cuda")
+    fpo.layer_optimize_grouped([g.cuda()] * layers, [a.cuda() for a in A], opt, Wm, states1=S1,
+                               states2=S2, workspace=ws)
+    assert fpo.get_device_status(ws) == fpo.OK
+    rest = np.ones((d, d_ff), bool)
+    rest[rows] = False
+    rest[:, cols] = False
+    for l in range(layers):
+        ref = oracle.optimizer_step(W[l].numpy(), Gs[l], kind=KINDS[kind], lr=lr, t=3,
+                                    clip=CLIPS[clip], s1=s1[l], s2=s2[l])
+        assert ref["scale"] < 1.0
+        W0 = W[l].double().numpy()
+        d_ref, d_got = (x[rest] - W0[rest] for x in (ref["W"].astype(np.float64), f64(Wm[l])))
+        assert abs(np.sum(d_got * d_ref) / np.sum(d_ref * d_ref) - 1) < 1e-4, l
