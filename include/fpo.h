@@ -161,22 +161,22 @@ typedef struct fpo_error_signal_desc {
 /*
  * Stage boundaries of fpo_error_signal at which desc->stage_events[i] is
  * recorded: 0 start, 1 after the RMSNorm forward, 2 after the logits pass (of
- * the last token chunk for FPO_ES_STORED_LOGITS), 3 after the log-sum-exp
- * combine (and loss), 4 after the recompute pass (FPO_ES_RECOMPUTE), the
- * logits-to-E conversion (FPO_ES_STORED_LOGITS) or the anchor-window fixup
- * (FPO_ES_DIRECT; with the loss mean) of the last token chunk, 5
- * after the projection of the last token chunk, 6 after the final-norm VJP
+ * the last token chunk, but for FPO_ES_RECOMPUTE), 3 after the log-sum-exp
+ * combine (FPO_ES_STORED_LOGITS forms lse in the next kernel: 2 to 3 is empty),
+ * 4 after the recompute pass (FPO_ES_RECOMPUTE), the conversion of logits to
+ * lse and E (FPO_ES_STORED_LOGITS) or the anchor-window fixup (FPO_ES_DIRECT;
+ * with the loss mean) of the last token chunk, 5 after the projection of the
+ * last token chunk, 6 after the final-norm VJP, which also takes the loss mean
  * (under FPO_ES_DIRECT the projection applies the VJP: 5 to 6 is empty).
- * With one chunk, consecutive events bracket one kernel each (plus the loss
- * mean in [2]-[3]).
+ * With one chunk, consecutive events bracket one of these stages each.
  * With stage_events_per_chunk = 1 and n token chunks the events are 3 + 4 n:
  * 0 start, 1 after the RMSNorm forward, then for chunk c = 0 .. n-1:
- * 2 + 4c after its logits pass, 3 + 4c after its combine (and, last chunk and
- * not FPO_ES_DIRECT, the loss mean), 4 + 4c after its E / fixup stage (and,
- * last chunk and FPO_ES_DIRECT, the loss mean), 5 + 4c after its projection;
- * and 2 + 4n after the VJP.  (FPO_ES_RECOMPUTE runs one logits pass and one
- * combine over all tokens: they fill chunk 0's first two slots; the other
- * chunks record those two at the chunk's start.)
+ * 2 + 4c after its logits pass, 3 + 4c after its combine (at once for
+ * FPO_ES_STORED_LOGITS), 4 + 4c after its E / fixup stage (and, last chunk and
+ * FPO_ES_DIRECT, the loss mean), 5 + 4c after its projection; and 2 + 4n after
+ * the VJP (with the loss mean unless FPO_ES_DIRECT).  (FPO_ES_RECOMPUTE runs one
+ * logits pass and one combine over all tokens: they fill chunk 0's first two
+ * slots; the other chunks record those two at the chunk's start.)
  */
 #define FPO_STAGE_EVENTS 7
 

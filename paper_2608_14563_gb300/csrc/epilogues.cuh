@@ -565,15 +565,6 @@ struct RowPos {
     }
 };
 
-// The operands of a chunk are loaded as one batch when the chunk before is done, with
-// nothing that waits between its loads: loads issued one by one between the uses of the
-// batch before shared the warp's few scoreboards with it, and each use waited for the
-// newest load (the update of T 512, d 2048, d_ff 8264, 4 layers: 278 us, 230 of them with
-// the loads alone, 115 without; 195 us with batches, and 176 with 256 bytes of two rows per
-// access (kRows 16) instead of 128 bytes of four (kRows 32).  512 bytes of one row (kRows 8)
-// gave 162 but cost 2% of a T 200 step, as every lane reads the accumulator once per row
-// group.  Two batches in flight gave nothing more, nor did 16 warps, L2 prefetches of the
-// next tile or streaming cache hints).
 // Slots of per-warp partial sums per (256-row block, 256 columns): 8 blocks of 32 rows times
 // 4 column quarters.  A warp with two column groups keeps their sums apart, so that tiles of
 // 128 columns leave the same slots.
@@ -628,6 +619,16 @@ __device__ __forceinline__ void GroupSums<N, kCG>::store(float* slot, int lane) 
 // Pseudogradient update (Eq. w3update, App. A): for group (layer) g,
 //   W_master[g] -= lr * G ;  W_out[g] = bf16(W_master[g]) ;  G_out[g] = bf16(G)
 // Any of the three pointers may be null for a layer.
+//
+// The operands of a chunk (here, in the cosine, plain G and gate / up) are loaded as one
+// batch when the chunk before is done, with nothing that waits between its loads: loads
+// issued one by one between the uses of the batch before shared the warp's few scoreboards
+// with it, and each use waited for the newest load (the update of T 512, d 2048, d_ff 8264, 4
+// layers: 278 us, 230 of them with the loads alone, 115 without; 195 us with batches, and 176
+// with 256 bytes of two rows per access (kRows 16) instead of 128 bytes of four (kRows 32).
+// 512 bytes of one row (kRows 8) gave 162 but cost 2% of a T 200 step, as every lane reads the
+// accumulator once per row group.  Two batches in flight gave nothing more, nor did 16 warps,
+// L2 prefetches of the next tile or streaming cache hints).
 struct EpiUpdateBase {
     struct Params {
         float* W_master[kMaxGroups];
@@ -830,12 +831,12 @@ struct EpiStoreGroupF32 : EpiStoreGroupF32Base {
 // clip on the step (Sec. 3.1: SGD, SGD with momentum, AdamW on the fp32 masters; App. A:
 // ||dW|| <= clip_frac ||W||).  With G from the accumulator, each element's optimizer state
 // advances and its unclipped step d = opt_step(G, W, s1, s2) is stored (fp32, D[g], null
-// for momentum, whose step -lr s1 the state holds; the state sees the unclipped gradient), and ||W||^2, ||d||^2 of the warp's 32 rows x 128
-// columns are written as one pair per slot; a kernel then scales each layer's steps
-// by min(1, clip_frac ||W|| / ||d||) and applies them (W is not written here, so its norm
-// is the pre-step one).  Without a clip the stand-alone passes are used: taking the whole
-// step here made the update faster but the power-capped step slower (its epilogue then
-// held the tensor pipe back at full draw).
+// for momentum, whose step -lr s1 the state holds; the state sees the unclipped gradient),
+// and ||W||^2, ||d||^2 are written as one pair per slot of 32 rows x 64 columns; a kernel
+// then scales each layer's steps by min(1, clip_frac ||W|| / ||d||) and applies them (W is
+// not written here, so its norm is the pre-step one).  Without a clip the stand-alone passes
+// are used: taking the whole step here made the update faster but the power-capped step
+// slower (its epilogue then held the tensor pipe back at full draw).
 // The operands of the access 4 ahead are loaded as each one is done: its arithmetic hides the
 // wait that the batches of the other epilogues avoid (T 4096, d 4096, d_ff 11008, 8 layers,
 // AdamW, with 4 rows x 128 bytes per access: 2362 us; batches of a whole or half a chunk

@@ -459,7 +459,7 @@ size_t fpo_layer_grad_cosine_workspace(int32_t n_layers, int64_t d, int64_t d_ff
     if (n_layers < 1 || n_layers > FPO_MAX_GROUPED_LAYERS || d <= 0 || d_ff <= 0 ||
         d > INT_MAX || d_ff > INT_MAX)
         return 0;
-    // bf16: the per-(tile, warp) triples of the fused epilogue; fp32: the partials of the
+    // bf16: the triples per 32 rows x 64 columns of the fused epilogue; fp32: those of the
     // separate grouped cosine (the larger of the two, so one size serves both)
     const size_t fused = grad_cosine_partial_bytes(n_layers, static_cast<int>(d),
                                                    static_cast<int>(d_ff));
@@ -518,7 +518,7 @@ int32_t fpo_layer_grad_cosine_grouped(int32_t n_layers, int64_t T, int64_t d, in
 }
 
 // Bytes of the optimizer's norm partials: those of the stand-alone passes or of the
-// fused epilogue's (layer, 256 rows, column tile, 32 rows) slots, whichever is larger.
+// fused epilogue's slots of 32 rows x 64 columns, whichever is larger.
 static size_t optimize_partials_area(int32_t n_layers, int64_t d, int64_t d_ff) {
     const size_t a = optim_partials_bytes(n_layers);
     const size_t b = opt_step_partial_bytes(n_layers, static_cast<int>(d), static_cast<int>(d_ff));
@@ -603,9 +603,9 @@ int32_t fpo_layer_optimize_grouped(int32_t n_layers, int64_t T, int64_t d, int64
         opt_step_partial_bytes(1, static_cast<int>(d), static_cast<int>(d_ff)) / (2 * sizeof(float)));
     if (dtype == FPO_BF16 && T > 0 && opt->clip == FPO_CLIP_STEP) {
         // the step clip's first pass in the GEMM's epilogue: the state advanced, the
-        // unclipped steps (in the G buffer) and their norm partials; then a scale and an
-        // apply pass (measured: the AdamW + step-clip step 0.6% faster than with G stored
-        // and three passes; without a clip the stand-alone passes are faster overall)
+        // unclipped steps (in the G buffer; a momentum step is in the state) and their norm
+        // partials; then a scale and an apply pass (without a clip the stand-alone passes
+        // are faster overall)
         const bool momentum = op.kind == FPO_OPT_SGD_MOMENTUM;  // its step is -lr s1
         FPO_TRY(launch_opt_step_bf16(n_layers, static_cast<int>(T), static_cast<int>(d),
                                      static_cast<int>(d_ff), g, A, op, W_master, s1, s2,

@@ -427,9 +427,14 @@ bool use_pair() { return g_gemm_variant.load(std::memory_order_relaxed) >= 1; }
 
 // Whether the GEMMs over the vocabulary of a chunk of T tokens run on CTA pairs: not, by
 // default, when an odd number of 128-row blocks, at most 5, leaves half of a pair's 256 rows
-// empty.  The single-CTA kernel is 10-25% slower per row but wastes at most 127 of them.
-// Logits pass, d 4096, V 100352, pair against single: T 128 167 and 145 us, 333 251 and
-// 224, 600 347 and 333 (seven blocks, T 900, V 50304: 237 and 268).  Same sums either way.
+// empty.  The single-CTA kernel is up to 20% slower per row but wastes at most 127 of them.
+// Logits pass in us, on pairs and on single CTAs, at T 128, 333, 600 and 1100 (9 blocks):
+//   d 2048, V  50304    52  49    75  64    95  96   145 154
+//   d 2048, V 100352    91  80   132 118   181 175   283 301
+//   d 4096, V  50304    89  87   137 118   177 181   270 292
+//   d 4096, V 100352   163 142   245 223   342 334   544 602
+// (V 8192: within 5 us up to 5 blocks.  d 512: single CTAs are faster at every T up to 2048,
+// 96 against 108 us there with V 50304.)  Same sums either way.
 bool use_pair_rows(int T) {
     const int blocks = (T + kBM - 1) / kBM;
     return use_pair() &&
@@ -523,6 +528,10 @@ int proj_clusters() {
 // Ranges of 256 x 512 tiles (670 ns a k-block, and 5000 for the store, which the next unit
 // of their single accumulator waits for) leave half as many parts to add: 200 x 4096 x
 // 100352 350 -> 338 us, 200 x 5120 x 152064 600 -> 570, 600 x 4096 x 100352 715 -> 695.
+//
+// The constants are of one state of the clock; what the choice needs is their ratios.  Over d
+// 512, 2048, 4096 x V 8192, 50304, 100352 x 13 T from 64 to 2048, the projection with its
+// fixup took 0.09 to 1.02 of its time in whole 256-column tiles.
 struct ProjPlan {
     int split = 0;        // K ranges per tile; 0: whole 512-column tiles
     int width = kWideBN;  // columns of a tile: of g, or kTurnBN tokens
@@ -812,6 +821,8 @@ cudaError_t launch_proj_bf16(const void* E, const void* W_U, int Tc, int T_all, 
             if (e != cudaSuccess) return e;
             return launch_sk_fixup<kWideBN>(plan, sh, sk_scratch, g, st);
         }
+        // (no tiles of 128 columns as in the direct algorithm: bf16 runs here only when the
+        // stored-logits or recompute algorithm is asked for)
         const GemmShape sh = make_shape(Tc, d, V, kProjBN, 1, band_for(true), kPairBM);
         const cudaError_t e = run_gemm_pair<kProjBN, false, true, kPairStages, 1, EpiStoreF32>(
             maps, ep, sh, status, st, pp.split > 1 ? sk_scratch : nullptr, &plan, pp.split);

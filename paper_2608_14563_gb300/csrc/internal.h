@@ -162,7 +162,7 @@ cudaError_t launch_grad_bf16(int n, int T, int d, int d_ff, const void* const* g
 
 // Grouped pseudogradients with the diagnostic's cosine: G_out[l] (bf16 [d, d_ff]) =
 // g[l]^T A[l], and out[4 l ..] = <G_l, Y_l>, ||G_l||^2, ||Y_l||^2, cos_l of the stored
-// G_l against Y[l] (bf16), from per-(tile, warp) partial sums in `part`
+// G_l against Y[l] (bf16), from partial sums per 32 rows x 64 columns in `part`
 // (grad_cosine_partial_bytes) without a second pass over G.
 size_t grad_cosine_partial_bytes(int n, int d, int d_ff);
 cudaError_t launch_grad_cosine_bf16(int n, int T, int d, int d_ff, const void* const* g,
@@ -188,9 +188,9 @@ struct OptimParams {
 };
 size_t optim_partials_bytes(int n_layers);
 // The step clip's first optimizer pass fused into the pseudogradient GEMM (bf16): the
-// state advanced, the unclipped steps in D and (||W||^2, ||d||^2) per (layer, 256 rows,
-// column tile half, 32 rows) in part, for launch_opt_scale and launch_opt_step_apply.  D is
-// not written for momentum (the step is -lr s1).
+// state advanced, the unclipped steps in D and (||W||^2, ||d||^2) per 32 rows x 64 columns
+// of a layer in part (slot_of, epilogues.cuh), for launch_opt_scale and
+// launch_opt_step_apply.  D is not written for momentum (the step is -lr s1).
 cudaError_t launch_opt_step_bf16(int n, int T, int d, int d_ff, const void* const* g,
                                  const void* const* A, const OptimParams& op,
                                  float* const* W_master, float* const* s1, float* const* s2,

@@ -150,10 +150,10 @@ __device__ __forceinline__ void out_stage_row(uint32_t buf, int r, const uint32_
 }
 
 // Chunks of the 8-warp epilogues: kRows of the warp's 32 rows x kCols of its fp32 columns
-// (half of the tile's: 128 or 64), staged in the warp's 4 KB of output staging by the lanes that hold the rows and
-// read back with kLanes lanes to a row, 4 columns each, so that every global access of a
-// warp covers kCols consecutive columns of kAccRows rows.  16-byte pieces are swizzled by
-// row, so neither side has bank conflicts.
+// (half of the tile's: 128 or 64), staged in the warp's 4 KB of output staging by the lanes
+// that hold the rows and read back with kLanes lanes to a row, 4 columns each, so that every
+// global access of a warp covers kCols consecutive columns of kAccRows rows.  16-byte pieces
+// are swizzled by row, so neither side has bank conflicts.
 struct RowChunk {
     static constexpr int kRows = 16;
     static constexpr int kCols = 1024 / kRows;
